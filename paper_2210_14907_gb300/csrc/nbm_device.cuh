@@ -456,11 +456,13 @@ __device__ __forceinline__ void tanh_stencil_fwd(float t, float mt, float dt, fl
 // Tm = 0, tw = t, dm = 0.
 template <bool FAST>
 __device__ __forceinline__ void tanh_stencil_fwd0(float t, float dt, float h, float inv_h,
-                                                  float inv_h2, float& mo, float& dout) {
-  const float Td = act_tanh<FAST>(dt * h);
+                                                  float inv_h2, float& mo, float& dout,
+                                                  bool small_de = false) {
+  const bool sde = !FAST && small_de;
+  const float Td = sde ? tanh_small(dt * h) : act_tanh<FAST>(dt * h);
   const float sw = fmaf(-t, t, 1.0f);
   const float Td2 = Td * Td;
-  const float r2 = rcp<FAST>(fmaf(-t * t, Td2, 1.0f));
+  const float r2 = sde ? rcp_one_minus_small(t * t * Td2) : rcp<FAST>(fmaf(-t * t, Td2, 1.0f));
   mo = (-t * sw * Td2 * r2) * inv_h2;
   dout = (sw * Td * r2) * inv_h;
 }

@@ -198,7 +198,6 @@ cudaError_t launch_adam(int64_t n, float* params, float* m, float* v, const floa
                         cudaStream_t st);
 size_t tc_smem_bytes(int L);
 cudaError_t launch_selftest_wait(long long budget, int* out, cudaStream_t st);
-size_t fp32_smem_bytes(int H, int L);
 int tc_supported(int H, int L);
 
 }  // namespace nbm

@@ -393,20 +393,64 @@ __global__ void __launch_bounds__(512, 1) k_eval_tc(ProbDev P, const float* __re
   if (w == 0) tmem_dealloc(tmem, kEvalTmemCols);
 }
 
-// Plain FP32 evaluation: one thread per node, activations in shared memory
-// ([unit][thread]), weights read through the read-only cache.
-template <int H, int L>
-__global__ void __launch_bounds__(128) k_eval_fp32(ProbDev P, const float* __restrict__ params,
-                                                   int n, const float* __restrict__ pts,
-                                                   int64_t npts, float* __restrict__ u_out) {
-  extern __shared__ float act[];  // [2][H][128]
-  const int tid = threadIdx.x;
+// Plain FP32 evaluation (FFMA): each point with the network of its side only.
+//
+// A CTA takes a contiguous range of the points, 1024 at a time: it decides their
+// sides, lists the two sides' points in shared memory, and runs each list in
+// tiles of TP points through its network.  A layer of a tile is one
+// [H x H] x [H x TP] product, activations [unit][point] in shared memory (in
+// place), a thread computing TU units x TQ points on packed point pairs (8 x 8 at
+// H = 128).  The weights stream through a ring of three 16-column chunks
+// [unit][16 (+ 4 of padding)] (4-byte cp.async: the parameter vector has no
+// better alignment), two chunks ahead and across layers and tiles, so a tile
+// reads each weight from L2 once.  Lane bits are dealt so that neighbouring
+// lanes (x ^ 1, x ^ 2) share one of the two operands: a 16-byte shared load of a
+// warp then takes two wavefronts instead of four.
+// Bound: the FFMA pipe (H^2 FMA per point and hidden layer).  200,000 points,
+// 3 -> 128 x 3 -> 1: 10.4 ms with one thread per point and both networks (a
+// shared and a global load per FMA), 0.38 ms now (35 TFLOP/s, 43 % of the FFMA
+// peak; the lists' part-filled last tiles are 15 % of it).
+// TP = 128 from 128 points per SM on; 32 for fewer, where a tile's latency counts
+// and wide tiles would leave SMs idle.
+template <int H, int TP>
+struct EvalCfg {
+  static constexpr int TU = H * TP / 256 >= 64 ? 8 : 4;  // units per thread
+  static constexpr int TQ = H * TP / 256 / TU;           // points per thread: 8, 4 or 2
+  static constexpr int NUG = H / TU, NPG = TP / TQ;      // unit and point groups
+  static constexpr int kKC = 16, kLD = kKC + 4;          // weight chunk: columns, row stride
+  static constexpr int kChunk = 1024;                    // points sorted by side at a time
+  static constexpr int kRing = H * TP;                   // float offsets in shared memory
+  static constexpr int kXs = kRing + 3 * H * kLD;        // [3][TP] coordinates
+  static constexpr int kRed = kXs + 3 * TP;              // [NUG / 8][TP] output partials
+  static constexpr int kList = kRed + (NUG / 8) * TP;    // [kChunk] point offsets by side
+  static constexpr size_t bytes = (size_t)(kList + kChunk) * sizeof(float);
+};
+
+template <int H, int L, int TP>
+__global__ void __launch_bounds__(256, 2) k_eval_fp32(ProbDev P, const float* __restrict__ params,
+                                                      int n, const float* __restrict__ pts,
+                                                      int64_t npts, float* __restrict__ u_out) {
+  using C = EvalCfg<H, TP>;
+  constexpr int TU = C::TU, TQ = C::TQ, NCH = H / C::kKC, SQ = C::NPG * 4;
+  static_assert(C::NUG * C::NPG == 256 && C::NUG % 8 == 0 && C::NPG % 4 == 0, "thread grid");
+  extern __shared__ __align__(16) float sm[];
+  __shared__ int cnt[2];
+  float* act = sm;  // [H][TP]
+  float* ring = sm + C::kRing;
+  float* xs = sm + C::kXs;
+  float* red = sm + C::kRed;
+  int* list = reinterpret_cast<int*>(sm + C::kList);  // minus points from the front, plus from the back
+  const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
+  constexpr int WU = C::NUG / 8;  // warps along the units
+  const int ug = (w % WU) * 8 + (((lane >> 1) & 3) | ((lane >> 4) << 2));
+  const int pg = (w / WU) * 4 + (lane & 1) + ((lane >> 3) & 1) * 2;
+  // units ug + NUG i; points 4 pg + 0..3 (+ SQ for the second four), or 2 pg + 0..1
+  const int p0 = TQ == 2 ? 2 * pg : 4 * pg;
+
   const int64_t N1 = n + 1, total = pts ? npts : N1 * N1 * N1;
-  const int64_t id = (int64_t)blockIdx.x * 128 + tid;
+  const int64_t rb = total * blockIdx.x / gridDim.x, re = total * (blockIdx.x + 1) / gridDim.x;
   const float hg = 2.0f / (float)n;
-  float x = 0.f, y = 0.f, z = 0.f;
-  int s = 0;
-  if (id < total) {
+  auto coords = [&](int64_t id, float& x, float& y, float& z) {
     if (pts) {
       x = pts[3 * id];
       y = pts[3 * id + 1];
@@ -417,34 +461,189 @@ __global__ void __launch_bounds__(128) k_eval_fp32(ProbDev P, const float* __res
       y = -1.f + hg * (float)j;
       z = -1.f + hg * (float)k;
     }
-    s = node_phase(P, x, y, z);
-  }
-  float result = 0.f;
-  for (int net = 0; net < 2; ++net) {
-    const float* th = params + net * P.p_net;
-    float* a0 = act;
-    float* a1 = act + H * 128;
-    for (int j = 0; j < H; ++j)
-      a0[j * 128 + tid] = tanhf(fmaf(__ldg(th + 3 * j), x,
-                                     fmaf(__ldg(th + 3 * j + 1), y,
-                                          fmaf(__ldg(th + 3 * j + 2), z, __ldg(th + 3 * H + j)))));
-    const float* Wl = th + 4 * H;
-    for (int g = 1; g < L; ++g) {
-      for (int j = 0; j < H; ++j) {
-        float acc = __ldg(Wl + (int64_t)H * H + j);
-        for (int k = 0; k < H; ++k) acc = fmaf(__ldg(Wl + (int64_t)j * H + k), a0[k * 128 + tid], acc);
-        a1[j * 128 + tid] = tanhf(acc);
+  };
+
+  int wst = 0, rst = 0;
+  // columns 16 ch .. of a [H][H] weight matrix into the ring
+  auto issue = [&](const float* W, int ch) {
+    if (W) {
+      const uint32_t d = smem_u32(ring + wst * (H * C::kLD));
+#pragma unroll
+      for (int i = 0; i < H * C::kKC / 256; ++i) {
+        const int e = tid + 256 * i, u = e >> 4, k = e & 15;
+        cp_async4(d + 4u * (uint32_t)(u * C::kLD + k), W + (int64_t)u * H + ch * C::kKC + k);
       }
-      float* tmp = a0;
-      a0 = a1;
-      a1 = tmp;
-      Wl += (int64_t)H * H + H;
+      wst = wst == 2 ? 0 : wst + 1;
     }
-    float o = __ldg(Wl + H);
-    for (int k = 0; k < H; ++k) o = fmaf(__ldg(Wl + k), a0[k * 128 + tid], o);
-    if (net == s) result = o;
+    asm volatile("cp.async.commit_group;" ::: "memory");
+  };
+
+#pragma unroll 1
+  for (int64_t c0 = rb; c0 < re; c0 += C::kChunk) {
+    const int m = (int)(re - c0 < C::kChunk ? re - c0 : C::kChunk);
+    if (tid < 2) cnt[tid] = 0;
+    __syncthreads();
+    for (int i0 = 0; i0 < m; i0 += 256) {
+      const int i = i0 + tid;
+      int s = -1;
+      if (i < m) {
+        float x, y, z;
+        coords(c0 + i, x, y, z);
+        s = node_phase(P, x, y, z);
+      }
+      // the order within a list does not matter: a point's value does not depend
+      // on its place in a tile
+#pragma unroll
+      for (int q = 0; q < 2; ++q) {
+        const unsigned b = __ballot_sync(0xffffffffu, s == q);
+        int base = 0;
+        if (lane == 0 && b) base = atomicAdd(&cnt[q], __popc(b));
+        base = __shfl_sync(0xffffffffu, base, 0);
+        if (s == q) {
+          const int at = base + __popc(b & ((1u << lane) - 1u));
+          list[q ? C::kChunk - 1 - at : at] = i;
+        }
+      }
+    }
+    __syncthreads();
+    const int cn[2] = {cnt[0], cnt[1]};
+    const float* W0 = params + (cn[0] ? 0 : P.p_net) + 4 * H;
+    issue(W0, 0);
+    issue(W0, 1);
+#pragma unroll 1
+    for (int s = 0; s < 2; ++s) {
+      const float* th = params + s * P.p_net;
+      const float* wo = th + 4 * H + (int64_t)(L - 1) * (H * H + H);
+#pragma unroll 1
+      for (int t0 = 0; t0 < cn[s]; t0 += TP) {
+        // the first weights of the tile after this one
+        const float* nxt = t0 + TP < cn[s] ? th + 4 * H
+                           : s == 0 && cn[1] ? params + P.p_net + 4 * H : nullptr;
+        auto entry = [&](int q) { return list[s ? C::kChunk - 1 - (t0 + q) : t0 + q]; };
+        if (tid < TP) {
+          float x = 0.f, y = 0.f, z = 0.f;
+          if (t0 + tid < cn[s]) coords(c0 + entry(tid), x, y, z);
+          xs[tid] = x;
+          xs[TP + tid] = y;
+          xs[2 * TP + tid] = z;
+        }
+        __syncthreads();
+        auto store = [&](int u, const float (&v)[TQ]) {
+          if constexpr (TQ == 2) {
+            *reinterpret_cast<float2*>(act + u * TP + p0) = make_float2(v[0], v[1]);
+          } else {
+#pragma unroll
+            for (int h4 = 0; h4 < TQ / 4; ++h4)
+              *reinterpret_cast<float4*>(act + u * TP + p0 + SQ * h4) =
+                  make_float4(v[4 * h4], v[4 * h4 + 1], v[4 * h4 + 2], v[4 * h4 + 3]);
+          }
+        };
+        auto point = [&](int q) { return p0 + (q & 3) + SQ * (q >> 2); };
+        // layer 1 (K = 3)
+#pragma unroll
+        for (int i = 0; i < TU; ++i) {
+          const int u = ug + C::NUG * i;
+          const float w0 = th[3 * u], w1 = th[3 * u + 1], w2 = th[3 * u + 2], bb = th[3 * H + u];
+          float v[TQ];
+#pragma unroll
+          for (int q = 0; q < TQ; ++q)
+            v[q] = tanhf(fmaf(w0, xs[point(q)],
+                              fmaf(w1, xs[TP + point(q)], fmaf(w2, xs[2 * TP + point(q)], bb))));
+          store(u, v);
+        }
+        float part[TQ];
+#pragma unroll
+        for (int q = 0; q < TQ; ++q) part[q] = 0.f;
+#pragma unroll 1
+        for (int g = 1; g < L; ++g) {
+          const float* W = th + 4 * H + (int64_t)(g - 1) * (H * H + H);
+          const float* nW = g < L - 1 ? W + H * H + H : nxt;
+          F2 acc[TU][TQ / 2];
+#pragma unroll
+          for (int i = 0; i < TU; ++i) {
+            const F2 bb = f2s(W[H * H + ug + C::NUG * i]);
+#pragma unroll
+            for (int q = 0; q < TQ / 2; ++q) acc[i][q] = bb;
+          }
+#pragma unroll 1
+          for (int ch = 0; ch < NCH; ++ch) {
+            asm volatile("cp.async.wait_group 1;" ::: "memory");
+            __syncthreads();  // the chunk has landed; every warp is done with the one before
+            if (ch + 2 < NCH) issue(W, ch + 2);
+            else issue(nW, ch + 2 - NCH);
+            const float* wr = ring + rst * (H * C::kLD) + ug * C::kLD;
+            const float* ar = act + ch * C::kKC * TP + p0;
+            rst = rst == 2 ? 0 : rst + 1;
+#pragma unroll 2
+            for (int k4 = 0; k4 < C::kKC; k4 += 4) {
+              float4 wv[TU];
+#pragma unroll
+              for (int i = 0; i < TU; ++i)
+                wv[i] = *reinterpret_cast<const float4*>(wr + C::NUG * C::kLD * i + k4);
+#pragma unroll
+              for (int k = 0; k < 4; ++k) {
+                F2 av[TQ / 2];
+                if constexpr (TQ == 2) {
+                  const float2 a2 = *reinterpret_cast<const float2*>(ar + (k4 + k) * TP);
+                  av[0] = f2(a2.x, a2.y);
+                } else {
+#pragma unroll
+                  for (int h4 = 0; h4 < TQ / 4; ++h4) {
+                    const float4 a4 = *reinterpret_cast<const float4*>(ar + (k4 + k) * TP + SQ * h4);
+                    av[2 * h4] = f2(a4.x, a4.y);
+                    av[2 * h4 + 1] = f2(a4.z, a4.w);
+                  }
+                }
+#pragma unroll
+                for (int i = 0; i < TU; ++i) {
+                  const F2 ww = f2s(k == 0 ? wv[i].x : k == 1 ? wv[i].y : k == 2 ? wv[i].z : wv[i].w);
+#pragma unroll
+                  for (int q = 0; q < TQ / 2; ++q) acc[i][q] = fma2(ww, av[q], acc[i][q]);
+                }
+              }
+            }
+          }
+          if (g < L - 1) __syncthreads();  // every read of act is done: overwrite it
+#pragma unroll
+          for (int i = 0; i < TU; ++i) {
+            const int u = ug + C::NUG * i;
+            float v[TQ];
+#pragma unroll
+            for (int q = 0; q < TQ / 2; ++q) {
+              f2get(acc[i][q], v[2 * q], v[2 * q + 1]);
+              v[2 * q] = tanhf(v[2 * q]);
+              v[2 * q + 1] = tanhf(v[2 * q + 1]);
+            }
+            if (g < L - 1) {
+              store(u, v);
+            } else {
+              const float wu = wo[u];
+#pragma unroll
+              for (int q = 0; q < TQ; ++q) part[q] = fmaf(wu, v[q], part[q]);
+            }
+          }
+        }
+        // output layer: over the warp's 8 unit groups, then over the warps
+#pragma unroll
+        for (int q = 0; q < TQ; ++q) {
+          part[q] += __shfl_xor_sync(0xffffffffu, part[q], 2);
+          part[q] += __shfl_xor_sync(0xffffffffu, part[q], 4);
+          part[q] += __shfl_xor_sync(0xffffffffu, part[q], 16);
+          if ((lane & 22) == 0) red[(w % WU) * TP + point(q)] = part[q];
+        }
+        __syncthreads();
+        if (tid < TP && t0 + tid < cn[s]) {
+          float o = wo[H];
+#pragma unroll
+          for (int q = 0; q < WU; ++q) o += red[q * TP + tid];
+          u_out[c0 + entry(tid)] = o;
+        }
+        // (xs, act and red are next written after barriers that follow these reads)
+      }
+    }
+    __syncthreads();  // the list is done with
   }
-  if (id < total) u_out[id] = result;
+  asm volatile("cp.async.wait_group 0;" ::: "memory");
 }
 
 // Narrow networks (width <= 32, up to five layers; tanh or the sine layers of
@@ -529,16 +728,26 @@ cudaError_t launch_eval_tc_t(const ProbDev& P, const float* params, const unsign
   return cudaGetLastError();
 }
 
+template <int H, int L, int TP>
+cudaError_t launch_eval_fp32_tp(const ProbDev& P, const float* params, int n, const float* pts,
+                                int64_t npts, float* u, int64_t total, int sms, cudaStream_t st) {
+  constexpr size_t smem = EvalCfg<H, TP>::bytes;
+  cudaError_t e = cudaFuncSetAttribute(k_eval_fp32<H, L, TP>,
+                                       cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  if (e != cudaSuccess) return e;
+  const int64_t tiles = (total + TP - 1) / TP;
+  const int grid = (int)(tiles < 2 * sms ? tiles : 2 * sms);  // two CTAs per SM
+  k_eval_fp32<H, L, TP><<<grid, 256, smem, st>>>(P, params, n, pts, npts, u);
+  return cudaGetLastError();
+}
+
 template <int H, int L>
 cudaError_t launch_eval_fp32_t(const ProbDev& P, const float* params, int n, const float* pts,
-                               int64_t npts, float* u, cudaStream_t st) {
-  const size_t smem = 2 * (size_t)H * 128 * sizeof(float);
-  cudaError_t e = cudaFuncSetAttribute(k_eval_fp32<H, L>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                       (int)smem);
-  if (e != cudaSuccess) return e;
+                               int64_t npts, float* u, int sms, cudaStream_t st) {
   const int64_t total = pts ? npts : (int64_t)(n + 1) * (n + 1) * (n + 1);
-  k_eval_fp32<H, L><<<(int)((total + 127) / 128), 128, smem, st>>>(P, params, n, pts, npts, u);
-  return cudaGetLastError();
+  return total > 2 * (int64_t)sms * 64
+             ? launch_eval_fp32_tp<H, L, 128>(P, params, n, pts, npts, u, total, sms, st)
+             : launch_eval_fp32_tp<H, L, 32>(P, params, n, pts, npts, u, total, sms, st);
 }
 
 }  // namespace
@@ -577,7 +786,8 @@ static int eval_common(nbm_problem* p, const float* params, int n, const float* 
   cudaError_t e = cudaSuccess;
   if (precision == NBM_PREC_FP32) {
 #define NBM_EVAL32(HH, LL) \
-  else if (d.width == HH && d.n_hidden == LL) e = launch_eval_fp32_t<HH, LL>(P, params, n, pts, npts, u_out, st);
+  else if (d.width == HH && d.n_hidden == LL) \
+    e = launch_eval_fp32_t<HH, LL>(P, params, n, pts, npts, u_out, problem_num_sms(p), st);
     if (d.width <= 32) {
       e = launch_eval_small(P, params, n, pts, npts, u_out, st);
     }

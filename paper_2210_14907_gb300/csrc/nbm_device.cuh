@@ -475,14 +475,27 @@ __device__ __forceinline__ void tanh_stencil_fwd0(float t, float dt, float h, fl
 //                                     - 2 sin z sin^2(d/2),
 //   [sin(w+d) - sin(w-d)]/2         = cos w sin d,
 // cos w = cos z (1 - 2 sin^2(mu/2)) - sin z sin mu: no O(1) values are
-// subtracted.  sz, cz = sin z, cos z of the centre column.
+// subtracted.  sz, cz = sin z, cos z of the centre column.  `small` (the
+// half-increments of every lane of the warp are at most 2^-4): their sine and
+// cosine by Taylor series, sin x = x (1 - x^2/6 + x^4/120) + R, |R| <= |x|^7/5040,
+// cos x = 1 - x^2/2 + x^4/24 + R, |R| <= x^6/720, relative errors below 1e-10.
 // ---------------------------------------------------------------------------
+constexpr float kSmallHalf = 0.0625f;
+__device__ __forceinline__ void sincos_half(float x, bool small, float& s, float& c) {
+  if (small) {
+    const float x2 = x * x;
+    s = x * fmaf(x2, fmaf(x2, 1.0f / 120.0f, -1.0f / 6.0f), 1.0f);
+    c = fmaf(x2, fmaf(x2, 1.0f / 24.0f, -0.5f), 1.0f);
+  } else {
+    sincosf(x, &s, &c);
+  }
+}
 __device__ __forceinline__ void sin_stencil_fwd(float sz, float cz, float mt, float dt, float h,
                                                 float h2, float inv_h, float inv_h2, float& mo,
-                                                float& dout) {
+                                                float& dout, bool small) {
   float sh, ch, shd, chd;
-  sincosf(0.5f * mt * h2, &sh, &ch);
-  sincosf(0.5f * dt * h, &shd, &chd);
+  sincos_half(0.5f * mt * h2, small, sh, ch);
+  sincos_half(0.5f * dt * h, small, shd, chd);
   const float sm = 2.f * sh * ch, sh2 = sh * sh;
   const float sd = 2.f * shd * chd, shd2 = shd * shd, cd = fmaf(-2.f, shd2, 1.f);
   const float dsw = fmaf(cz, sm, -2.f * sz * sh2);  // sin w - sin z
@@ -501,10 +514,10 @@ __device__ __forceinline__ void sin_stencil_fwd(float sz, float cz, float mt, fl
 __device__ __forceinline__ float sin_stencil_bwd(float sz, float cz, float mt, float dt,
                                                  float Gm_s, float Gd_s, float h, float h2,
                                                  float inv_h, float inv_h2, float& gmu_s,
-                                                 float& gdel_s) {
+                                                 float& gdel_s, bool small) {
   float sh, ch, shd, chd;
-  sincosf(0.5f * mt * h2, &sh, &ch);
-  sincosf(0.5f * dt * h, &shd, &chd);
+  sincos_half(0.5f * mt * h2, small, sh, ch);
+  sincos_half(0.5f * dt * h, small, shd, chd);
   const float sm = 2.f * sh * ch, sh2 = sh * sh;
   const float sd = 2.f * shd * chd, shd2 = shd * shd, cd = fmaf(-2.f, shd2, 1.f);
   const float cmu = fmaf(-2.f, sh2, 1.f);

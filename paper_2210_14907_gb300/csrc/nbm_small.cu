@@ -2,25 +2,33 @@
 // to five tanh or sine layers): the sine-activated 5 x 10 networks of the
 // convergence study (arXiv 2210.14907, Sec. 4.1).
 //
-// Same organisation as the wide FP32 kernel: 8-point tiles, one warp per
-// point, every point carrying 8 difference-form stencil columns (centre
-// value, symmetric and antisymmetric increments of the three axes, value at
-// the interface point of a cut cell); lane u < H owns unit u.  Each layer
-// keeps its pre-activation columns (the sine adjoint needs z, mu, del) and its
-// output columns (the next layer's input and the weight-gradient operand) in
-// shared memory.  The weight gradient of a hidden layer is accumulated per
-// tile into this CTA's partial slice in a fixed order (deterministic); the
-// small parameters are accumulated per lane and written once per network.
+// Every point carries 8 difference-form stencil columns (centre value,
+// symmetric and antisymmetric increments of the three axes, value at the
+// interface point of a cut cell).  A warp takes as many points as its lanes
+// hold (32 / H, at most 4; three at H = 10), one lane per point and unit, and
+// runs them through forward, rows and backward by itself: each layer's
+// pre-activation columns (the sine adjoint needs z, mu, del) and output
+// columns are in the warp's own shared memory, and the weight gradient of a
+// lane's unit stays in its registers over all of the warp's tiles.  So no
+// barrier wider than the warp occurs in a tile, and the warps of an SM fill
+// each other's latencies.  With one point per warp (10 of 32 lanes busy),
+// block barriers in every layer and the weight gradient summed in global
+// memory tile by tile, a step of 16,384 points through 5 x 10 sine networks took
+// 229 us in this kernel; the bound now is the warps' dependency chains.
+// At the end of a network the lanes' sums are added over the warps in a fixed
+// order (deterministic).
+#include <climits>
+
 #include "nbm_device.cuh"
+#include "nbm_f32x2.cuh"
 #include "nbm_host.h"
 
 namespace nbm {
 
 namespace {
 
-constexpr int kSPT = 8;   // points per tile (one per warp)
-constexpr int kHM = 32;   // unit slots per point (lanes)
-constexpr int kLM = 5;    // maximum number of activation layers
+constexpr int kLM = 5;     // maximum number of activation layers
+constexpr int kMaxPt = 4;  // points per warp (8 lanes each for the rows)
 
 template <int ACT>
 __device__ __forceinline__ float act_f(float z) {
@@ -28,23 +36,41 @@ __device__ __forceinline__ float act_f(float z) {
   else return act_tanh<false>(z);
 }
 
+// whether the stencil increments of every lane allow their series
+template <int ACT>
+__device__ __forceinline__ void small_increments(const float zc[8], float h, float h2, bool& sm_mu,
+                                                 bool& sm_de) {
+  const float mm = fmaxf(fabsf(zc[1]), fmaxf(fabsf(zc[2]), fabsf(zc[3]))) * h2;
+  const float md = fmaxf(fabsf(zc[4]), fmaxf(fabsf(zc[5]), fabsf(zc[6]))) * h;
+  if constexpr (ACT == NBM_ACT_SIN) {
+    sm_mu = sm_de = __all_sync(0xffffffffu, 0.5f * fmaxf(mm, md) <= kSmallHalf);
+  } else {
+    sm_mu = __all_sync(0xffffffffu, mm <= kSmallMuAccurate);
+    sm_de = __all_sync(0xffffffffu, md <= kSmallDelAccurate);
+  }
+}
+
 // outputs of one unit's activation layer from its pre-activation columns
 // zc[8] (scaled convention); o[8] receives the output columns
 template <int ACT>
 __device__ __forceinline__ void layer_fwd(const float zc[8], bool jump, float h, float h2,
                                           float ih, float ih2, float o[8]) {
+  bool sm_mu, sm_de;
+  small_increments<ACT>(zc, h, h2, sm_mu, sm_de);
   if constexpr (ACT == NBM_ACT_SIN) {
     float sz, cz;
     sincosf(zc[0], &sz, &cz);
     o[0] = sz;
 #pragma unroll
-    for (int i = 0; i < 3; ++i) sin_stencil_fwd(sz, cz, zc[1 + i], zc[4 + i], h, h2, ih, ih2, o[1 + i], o[4 + i]);
+    for (int i = 0; i < 3; ++i)
+      sin_stencil_fwd(sz, cz, zc[1 + i], zc[4 + i], h, h2, ih, ih2, o[1 + i], o[4 + i], sm_mu);
   } else {
     const float t = act_tanh<false>(zc[0]);
     o[0] = t;
 #pragma unroll
     for (int i = 0; i < 3; ++i)
-      tanh_stencil_fwd<false>(t, zc[1 + i], zc[4 + i], h, h2, ih, ih2, o[1 + i], o[4 + i]);
+      tanh_stencil_fwd<false>(t, zc[1 + i], zc[4 + i], h, h2, ih, ih2, o[1 + i], o[4 + i], sm_mu,
+                              sm_de);
   }
   o[7] = jump ? act_f<ACT>(zc[7]) : 0.f;
 }
@@ -54,17 +80,20 @@ __device__ __forceinline__ void layer_fwd(const float zc[8], bool jump, float h,
 // pre-activation columns
 template <int ACT>
 __device__ __forceinline__ void layer_bwd(const float zc[8], const float oc[8], const float G[8],
-                                          float h, float h2, float ih, float ih2, float gz[8]) {
+                                          bool jump, float h, float h2, float ih, float ih2,
+                                          float gz[8]) {
   if constexpr (ACT == NBM_ACT_SIN) {
+    bool small, unused;
+    small_increments<ACT>(zc, h, h2, small, unused);
     float sz, cz;
     sincosf(zc[0], &sz, &cz);
     float gzc = cz * G[0];
 #pragma unroll
     for (int i = 0; i < 3; ++i)
       gzc += sin_stencil_bwd(sz, cz, zc[1 + i], zc[4 + i], G[1 + i], G[4 + i], h, h2, ih, ih2,
-                             gz[1 + i], gz[4 + i]);
+                             gz[1 + i], gz[4 + i], small);
     gz[0] = gzc;
-    gz[7] = cosf(zc[7]) * G[7];
+    gz[7] = jump ? cosf(zc[7]) * G[7] : 0.f;
   } else {
     const float t = oc[0], s0 = fmaf(-t, t, 1.f);
     float gzc = s0 * G[0];
@@ -77,309 +106,363 @@ __device__ __forceinline__ void layer_bwd(const float zc[8], const float oc[8], 
   }
 }
 
-__device__ __forceinline__ void ld8(const float* p, float v[8]) {
-  const float4 a = *reinterpret_cast<const float4*>(p), b = *reinterpret_cast<const float4*>(p + 4);
+// 8 columns of lane `ln`: the two 16-byte halves swapped for every other group of
+// 4 lanes, so that 8 neighbouring lanes' same halves lie in distinct banks
+__device__ __forceinline__ int half_off(int ln, int hf) { return ln * 8 + ((hf ^ ((ln >> 2) & 1)) << 2); }
+__device__ __forceinline__ void ld8(const float* p, int ln, float v[8]) {
+  const float4 a = *reinterpret_cast<const float4*>(p + half_off(ln, 0));
+  const float4 b = *reinterpret_cast<const float4*>(p + half_off(ln, 1));
   v[0] = a.x; v[1] = a.y; v[2] = a.z; v[3] = a.w;
   v[4] = b.x; v[5] = b.y; v[6] = b.z; v[7] = b.w;
 }
-__device__ __forceinline__ void st8(float* p, const float v[8]) {
-  reinterpret_cast<float4*>(p)[0] = make_float4(v[0], v[1], v[2], v[3]);
-  reinterpret_cast<float4*>(p)[1] = make_float4(v[4], v[5], v[6], v[7]);
+__device__ __forceinline__ void st8(float* p, int ln, const float v[8]) {
+  *reinterpret_cast<float4*>(p + half_off(ln, 0)) = make_float4(v[0], v[1], v[2], v[3]);
+  *reinterpret_cast<float4*>(p + half_off(ln, 1)) = make_float4(v[4], v[5], v[6], v[7]);
+}
+
+struct SmallRec {  // one point of a warp's tile
+  float x, y, z;
+  float gx, gy, gz;  // cut cell: interface point
+  int pt;            // -1: padding
+  int cutj;          // -1: uncut, else 2 cut_id + has_jump
+};
+static_assert(sizeof(SmallRec) == 32, "eight words");
+
+// Threads of a CTA: at H <= 16 a lane holds at most 4 x 16 weight-gradient sums,
+// and 16 warps fit the register file; at H <= 32 twice as many, and 8 do.
+constexpr int small_threads(int HM) { return HM <= 16 ? 512 : 256; }
+// floats of a warp's shared memory: columns, seeds, two sets of records
+constexpr int small_warp_floats(int L) { return 2 * L * 256 + kMaxPt * 8 + 2 * kMaxPt * 8; }
+size_t small_smem_bytes(int H, int L, int HM) {
+  return ((size_t)(small_threads(HM) / 32) * small_warp_floats(L) + 2 * (size_t)(L - 1) * H * H) *
+         sizeof(float);
 }
 
 }  // namespace
 
-size_t small_smem_bytes(int L) { return (size_t)2 * L * kSPT * kHM * 8 * sizeof(float); }
-
-template <int ACT>
-__global__ void __launch_bounds__(256, 1) k_step_small(ProbDev P, StepArgs a) {
+template <int ACT, int HM>
+__global__ void __launch_bounds__(small_threads(HM), 1) k_step_small(ProbDev P, StepArgs a) {
   pdl_enter();
+  constexpr int NT = small_threads(HM), NW = NT / 32;
   extern __shared__ __align__(16) float sbuf[];
-  __shared__ double loss_red[8];
+  __shared__ double loss_red[NW];
+  __shared__ float gbo_red[NW];
   const int H = P.H, L = P.L;
-  float* Zb = sbuf;                                   // [L][kSPT][kHM][8] pre-activations
-  float* Ab = sbuf + (size_t)L * kSPT * kHM * 8;      // [L][kSPT][kHM][8] outputs
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, tid = threadIdx.x;
-  const bool own = lane < H;  // lane u owns unit u
-  auto Z = [&](int l, int pw, int u) -> float* { return Zb + (((size_t)l * kSPT + pw) * kHM + u) * 8; };
-  auto A = [&](int l, int pw, int u) -> float* { return Ab + (((size_t)l * kSPT + pw) * kHM + u) * 8; };
+  const int ppw = 32 / H < kMaxPt ? 32 / H : kMaxPt;  // points per warp
+  const bool own = lane < ppw * H;                    // lane pq H + u: unit u of point pq
+  const int pq = own ? lane / H : 0, u = own ? lane - pq * H : 0, pbase = pq * H;
+  float* wsm = sbuf + w * small_warp_floats(L);
+  float* Zb = wsm;                    // [L][32][8] pre-activations, then their gradients
+  float* Ab = wsm + L * 256;          // [L][32][8] outputs
+  float* seeds_s = wsm + 2 * L * 256;  // [4][8]
+  SmallRec* recs = reinterpret_cast<SmallRec*>(seeds_s + kMaxPt * 8);  // [2][4]
+  float* Wf = sbuf + NW * small_warp_floats(L);  // [L-1][k][u] hidden weights, transposed
+  float* Wb = Wf + (L - 1) * H * H;              // [L-1][u][k]
 
   const int nm = a.counters[0], np = a.counters[1], nc = a.counters[2];
-  int64_t T0, T;
-  if (a.mode == MODE_CUT_FWD) {
-    T0 = (nc + kSPT - 1) / kSPT;
-    T = 2 * T0;
-  } else {
-    T0 = (nm + kSPT - 1) / kSPT;
-    T = T0 + (np + kSPT - 1) / kSPT;
-  }
+  const bool cutfwd = a.mode == MODE_CUT_FWD, train = a.mode == MODE_TRAIN;
+  const int64_t T0 = ((cutfwd ? nc : nm) + ppw - 1) / ppw;
+  const int64_t T = cutfwd ? 2 * T0 : T0 + (np + ppw - 1) / ppw;
   const int64_t tb = (int64_t)blockIdx.x * T / gridDim.x;
   const int64_t te = (int64_t)(blockIdx.x + 1) * T / gridDim.x;
   const float hf = P.hf, h2f = P.h2f, ihf = P.inv_hf, ih2f = P.inv_h2f;
-  const bool train = a.mode == MODE_TRAIN;
 
-  // small-parameter gradient accumulators of the current net (per lane)
+  // gradient sums of this lane's unit (its point slot's share of the current net)
   float gW1[3] = {0.f, 0.f, 0.f}, gb1 = 0.f, gwo = 0.f, gbo = 0.f;
-  float gbh[kLM - 1];
+  float gbh[kLM - 1], gW[kLM - 1][HM];
 #pragma unroll
-  for (int i = 0; i < kLM - 1; ++i) gbh[i] = 0.f;
+  for (int g = 0; g < kLM - 1; ++g) {
+    gbh[g] = 0.f;
+#pragma unroll
+    for (int k = 0; k < HM; ++k) gW[g][k] = 0.f;
+  }
   double loss_acc = 0.0;
-  int cur_net = -1;
-  bool first_tile = true;
   int wrote0 = 0, wrote1 = 0;
 
+  // this CTA's partial of net `net`: the lanes' sums staged in each warp's column
+  // memory, added over warps and point slots in a fixed order
   auto flush = [&](int net) {
+    float* gp = a.gpart + ((int64_t)blockIdx.x * 2 + net) * P.gstride;
+    const int wf = small_warp_floats(L), hh = H * H;
+    const int64_t oo = 4 * H + (int64_t)(L - 1) * (hh + H);
+#pragma unroll
+    for (int g = 0; g < kLM - 1; ++g) {
+      if (g >= L - 1) break;
+      __syncthreads();
+      if (own) {
+        float* st = wsm + pq * (hh + H);
+#pragma unroll
+        for (int k = 0; k < HM; ++k)
+          if (k < H) st[u * H + k] = gW[g][k];
+        st[hh + u] = gbh[g];
+      }
+      __syncthreads();
+      for (int i = tid; i < hh + H; i += NT) {
+        float s = 0.f;
+        for (int ww = 0; ww < NW; ++ww)
+          for (int q = 0; q < ppw; ++q) s += sbuf[ww * wf + q * (hh + H) + i];
+        gp[4 * H + (int64_t)g * (hh + H) + i] = s;  // weights, then biases
+      }
+    }
     __syncthreads();
-    float* stage = Ab;  // [8 warps][nsmall]; activations are dead here
-    const int nsmall = 4 * H + (L - 1) * H + H + 1;
     if (own) {
-      float* st = stage + (size_t)w * nsmall;
-      const int u = lane;
+      float* st = wsm + pq * 5 * H;
       st[3 * u] = gW1[0];
       st[3 * u + 1] = gW1[1];
       st[3 * u + 2] = gW1[2];
       st[3 * H + u] = gb1;
+      st[4 * H + u] = gwo;
+    }
+    float go = gbo;
 #pragma unroll
-      for (int g = 0; g < kLM - 1; ++g)
-        if (g < L - 1) st[4 * H + g * H + u] = gbh[g];
-      st[4 * H + (L - 1) * H + u] = gwo;
-    }
-    if (lane == 0) stage[(size_t)w * nsmall + nsmall - 1] = gbo;
+    for (int o = 16; o > 0; o >>= 1) go += __shfl_xor_sync(0xffffffffu, go, o);
+    if (lane == 0) gbo_red[w] = go;
     __syncthreads();
-    float* gp = a.gpart + ((int64_t)blockIdx.x * 2 + net) * P.gstride;
-    for (int idx = tid; idx < nsmall; idx += blockDim.x) {
+    for (int i = tid; i < 5 * H; i += NT) {
       float s = 0.f;
-      for (int ww = 0; ww < 8; ++ww) s += stage[(size_t)ww * nsmall + idx];
-      int64_t dst;
-      if (idx < 4 * H) {
-        dst = idx;  // W1, b1
-      } else if (idx < 4 * H + (L - 1) * H) {
-        const int g = (idx - 4 * H) / H, u = (idx - 4 * H) % H;  // bias of hidden layer g+1
-        dst = 4 * H + (int64_t)g * (H * H + H) + (int64_t)H * H + u;
-      } else {
-        dst = 4 * H + (int64_t)(L - 1) * (H * H + H) + (idx - 4 * H - (L - 1) * H);
-      }
-      gp[dst] = s;
+      for (int ww = 0; ww < NW; ++ww)
+        for (int q = 0; q < ppw; ++q) s += sbuf[ww * wf + q * 5 * H + i];
+      gp[i < 4 * H ? i : oo + i - 4 * H] = s;
     }
-    if (net) wrote1 = 1; else wrote0 = 1;
+    if (tid == 0) {
+      float s = 0.f;
+      for (int ww = 0; ww < NW; ++ww) s += gbo_red[ww];
+      gp[oo + H] = s;
+    }
     gW1[0] = gW1[1] = gW1[2] = gb1 = gwo = gbo = 0.f;
 #pragma unroll
-    for (int i = 0; i < kLM - 1; ++i) gbh[i] = 0.f;
+    for (int g = 0; g < kLM - 1; ++g) {
+      gbh[g] = 0.f;
+#pragma unroll
+      for (int k = 0; k < HM; ++k) gW[g][k] = 0.f;
+    }
+    if (net) wrote1 = 1; else wrote0 = 1;
     __syncthreads();
   };
 
-  for (int64_t tau = tb; tau < te; ++tau) {
-    const int net = tau < T0 ? 0 : 1;
-    const int64_t local = tau - (net ? T0 : 0);
-    if (train && net != cur_net) {
-      if (cur_net >= 0) flush(cur_net);
-      cur_net = net;
-      first_tile = true;
-    }
-    // ---- this warp's point (list entry >= 0: point index; < 0: cut id)
-    const int64_t slot = local * kSPT + w;
-    bool valid;
-    int cut_id = -1, pt = 0;
-    if (a.mode == MODE_CUT_FWD) {
-      valid = slot < nc;
-      if (valid) {
-        cut_id = (int)slot;
-        pt = a.cut[cut_id].point;
-      }
-    } else {
-      valid = slot < (net ? np : nm);
-      if (valid) {
-        const int e = a.list[net][slot];
-        if (e < 0) {
-          cut_id = -e - 1;
-          pt = a.cut[cut_id].point;
-        } else {
-          pt = e;
-        }
-      }
-    }
-    float px = 0.f, py = 0.f, pz = 0.f, gx = 0.f, gy = 0.f, gz = 0.f;
-    bool jump = false;
-    if (valid) {
-      px = a.x[pt];
-      py = a.y[pt];
-      pz = a.z[pt];
-      if (cut_id >= 0) {
-        const CutRec& cr = a.cut[cut_id];
-        jump = cr.has_jump;
-        gx = (float)cr.xg[0];
-        gy = (float)cr.xg[1];
-        gz = (float)cr.xg[2];
-      }
-    }
+#pragma unroll 1
+  for (int net = 0; net < 2; ++net) {
+    const int64_t s0 = net == 0 ? tb : (tb > T0 ? tb : T0);
+    const int64_t s1 = net == 0 ? (te < T0 ? te : T0) : te;
+    if (s0 >= s1) continue;  // the same in every thread
     const float* th = a.params + net * P.p_net;
     const float* wo = th + 4 * H + (int64_t)(L - 1) * (H * H + H);
-
-    // ---- layer 1 (3 -> H): exact increments mu = 0, del_i = h W1[u][i]
-    if (own) {
-      const int u = lane;
-      const float w0 = th[3 * u], w1 = th[3 * u + 1], w2 = th[3 * u + 2], bb = th[3 * H + u];
-      float zc[8] = {fmaf(w0, px, fmaf(w1, py, fmaf(w2, pz, bb))), 0.f, 0.f, 0.f, w0, w1, w2,
-                     jump ? fmaf(w0, gx, fmaf(w1, gy, fmaf(w2, gz, bb))) : 0.f};
-      float o[8];
-      layer_fwd<ACT>(zc, jump, hf, h2f, ihf, ih2f, o);
-      st8(Z(0, w, u), zc);
-      st8(A(0, w, u), o);
+    for (int i = tid; i < (L - 1) * H * H; i += NT) {
+      const int g = i / (H * H), r = i - g * H * H;
+      const float v = th[4 * H + (int64_t)g * (H * H + H) + r];
+      Wb[i] = v;
+      Wf[g * H * H + (r % H) * H + r / H] = v;
     }
-    __syncwarp();
-
-    // ---- hidden layers (H -> H), FP32 FFMA
-#pragma unroll 1
-    for (int g = 1; g < L; ++g) {
-      const float* WT = a.wt + ((int64_t)net * (L - 1) + (g - 1)) * H * H;  // [k][u]
-      const float* bg = th + 4 * H + (int64_t)(g - 1) * (H * H + H) + (int64_t)H * H;
-      if (own) {
-        const int u = lane;
-        const float bb = bg[u];
-        float acc[8] = {bb, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, bb};
-        for (int k = 0; k < H; ++k) {
-          float av[8];
-          ld8(A(g - 1, w, k), av);
-          const float wv = WT[(int64_t)k * H + u];
-#pragma unroll
-          for (int c = 0; c < 8; ++c) acc[c] = fmaf(wv, av[c], acc[c]);
+    // record of point q < ppw of tile tau: the list entry, then what it points to
+    auto entry = [&](int64_t tau) -> int {
+      const int64_t slot = (tau - (net ? T0 : 0)) * ppw + lane;
+      if (tau >= s1 || lane >= ppw) return INT_MIN;  // no point
+      if (cutfwd) return slot < nc ? -(int)slot - 1 : INT_MIN;
+      return slot < (net ? np : nm) ? a.list[net][slot] : INT_MIN;
+    };
+    auto fill = [&](int e, int b) {
+      if (lane >= ppw) return;
+      SmallRec r;
+      r.x = r.y = r.z = r.gx = r.gy = r.gz = 0.f;
+      r.pt = -1;
+      r.cutj = -1;
+      if (e != INT_MIN) {
+        r.pt = e;
+        if (e < 0) {
+          const CutRec& c = a.cut[-e - 1];
+          r.pt = c.point;
+          r.cutj = 2 * (-e - 1) + (c.has_jump ? 1 : 0);
+          r.gx = (float)c.xg[0];
+          r.gy = (float)c.xg[1];
+          r.gz = (float)c.xg[2];
         }
+        r.x = a.x[r.pt];
+        r.y = a.y[r.pt];
+        r.z = a.z[r.pt];
+      }
+      recs[b * kMaxPt + lane] = r;
+    };
+    if (s0 + w < s1) fill(entry(s0 + w), 0);
+    __syncthreads();  // the weights
+
+    int buf = 0;
+#pragma unroll 1
+    for (int64_t tau = s0 + w; tau < s1; tau += NW, buf ^= 1) {
+      __syncwarp();
+      const int e_next = entry(tau + NW);  // loaded while this tile computes
+      const SmallRec& r = recs[buf * kMaxPt + pq];
+      const bool jump = r.cutj >= 0 && (r.cutj & 1);
+
+      // ---- layer 1 (3 -> H): exact increments mu = 0, del_i = h W1[u][i]
+      {
+        const float w0 = th[3 * u], w1 = th[3 * u + 1], w2 = th[3 * u + 2], bb = th[3 * H + u];
+        const float zc[8] = {fmaf(w0, r.x, fmaf(w1, r.y, fmaf(w2, r.z, bb))), 0.f, 0.f, 0.f, w0, w1,
+                             w2, jump ? fmaf(w0, r.gx, fmaf(w1, r.gy, fmaf(w2, r.gz, bb))) : 0.f};
         float o[8];
-        layer_fwd<ACT>(acc, jump, hf, h2f, ihf, ih2f, o);
-        st8(Z(g, w, u), acc);
-        st8(A(g, w, u), o);
+        layer_fwd<ACT>(zc, jump, hf, h2f, ihf, ih2f, o);
+        if (own) {
+          if constexpr (ACT == NBM_ACT_SIN) st8(Zb, lane, zc);
+          st8(Ab, lane, o);
+        }
       }
       __syncwarp();
-    }
 
-    // ---- output layer (H -> 1): warp reduction over units
-    float out[8];
-    {
-      float oc[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
-      if (own) ld8(A(L - 1, w, lane), oc);
-      const float wv = own ? wo[lane] : 0.f;
-#pragma unroll
-      for (int c = 0; c < 8; ++c) {
-        float v = wv * oc[c];
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-        out[c] = v;
-      }
-      out[0] += wo[H];
-      out[7] += wo[H];
-    }
-
-    if (a.mode == MODE_CUT_FWD) {
-      if (valid && lane == 0) {
-        float* co = a.cut_out + (int64_t)cut_id * 16 + net * 8;
-        st8(co, out);
-      }
-      continue;
-    }
-
-    // ---- residual row and seeds (every lane computes the same row)
-    float seeds[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
-    if (valid && cut_id < 0) {
-      double r2;
-      if (P.fp64) r2 = uncut_residual<double>(P, net, px, py, pz, out, (double)a.scale, seeds);
-      else r2 = (double)uncut_residual<float>(P, net, px, py, pz, out, a.scale, seeds);
-      if (lane == 0) {
-        loss_acc += r2;
-        if (a.r2_out) a.r2_out[pt] = (P.level ? a.r2_out[pt] : 0.f) + (float)r2;
-      }
-    } else if (valid && train) {
-      ld8(a.cut_seed + (int64_t)cut_id * 16 + net * 8, seeds);
-    }
-    if (!train) continue;
-
-    // ---- backward: output layer
-    float G[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
-    if (own) {
-      float oc[8];
-      ld8(A(L - 1, w, lane), oc);
-      const float wv = wo[lane];
-      float s = 0.f;
-#pragma unroll
-      for (int c = 0; c < 8; ++c) {
-        s = fmaf(seeds[c], oc[c], s);
-        G[c] = wv * seeds[c];
-      }
-      gwo += s;
-    }
-    if (lane == 0) gbo += seeds[0] + seeds[7];
-
-    // ---- backward through the hidden layers g = L-1 .. 1
+      // ---- hidden layers (H -> H), FP32 FFMA
 #pragma unroll 1
-    for (int g = L - 1; g >= 1; --g) {
-      // adjoint of the activation layer that produced act[g]; the gradient with
-      // respect to its pre-activation columns replaces them in Z
-      if (own) {
-        float zc[8], oc[8], gzv[8];
-        ld8(Z(g, w, lane), zc);
-        ld8(A(g, w, lane), oc);
-        layer_bwd<ACT>(zc, oc, G, hf, h2f, ihf, ih2f, gzv);
-        const float gsum = gzv[0] + gzv[7];
+      for (int g = 1; g < L; ++g) {
+        const float* Wg = Wf + (g - 1) * H * H + u;
+        const float* ap = Ab + (g - 1) * 256;
+        const float bb = th[4 * H + (int64_t)(g - 1) * (H * H + H) + H * H + u];
+        F2 acc[4] = {f2(bb, 0.f), f2(0.f, 0.f), f2(0.f, 0.f), f2(0.f, bb)};
+#pragma unroll 2
+        for (int k = 0; k < H; ++k) {
+          float av[8];
+          ld8(ap, pbase + k, av);
+          const F2 wv = f2s(Wg[k * H]);
 #pragma unroll
-        for (int i = 0; i < kLM - 1; ++i) gbh[i] += (g - 1 == i) ? gsum : 0.f;
-        st8(Z(g, w, lane), gzv);
+          for (int c = 0; c < 4; ++c) acc[c] = fma2(wv, f2(av[2 * c], av[2 * c + 1]), acc[c]);
+        }
+        float zc[8], o[8];
+#pragma unroll
+        for (int c = 0; c < 4; ++c) f2get(acc[c], zc[2 * c], zc[2 * c + 1]);
+        layer_fwd<ACT>(zc, jump, hf, h2f, ihf, ih2f, o);
+        if (own) {
+          if constexpr (ACT == NBM_ACT_SIN) st8(Zb + g * 256, lane, zc);
+          st8(Ab + g * 256, lane, o);
+        }
+        __syncwarp();
       }
-      __syncthreads();
-      // weight gradient of hidden layer g: dW[u][k] += sum_{pw,c} gz[pw][u][c] act[g-1][pw][k][c]
+
+      // ---- output layer and residual rows: 8 lanes per point, lane 8 q + c sums
+      // column c of point q and takes one face of its row
       {
-        float* gp = a.gpart + ((int64_t)blockIdx.x * 2 + net) * P.gstride + 4 * H +
-                    (int64_t)(g - 1) * (H * H + H);
-        for (int idx = tid; idx < H * H; idx += blockDim.x) {
-          const int u = idx / H, k = idx % H;
-          float acc = 0.f;
-#pragma unroll 1
-          for (int pw = 0; pw < kSPT; ++pw) {
-            float gv[8], av[8];
-            ld8(Z(g, pw, u), gv);
-            ld8(A(g - 1, pw, k), av);
-#pragma unroll
-            for (int c = 0; c < 8; ++c) acc = fmaf(gv[c], av[c], acc);
+        const int q = lane >> 3, c = lane & 7;
+        const unsigned gmask = 0xFFu << (lane & 24);
+        if (q < ppw) {
+          const SmallRec& rq = recs[buf * kMaxPt + q];
+          const float* ap = Ab + (L - 1) * 256;
+          float oc = (c == 0 || c == 7) ? wo[H] : 0.f;
+          for (int k = 0; k < H; ++k)
+            oc = fmaf(wo[k], ap[half_off(q * H + k, c >> 2) + (c & 3)], oc);
+          const float Uc = __shfl_sync(gmask, oc, 0, 8);
+          const float Mtc = __shfl_sync(gmask, oc, 1 + (c >> 1), 8);
+          const float Dtc = __shfl_sync(gmask, oc, 4 + (c >> 1), 8);
+          float sd = 0.f;
+          if (cutfwd) {
+            if (rq.pt >= 0) a.cut_out[(int64_t)(rq.cutj >> 1) * 16 + net * 8 + c] = oc;
+          } else if (rq.pt >= 0 && rq.cutj < 0) {
+            double r2;
+            if (P.fp64) {
+              const double f = c == 6 ? rhs_f<double>(P, net, rq.x, rq.y, rq.z) : 0.0;
+              r2 = uncut_residual_lanes<double>(P, net, rq.x, rq.y, rq.z, f, Uc, Mtc, Dtc,
+                                                (double)a.scale, c, gmask, sd);
+            } else {
+              const float f = c == 6 ? rhs_f<float>(P, net, rq.x, rq.y, rq.z) : 0.f;
+              r2 = uncut_residual_lanes<float>(P, net, rq.x, rq.y, rq.z, f, Uc, Mtc, Dtc, a.scale,
+                                               c, gmask, sd);
+            }
+            if (c == 0) {
+              loss_acc += r2;
+              if (a.r2_out) a.r2_out[rq.pt] = (P.level ? a.r2_out[rq.pt] : 0.f) + (float)r2;
+            }
+          } else if (rq.pt >= 0 && train) {
+            sd = a.cut_seed[(int64_t)(rq.cutj >> 1) * 16 + net * 8 + c];
           }
-          gp[idx] = first_tile ? acc : gp[idx] + acc;
+          seeds_s[lane] = sd;
+          if (c == 0 || c == 7) gbo += sd;
         }
       }
-      // input gradient: G[k][c] = sum_u W_g[u][k] gz[u][c]
-      if (own) {
-        const float* Wg = th + 4 * H + (int64_t)(g - 1) * (H * H + H);
-#pragma unroll
-        for (int c = 0; c < 8; ++c) G[c] = 0.f;
-        for (int u = 0; u < H; ++u) {
-          float gv[8];
-          ld8(Z(g, w, u), gv);
-          const float wv = Wg[(int64_t)u * H + lane];
-#pragma unroll
-          for (int c = 0; c < 8; ++c) G[c] = fmaf(wv, gv[c], G[c]);
-        }
-      }
-      __syncthreads();
-    }
+      fill(e_next, buf ^ 1);
+      if (!train) continue;
+      __syncwarp();
 
-    // ---- adjoint of layer 1 and its (3 -> H) parameter gradient; the
-    // increments del_i = h W1[u][i] give d(dt_i)/dW1[u][i] = 1 (scaled columns)
-    if (own) {
-      float zc[8], oc[8], gzv[8];
-      ld8(Z(0, w, lane), zc);
-      ld8(A(0, w, lane), oc);
-      layer_bwd<ACT>(zc, oc, G, hf, h2f, ihf, ih2f, gzv);
-      gW1[0] += fmaf(gzv[0], px, fmaf(gzv[7], gx, gzv[4]));
-      gW1[1] += fmaf(gzv[0], py, fmaf(gzv[7], gy, gzv[5]));
-      gW1[2] += fmaf(gzv[0], pz, fmaf(gzv[7], gz, gzv[6]));
-      gb1 += gzv[0] + gzv[7];
+      // ---- backward: output layer
+      float G[8];
+      {
+        const float4 lo = *reinterpret_cast<const float4*>(seeds_s + 8 * pq);
+        const float4 hi = *reinterpret_cast<const float4*>(seeds_s + 8 * pq + 4);
+        const float sd[8] = {lo.x, lo.y, lo.z, lo.w, hi.x, hi.y, hi.z, hi.w};
+        float oc[8];
+        ld8(Ab + (L - 1) * 256, lane, oc);
+        const float wv = wo[u];
+        float s = 0.f;
+#pragma unroll
+        for (int c = 0; c < 8; ++c) {
+          s = fmaf(sd[c], oc[c], s);
+          G[c] = wv * sd[c];
+        }
+        gwo += s;
+      }
+
+      // ---- backward through the hidden layers g = L-1 .. 1: the adjoint of the
+      // activation layer, then the weight gradient dW[u][k] += gz[u] . act[k] of
+      // this lane's unit and point, and G[u] = sum_k W[k][u] gz[k]
+#pragma unroll
+      for (int g = kLM - 1; g >= 1; --g) {
+        if (g >= L) continue;
+        float zc[8], oc[8], gzv[8];
+        if constexpr (ACT == NBM_ACT_SIN) ld8(Zb + g * 256, lane, zc);
+        ld8(Ab + g * 256, lane, oc);
+        layer_bwd<ACT>(zc, oc, G, jump, hf, h2f, ihf, ih2f, gzv);
+        gbh[g - 1] += gzv[0] + gzv[7];
+        if (own) st8(Zb + g * 256, lane, gzv);
+        __syncwarp();
+        const float* ap = Ab + (g - 1) * 256;
+        const float* zp = Zb + g * 256;
+        const float* Wg = Wb + (g - 1) * H * H + u;
+        F2 gg[4], acc[4];
+#pragma unroll
+        for (int c = 0; c < 4; ++c) {
+          gg[c] = f2(gzv[2 * c], gzv[2 * c + 1]);
+          acc[c] = f2(0.f, 0.f);
+        }
+#pragma unroll
+        for (int k = 0; k < HM; ++k) {
+          if (k < H) {
+            float av[8], gv[8];
+            ld8(ap, pbase + k, av);
+            ld8(zp, pbase + k, gv);
+            F2 d = mul2(gg[0], f2(av[0], av[1]));
+#pragma unroll
+            for (int c = 1; c < 4; ++c) d = fma2(gg[c], f2(av[2 * c], av[2 * c + 1]), d);
+            float ev, od;
+            f2get(d, ev, od);
+            gW[g - 1][k] += ev + od;
+            const F2 wv = f2s(Wg[k * H]);
+#pragma unroll
+            for (int c = 0; c < 4; ++c) acc[c] = fma2(wv, f2(gv[2 * c], gv[2 * c + 1]), acc[c]);
+          }
+        }
+#pragma unroll
+        for (int c = 0; c < 4; ++c) f2get(acc[c], G[2 * c], G[2 * c + 1]);
+      }
+
+      // ---- adjoint of layer 1 and its (3 -> H) parameter gradient; the
+      // increments del_i = h W1[u][i] give d(dt_i)/dW1[u][i] = 1 (scaled columns)
+      {
+        float zc[8], oc[8], gzv[8];
+        if constexpr (ACT == NBM_ACT_SIN) ld8(Zb, lane, zc);
+        ld8(Ab, lane, oc);
+        layer_bwd<ACT>(zc, oc, G, jump, hf, h2f, ihf, ih2f, gzv);
+        gW1[0] += fmaf(gzv[0], r.x, fmaf(gzv[7], r.gx, gzv[4]));
+        gW1[1] += fmaf(gzv[0], r.y, fmaf(gzv[7], r.gy, gzv[5]));
+        gW1[2] += fmaf(gzv[0], r.z, fmaf(gzv[7], r.gz, gzv[6]));
+        gb1 += gzv[0] + gzv[7];
+      }
     }
-    first_tile = false;
+    if (train) flush(net);
+    else __syncthreads();  // before the next network's weights
   }
-  if (train && cur_net >= 0) flush(cur_net);
   // loss partial of this CTA (fixed order)
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) loss_acc += __shfl_xor_sync(0xffffffffu, loss_acc, o);
   if (lane == 0) loss_red[w] = loss_acc;
   __syncthreads();
   if (tid == 0) {
     double s = 0.0;
-    for (int ww = 0; ww < 8; ++ww) s += loss_red[ww];
-    if (a.mode != MODE_CUT_FWD) a.loss_part[blockIdx.x] = s;
+    for (int ww = 0; ww < NW; ++ww) s += loss_red[ww];
+    if (!cutfwd) a.loss_part[blockIdx.x] = s;
     if (train) {
       a.gpart_flag[2 * blockIdx.x] = wrote0;
       a.gpart_flag[2 * blockIdx.x + 1] = wrote1;
@@ -387,19 +470,22 @@ __global__ void __launch_bounds__(256, 1) k_step_small(ProbDev P, StepArgs a) {
   }
 }
 
-template <int ACT>
+template <int ACT, int HM>
 static cudaError_t launch_small_t(const ProbDev& P, const StepArgs& a, int grid, cudaStream_t st) {
-  const size_t smem = small_smem_bytes(P.L);
-  cudaError_t e = cudaFuncSetAttribute(k_step_small<ACT>,
+  const size_t smem = small_smem_bytes(P.H, P.L, HM);
+  cudaError_t e = cudaFuncSetAttribute(k_step_small<ACT, HM>,
                                        cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;
-  return launch_pdl(k_step_small<ACT>, dim3(grid), dim3(256), smem, st, P, a);
+  return launch_pdl(k_step_small<ACT, HM>, dim3(grid), dim3(small_threads(HM)), smem, st, P, a);
 }
 
 cudaError_t launch_step_small(const ProbDev& P, const StepArgs& a, int grid, cudaStream_t st) {
-  if (P.H < 1 || P.H > kHM || P.L < 2 || P.L > kLM) return cudaErrorInvalidValue;
-  if (P.activation == NBM_ACT_SIN) return launch_small_t<NBM_ACT_SIN>(P, a, grid, st);
-  return launch_small_t<NBM_ACT_TANH>(P, a, grid, st);
+  if (P.H < 1 || P.H > 32 || P.L < 2 || P.L > kLM) return cudaErrorInvalidValue;
+  const bool sine = P.activation == NBM_ACT_SIN;
+  if (P.H <= 16) return sine ? launch_small_t<NBM_ACT_SIN, 16>(P, a, grid, st)
+                             : launch_small_t<NBM_ACT_TANH, 16>(P, a, grid, st);
+  return sine ? launch_small_t<NBM_ACT_SIN, 32>(P, a, grid, st)
+              : launch_small_t<NBM_ACT_TANH, 32>(P, a, grid, st);
 }
 
 }  // namespace nbm

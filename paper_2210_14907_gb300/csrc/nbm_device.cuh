@@ -480,14 +480,23 @@ __device__ __forceinline__ void tanh_stencil_fwd0(float t, float dt, float h, fl
 // cosine by Taylor series, sin x = x (1 - x^2/6 + x^4/120) + R, |R| <= |x|^7/5040,
 // cos x = 1 - x^2/2 + x^4/24 + R, |R| <= x^6/720, relative errors below 1e-10.
 // ---------------------------------------------------------------------------
+// The full-range sincosf is a call: inlined at each of its 50 places it made the
+// narrow step kernel 100 KB of code, and its warps waited for instructions.
 constexpr float kSmallHalf = 0.0625f;
+static __device__ __noinline__ float2 sincos_full(float x) {
+  float2 r;
+  sincosf(x, &r.x, &r.y);
+  return r;
+}
 __device__ __forceinline__ void sincos_half(float x, bool small, float& s, float& c) {
   if (small) {
     const float x2 = x * x;
     s = x * fmaf(x2, fmaf(x2, 1.0f / 120.0f, -1.0f / 6.0f), 1.0f);
     c = fmaf(x2, fmaf(x2, 1.0f / 24.0f, -0.5f), 1.0f);
   } else {
-    sincosf(x, &s, &c);
+    const float2 r = sincos_full(x);
+    s = r.x;
+    c = r.y;
   }
 }
 __device__ __forceinline__ void sin_stencil_fwd(float sz, float cz, float mt, float dt, float h,

@@ -32,7 +32,7 @@ constexpr int kMaxPt = 4;  // points per warp (8 lanes each for the rows)
 
 template <int ACT>
 __device__ __forceinline__ float act_f(float z) {
-  if constexpr (ACT == NBM_ACT_SIN) return sinf(z);
+  if constexpr (ACT == NBM_ACT_SIN) return sincos_full(z).x;
   else return act_tanh<false>(z);
 }
 
@@ -58,8 +58,8 @@ __device__ __forceinline__ void layer_fwd(const float zc[8], bool jump, float h,
   bool sm_mu, sm_de;
   small_increments<ACT>(zc, h, h2, sm_mu, sm_de);
   if constexpr (ACT == NBM_ACT_SIN) {
-    float sz, cz;
-    sincosf(zc[0], &sz, &cz);
+    const float2 sc = sincos_full(zc[0]);
+    const float sz = sc.x, cz = sc.y;
     o[0] = sz;
 #pragma unroll
     for (int i = 0; i < 3; ++i)
@@ -85,15 +85,15 @@ __device__ __forceinline__ void layer_bwd(const float zc[8], const float oc[8], 
   if constexpr (ACT == NBM_ACT_SIN) {
     bool small, unused;
     small_increments<ACT>(zc, h, h2, small, unused);
-    float sz, cz;
-    sincosf(zc[0], &sz, &cz);
+    const float2 sc = sincos_full(zc[0]);
+    const float sz = sc.x, cz = sc.y;
     float gzc = cz * G[0];
 #pragma unroll
     for (int i = 0; i < 3; ++i)
       gzc += sin_stencil_bwd(sz, cz, zc[1 + i], zc[4 + i], G[1 + i], G[4 + i], h, h2, ih, ih2,
                              gz[1 + i], gz[4 + i], small);
     gz[0] = gzc;
-    gz[7] = jump ? cosf(zc[7]) * G[7] : 0.f;
+    gz[7] = jump ? sincos_full(zc[7]).y * G[7] : 0.f;
   } else {
     const float t = oc[0], s0 = fmaf(-t, t, 1.f);
     float gzc = s0 * G[0];
@@ -397,15 +397,17 @@ __global__ void __launch_bounds__(small_threads(HM), 1) k_step_small(ProbDev P, 
 
       // ---- backward through the hidden layers g = L-1 .. 1: the adjoint of the
       // activation layer, then the weight gradient dW[u][k] += gz[u] . act[k] of
-      // this lane's unit and point, and G[u] = sum_k W[k][u] gz[k]
-#pragma unroll
-      for (int g = kLM - 1; g >= 1; --g) {
-        if (g >= L) continue;
+      // this lane's unit and point, and G[u] = sum_k W[k][u] gz[k].  (Not unrolled:
+      // the layer's sums are picked by a predicate, four copies of this body
+      // would not fit the instruction cache.)
+#pragma unroll 1
+      for (int g = L - 1; g >= 1; --g) {
         float zc[8], oc[8], gzv[8];
         if constexpr (ACT == NBM_ACT_SIN) ld8(Zb + g * 256, lane, zc);
         ld8(Ab + g * 256, lane, oc);
         layer_bwd<ACT>(zc, oc, G, jump, hf, h2f, ihf, ih2f, gzv);
-        gbh[g - 1] += gzv[0] + gzv[7];
+#pragma unroll
+        for (int i = 0; i < kLM - 1; ++i) gbh[i] += (g - 1 == i) ? gzv[0] + gzv[7] : 0.f;
         if (own) st8(Zb + g * 256, lane, gzv);
         __syncwarp();
         const float* ap = Ab + (g - 1) * 256;
@@ -428,7 +430,10 @@ __global__ void __launch_bounds__(small_threads(HM), 1) k_step_small(ProbDev P, 
             for (int c = 1; c < 4; ++c) d = fma2(gg[c], f2(av[2 * c], av[2 * c + 1]), d);
             float ev, od;
             f2get(d, ev, od);
-            gW[g - 1][k] += ev + od;
+            const float dw = ev + od;
+#pragma unroll
+            for (int i = 0; i < kLM - 1; ++i)
+              if (g - 1 == i) gW[i][k] += dw;
             const F2 wv = f2s(Wg[k * H]);
 #pragma unroll
             for (int c = 0; c < 4; ++c) acc[c] = fma2(wv, f2(gv[2 * c], gv[2 * c + 1]), acc[c]);

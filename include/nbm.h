@@ -258,8 +258,9 @@ int nbm_train_steps(nbm_problem* p, float* params, float* adam_m, float* adam_v,
  * Node (i,j,k) is u_out[i + (n+1)(j + (n+1)k)], a caller-owned DEVICE array.
  * `precision` selects the hidden-GEMM type (nbm_precision): NBM_PREC_FP32
  * (CUDA cores; asynchronous), or NBM_PREC_BF16 / NBM_PREC_FP16 (tensor cores;
- * width 128 and 2..4 hidden layers only; these allocate their scratch,
- * synchronize the stream and free it).
+ * width 128 and 2..4 hidden layers only; these keep their scratch with the
+ * problem -- the sides of more than 2^29 points or so are allocated for the
+ * call -- and synchronize the stream).
  * Returns NBM_ERR_INVALID_ARG for a NULL or misaligned argument, n outside
  * 1..4096 or an unsupported precision, NBM_ERR_OOM if the scratch cannot be
  * allocated, NBM_ERR_DEVICE_TIMEOUT if a bounded device wait gave up. */

@@ -320,6 +320,7 @@ namespace nbm {
 void set_error_message(const char* msg) { snprintf(g_err, sizeof(g_err), "%s", msg); }
 const nbm_problem_desc& problem_desc(const nbm_problem* p) { return p->pb.desc; }
 int problem_num_sms(const nbm_problem* p) { return p->pb.num_sms; }
+EvalScratch& problem_eval_scratch(nbm_problem* p) { return p->pb.eval; }
 int check_aligned(const void* ptr, size_t align, const char* name) {
   if (ptr && ((uintptr_t)ptr & (align - 1)) != 0)
     return fail(NBM_ERR_INVALID_ARG, "%s is not %zu-byte aligned", name, align);
@@ -365,6 +366,9 @@ int nbm_destroy(nbm_problem* p) {
   if (!p) return NBM_OK;
   ws_free(p->pb.ws);
   if (p->pb.phi_grid) cudaFree(p->pb.phi_grid);
+  const EvalScratch& ev = p->pb.eval;
+  for (void* q : {(void*)ev.wimg, (void*)ev.status, (void*)ev.side})
+    if (q) cudaFree(q);
   for (cudaEvent_t& e : p->pb.prof.ev)
     if (e) cudaEventDestroy(e);
   delete p;

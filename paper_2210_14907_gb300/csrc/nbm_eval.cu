@@ -26,6 +26,7 @@ namespace {
 using namespace tc;
 
 constexpr int kImgE = 32768;
+constexpr size_t kKeepSideBytes = (size_t)64 << 20;
 // 64-point tiles in flight per warp group of the tensor-core evaluation, and the
 // TMEM columns they take (2 groups x kEvalTiles x 64, rounded up to a power of 2)
 constexpr int kEvalTiles = 3;
@@ -796,20 +797,37 @@ static int eval_common(nbm_problem* p, const float* params, int n, const float* 
 #undef NBM_EVAL32
     else e = cudaErrorInvalidValue;
   } else {
-    // the 16-bit weight images of both networks, in the shared-memory layout
+    // The scratch stays with the problem: three allocations and frees per call cost
+    // 160 us of the 220 that a call with a few points took.  The sides of very many
+    // points (over kKeepSideBytes, 537 M points) are allocated for the call.
     const size_t bytes = (size_t)2 * (d.n_hidden - 1) * kImgE;
-    unsigned char* wimg = nullptr;
-    int* status = nullptr;
-    uint4* side = nullptr;  // per 128-point tile: bit c set if point c is in Omega-
     const int64_t total = pts ? npts : (int64_t)(n + 1) * (n + 1) * (n + 1);
-    e = cudaMalloc((void**)&wimg, bytes);
-    if (e == cudaSuccess) e = cudaMalloc((void**)&status, sizeof(int));
-    if (e == cudaSuccess) e = cudaMalloc((void**)&side, sizeof(uint4) * (size_t)((total + 127) / 128));
+    const int64_t side_n = (total + 127) / 128;
+    EvalScratch& ev = problem_eval_scratch(p);
+    if (!ev.wimg) e = cudaMalloc((void**)&ev.wimg, bytes);
+    if (e == cudaSuccess && !ev.status) e = cudaMalloc((void**)&ev.status, sizeof(int));
+    uint4* side = nullptr;  // per 128-point tile: bit c set if point c is in Omega-
+    const bool own_side = sizeof(uint4) * (size_t)side_n > kKeepSideBytes;
+    if (e == cudaSuccess && own_side) {
+      e = cudaMalloc((void**)&side, sizeof(uint4) * (size_t)side_n);
+    } else if (e == cudaSuccess) {
+      if (ev.side_cap < side_n) {
+        if (ev.side) cudaFree(ev.side);
+        ev.side = nullptr;
+        ev.side_cap = 0;
+        e = cudaMalloc((void**)&ev.side, sizeof(uint4) * (size_t)side_n);
+        if (e == cudaSuccess) ev.side_cap = side_n;
+      }
+      side = ev.side;
+    }
+    unsigned char* wimg = ev.wimg;
+    int* status = ev.status;
     if (e == cudaSuccess) e = cudaMemsetAsync(status, 0, sizeof(int), st);
     Workspace tmp;
     tmp.wtc = wimg;
     if (e == cudaSuccess) e = launch_prep_weights(P, params, precision, tmp, st);
-    const int grid = problem_num_sms(p);
+    const int64_t tiles = (total + 63) / 64;
+    const int grid = (int)(tiles < problem_num_sms(p) ? tiles : problem_num_sms(p));
     const bool bf = precision == NBM_PREC_BF16;
     if (e == cudaSuccess) {
       if (d.n_hidden == 2) e = bf ? launch_eval_tc_t<2, true>(P, params, wimg, n, pts, npts, u_out, side, grid, status, st)
@@ -822,9 +840,8 @@ static int eval_common(nbm_problem* p, const float* params, int n, const float* 
     int hs = 0;
     if (e == cudaSuccess) e = cudaMemcpyAsync(&hs, status, sizeof(int), cudaMemcpyDeviceToHost, st);
     if (e == cudaSuccess) e = cudaStreamSynchronize(st);
-    if (wimg) cudaFree(wimg);
-    if (status) cudaFree(status);
-    if (side) cudaFree(side);
+    else cudaStreamSynchronize(st);  // nothing of a failed call still uses the scratch
+    if (own_side && side) cudaFree(side);
     if (e == cudaSuccess && (hs & 2)) {
       set_error_message("grid evaluation: a bounded device wait gave up");
       return NBM_ERR_DEVICE_TIMEOUT;

@@ -125,8 +125,18 @@ struct Profiler {
   std::vector<cudaEvent_t> ev = std::vector<cudaEvent_t>(2 * kMax, nullptr);
 };
 
+// Scratch of the tensor-core evaluation, kept by the problem between calls (a call
+// synchronizes its stream before it returns, so calls never share it on the GPU).
+struct EvalScratch {
+  unsigned char* wimg = nullptr;  // 16-bit weight images of both networks
+  int* status = nullptr;
+  uint4* side = nullptr;          // sides of side_cap 128-point tiles
+  int64_t side_cap = 0;
+};
+
 struct Problem {
   Profiler prof;
+  EvalScratch eval;
   nbm_problem_desc desc;
   int device = 0;
   int num_sms = 0;
@@ -142,6 +152,7 @@ void make_prob_dev(const nbm_problem_desc& d, ProbDev& P, int level = 0);
 void set_error_message(const char* msg);
 const nbm_problem_desc& problem_desc(const nbm_problem* p);
 int problem_num_sms(const nbm_problem* p);
+EvalScratch& problem_eval_scratch(nbm_problem* p);
 // Gives P the problem's mesh level set; NBM_ERR_INVALID_ARG (with the message
 // set) for an NBM_GEOM_GRID problem whose level set has not been set.
 int attach_level_set(const nbm_problem* p, ProbDev& P);

@@ -96,12 +96,19 @@ __device__ __forceinline__ uint32_t tanh_pack2(float a, float b) {
 // a group, thread (q = warp & 3, cg = (warp >> 2) & 1) owns unit 32 q + lane
 // (its TMEM lane) and the tile's points 32 cg .. 32 cg + 31.
 //
+// A 17th and an 18th warp issue the two groups' GEMMs.  A compute warp that has
+// written its part of a tile's image arrives on the tile's `ready` barrier and goes
+// on to the next tile, whose accumulators it waits for by itself; the issuing
+// warp waits for all 8 arrivals.  So the warps of a group meet only at the ends of
+// a set, not after every tile and layer, and run up to a tile apart.
+//
 // Pass 0 (the minus network) decides every point's side and keeps it in
 // `side` (per 128 points, bit c: point c is in Omega-; each 64-point tile owns
 // two of the four words); pass 1 reads it back instead of evaluating the
 // level set again.  A tile without a point of the pass's side is skipped.
+constexpr int kEvalThreads = 576;
 template <int L, bool BF>
-__global__ void __launch_bounds__(512, 1) k_eval_tc(ProbDev P, const float* __restrict__ params,
+__global__ void __launch_bounds__(kEvalThreads, 1) k_eval_tc(ProbDev P, const float* __restrict__ params,
                                                     const unsigned char* __restrict__ wimg, int n,
                                                     const float* __restrict__ pts, int64_t npts,
                                                     float* __restrict__ u_out, uint4* side,
@@ -110,7 +117,8 @@ __global__ void __launch_bounds__(512, 1) k_eval_tc(ProbDev P, const float* __re
   extern __shared__ unsigned char smem_raw[];
   unsigned char* sm = (unsigned char*)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
   const int tid = threadIdx.x, w = tid >> 5, lane = tid & 31;
-  const int grp = tid >> 8, gtid = tid & 255, gw = gtid >> 5;
+  const bool issuer = w >= 16;
+  const int grp = issuer ? w - 16 : tid >> 8, gtid = tid & 255, gw = gtid >> 5;
   const int q = w & 3, cg = (w >> 2) & 1, u = 32 * q + lane, col0 = 32 * cg;
   const uint32_t gbar = 1u + (uint32_t)grp;
   unsigned char* Wimg = sm;                                    // [NG] 32 KB
@@ -118,6 +126,7 @@ __global__ void __launch_bounds__(512, 1) k_eval_tc(ProbDev P, const float* __re
   unsigned char* misc = sm + NG * kImgE + 2 * kX * kImgG;
   uint64_t* bar_w = (uint64_t*)misc;
   uint64_t* bar_mma = (uint64_t*)(misc + 8) + kX * grp;        // this group's [kX]
+  uint64_t* bar_rdy = (uint64_t*)(misc + 64) + kX * grp;       // this group's [kX]
   uint32_t* tslot = (uint32_t*)(misc + 8 + 16 * kX);
   volatile int* abort_f = (volatile int*)(misc + 12 + 16 * kX);
   int* actw = (int*)(misc + 128) + grp * 4 * kX;               // [2 set parities][2 kX warps]
@@ -129,7 +138,10 @@ __global__ void __launch_bounds__(512, 1) k_eval_tc(ProbDev P, const float* __re
   const uint32_t idf = idesc_f16_n(BF, false, true, kTP);
   if (tid == 0) {
     mbar_init(smem_u32(bar_w), 1);
-    for (int b = 0; b < 2 * kX; ++b) mbar_init(smem_u32((uint64_t*)(misc + 8) + b), 1);
+    for (int b = 0; b < 2 * kX; ++b) {
+      mbar_init(smem_u32((uint64_t*)(misc + 8) + b), 1);
+      mbar_init(smem_u32((uint64_t*)(misc + 64) + b), 8);  // one arrival per warp
+    }
     *abort_f = 0;
     fence_mbar_init();
   }
@@ -140,7 +152,8 @@ __global__ void __launch_bounds__(512, 1) k_eval_tc(ProbDev P, const float* __re
   const uint32_t tmem = *tslot;
   const uint32_t d_tm = tmem + (uint32_t)(kX * kTP * grp);  // tile X: d_tm + 64 X
   const uint32_t lane_base = (uint32_t)(32 * q) << 16;
-  // per-tile state as bit X: MMA barrier phase, and a commit not yet waited for
+  // per-tile state as bit X: barrier phase (MMA; in the issuing warps: ready), and
+  // a commit not yet waited for
   uint32_t ph_w = 0, ph_bits = 0, pending_bits = 0;
   const int64_t N1 = n + 1, total = pts ? npts : N1 * N1 * N1;
   const int64_t T = (total + kTP - 1) / kTP;
@@ -155,24 +168,42 @@ __global__ void __launch_bounds__(512, 1) k_eval_tc(ProbDev P, const float* __re
   constexpr int kFreeLayers = (kEvalTmemCols - (int)kWCol) / 64;
   constexpr int kWT = NG < kFreeLayers ? NG : kFreeLayers;
   // the layer-g GEMM of tile X: weights g (K-major; TMEM for g < kWT) x image X
-  // (MN-major)
-  auto issue = [&](int X, int g) {
-    if (gtid == 0) {
-      fence_after_sync();
-      const uint32_t ab = smem_u32(Aimg + X * kImgG);
-      if (g < kWT) {
-        const uint32_t wt = tmem + kWCol + 64u * (uint32_t)g;
-#pragma unroll
-        for (int k = 0; k < 8; ++k)
-          mma_f16_ta(d_tm + kTP * X, wt + 8u * (uint32_t)k, desc_mnmajor(ab, k), idf, k > 0);
+  // (MN-major), once the 8 warps have written the image (issuing warp; a wait that
+  // gave up wakes the waiters without a GEMM)
+  auto issue = [&](int X, int g) -> bool {
+    const bool ok = mbar_wait_bounded(smem_u32(bar_rdy + X), (ph_bits >> X) & 1u);
+    ph_bits ^= 1u << X;
+    fence_after_sync();
+    if (lane == 0) {
+      if (!ok) {
+        atomicOr(status, 2);
+        *abort_f = 1;
+        mbar_arrive(smem_u32(bar_mma + X));
       } else {
-        const uint32_t wa = smem_u32(Wimg + g * kImgE);
+        const uint32_t ab = smem_u32(Aimg + X * kImgG);
+        if (g < kWT) {
+          const uint32_t wt = tmem + kWCol + 64u * (uint32_t)g;
 #pragma unroll
-        for (int k = 0; k < 8; ++k)
-          mma_f16(d_tm + kTP * X, desc_kmajor(wa, k), desc_mnmajor(ab, k), idf, k > 0);
+          for (int k = 0; k < 8; ++k)
+            mma_f16_ta(d_tm + kTP * X, wt + 8u * (uint32_t)k, desc_mnmajor(ab, k), idf, k > 0);
+        } else {
+          const uint32_t wa = smem_u32(Wimg + g * kImgE);
+#pragma unroll
+          for (int k = 0; k < 8; ++k)
+            mma_f16(d_tm + kTP * X, desc_kmajor(wa, k), desc_mnmajor(ab, k), idf, k > 0);
+        }
+        mma_commit(smem_u32(bar_mma + X));
       }
-      mma_commit(smem_u32(bar_mma + X));
     }
+    __syncwarp();
+    return ok;
+  };
+  // this warp's part of tile X's image is written (and its accumulators are read)
+  auto ready = [&](int X) {
+    fence_proxy_async();
+    fence_before_sync();
+    __syncwarp();
+    if (lane == 0) mbar_arrive(smem_u32(bar_rdy + X));
     pending_bits |= 1u << X;
   };
   // bounded wait for tile X's GEMM; false if it gave up
@@ -189,8 +220,8 @@ __global__ void __launch_bounds__(512, 1) k_eval_tc(ProbDev P, const float* __re
   auto end_phase = [&](bool ok) -> bool {
     fence_before_sync();
     fence_proxy_async();
-    const bool bad = named_sync_or(gbar, 256, !ok || *abort_f != 0);
-    if (bad && gtid == 0) {
+    const bool bad = named_sync_or(gbar, 288, !ok || *abort_f != 0);
+    if (bad && !issuer && gtid == 0) {
       if (!ok) atomicOr(status, 2);
       *abort_f = 1;
     }
@@ -233,7 +264,7 @@ __global__ void __launch_bounds__(512, 1) k_eval_tc(ProbDev P, const float* __re
       // set without active tiles has no barrier after its reads
       int* aw = actw + 2 * kX * (set & 1);
       // coordinates and side flags of the tiles' 64 points (threads 0 .. 64 kX - 1)
-      if (gtid < kX * kTP) {
+      if (!issuer && gtid < kX * kTP) {
         const int X = gtid >> 6, c = gtid & 63;
         const int64_t tx = t + 2 * X;
         const int64_t id = tx * kTP + c;
@@ -277,11 +308,24 @@ __global__ void __launch_bounds__(512, 1) k_eval_tc(ProbDev P, const float* __re
         const uint32_t any = __ballot_sync(0xffffffffu, f);
         if (lane == 0) aw[gw] = any != 0u;
       }
-      named_sync(gbar, 256);
+      named_sync(gbar, 288);
       uint32_t act = 0;
 #pragma unroll
       for (int X = 0; X < kX; ++X) act |= ((aw[2 * X] | aw[2 * X + 1]) ? 1u : 0u) << X;
       if (!act) continue;
+      if (issuer) {
+        bool ok = true;
+#pragma unroll 1
+        for (int g = 0; g < NG; ++g)
+#pragma unroll 1
+          for (int X = 0; X < kX; ++X)
+            if ((act >> X) & 1u) ok = issue(X, g) && ok;
+        if (!end_phase(ok)) {
+          aborted = true;
+          break;
+        }
+        continue;
+      }
       // layer 1 (FP32, K = 3) of each active tile -> its image; then its GEMM
 #pragma unroll
       for (int X = 0; X < kX; ++X) {
@@ -306,17 +350,12 @@ __global__ void __launch_bounds__(512, 1) k_eval_tc(ProbDev P, const float* __re
               make_uint4(tanh_pack2<BF>(z[0], z[1]), tanh_pack2<BF>(z[2], z[3]),
                          tanh_pack2<BF>(z[4], z[5]), tanh_pack2<BF>(z[6], z[7]));
         }
+        ready(X);
       }
-      if (!end_phase(true)) {
-        aborted = true;
-        break;
-      }
-      for (int X = 0; X < kX; ++X)
-        if ((act >> X) & 1u) issue(X, 0);
       // hidden layers: while one tile's epilogue runs, the other tile's GEMM does
       bool ok_all = true;  // this thread's MMA waits of the pair
 #pragma unroll 1
-      for (int g = 1; g <= NG && !aborted; ++g) {
+      for (int g = 1; g <= NG; ++g) {
         float bb = bh[0];
 #pragma unroll
         for (int i = 1; i < NG; ++i) bb = (g - 1 == i) ? bh[i] : bb;
@@ -340,11 +379,7 @@ __global__ void __launch_bounds__(512, 1) k_eval_tc(ProbDev P, const float* __re
                   make_uint4(tanh_pack2<BF>(z[0], z[1]), tanh_pack2<BF>(z[2], z[3]),
                              tanh_pack2<BF>(z[4], z[5]), tanh_pack2<BF>(z[6], z[7]));
             }
-            if (!end_phase(ok_all)) {
-              aborted = true;
-              break;
-            }
-            issue(X, g);
+            ready(X);
           } else {
             // output layer (FP32): the sum over units of wo * tanh
             float v[32], sres;
@@ -360,7 +395,6 @@ __global__ void __launch_bounds__(512, 1) k_eval_tc(ProbDev P, const float* __re
           }
         }
       }
-      if (aborted) break;
       if (!end_phase(ok_all)) {
         aborted = true;
         break;
@@ -379,7 +413,7 @@ __global__ void __launch_bounds__(512, 1) k_eval_tc(ProbDev P, const float* __re
     // both groups are done with this network before its weights are replaced
     if (__syncthreads_or(aborted)) aborted = true;
   }
-  if (aborted) {
+  if (aborted && !issuer) {
     if (tid == 0) atomicOr(status, 2);
     // let any GEMM still committed, and a weight copy that a wait gave up on,
     // finish (bounded) before TMEM and shared memory are released
@@ -725,7 +759,7 @@ cudaError_t launch_eval_tc_t(const ProbDev& P, const float* params, const unsign
   cudaError_t e = cudaFuncSetAttribute(k_eval_tc<L, BF>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                        (int)smem);
   if (e != cudaSuccess) return e;
-  k_eval_tc<L, BF><<<grid, 512, smem, st>>>(P, params, wimg, n, pts, npts, u, side, status);
+  k_eval_tc<L, BF><<<grid, kEvalThreads, smem, st>>>(P, params, wimg, n, pts, npts, u, side, status);
   return cudaGetLastError();
 }
 

@@ -60,9 +60,50 @@ __device__ inline void jump_corr(double jmp, int sx, double c[2]) {
   c[1] = sx == 0 ? jmp : 0.0;
 }
 
+// Whether the level set's FP32 value decides the sign of phi outside a band of
+// kSignBand about 0: the sphere, and the flower with few integer lobes (FP32
+// Chebyshev recurrences of degree m err by about m^2 2^-24, at most 1.6e-5 here;
+// the sphere by 2^-22).
+constexpr float kSignBand = 2e-4f;
+inline bool f32_signs(const ProbDev& P) {
+  if (P.geometry == NBM_GEOM_FLOWER)
+    return P.lt_i >= 0 && P.lt_i <= 16 && P.lp_i >= 0 && P.lp_i <= 16;
+  return P.geometry != NBM_GEOM_GRID;
+}
+
+// Whether the cell of node p and its six neighbour nodes lie on one side, by FP32
+// values all outside the band about 0 (false: undecided, or cut).  Sets that side.
+__device__ inline bool one_sided(const ProbDev& P, const double p[3], double h, int& side) {
+  const float x = (float)p[0], y = (float)p[1], z = (float)p[2], hh = (float)(0.5 * h), hf = (float)h;
+  float lo = phi_f(P, x, y, z), hi = lo;
+  auto add = [&](float f) {
+    lo = fminf(lo, f);
+    hi = fmaxf(hi, f);
+  };
+#pragma unroll
+  for (int c = 0; c < 8; ++c)
+    add(phi_f(P, x + ((c & 1) ? hh : -hh), y + ((c & 2) ? hh : -hh), z + ((c & 4) ? hh : -hh)));
+#pragma unroll
+  for (int c = 0; c < 2; ++c) {
+    const float d = c ? hf : -hf;
+    add(phi_f(P, x + d, y, z));
+    add(phi_f(P, x, y + d, z));
+    add(phi_f(P, x, y, z + d));
+  }
+  side = lo > 0.f ? 1 : 0;
+  return lo > kSignBand || hi < -kSignBand;
+}
+
 // Rows of every interior node.  Jn (interior-node array) holds the node jump
 // J = u+ - u- carried to each node; NULL takes the manufactured pair's own
 // u+(x) - u-(x) (the exact jump).
+// FAST: a node whose cell and neighbours are on one side (FP32 decides) takes
+// its row without cell geometry and node jumps: every term left out is a product
+// with an exact 0, and the rest is summed in the same order, so the rows are the
+// same to the last bit.  The FP64 pipe bounds the full row (15 level-set values
+// and 7 exact jumps per node): 256^3 took 35 ms, and only the few per cent of
+// nodes about the interface still pay for it.
+template <bool FAST>
 __global__ void __launch_bounds__(kB) k_grid_rows(ProbDev P, Grid G, const double* Jn,
                                                   double* diag, double* wx, double* wy, double* wz,
                                                   double* rhs) {
@@ -73,6 +114,33 @@ __global__ void __launch_bounds__(kB) k_grid_rows(ProbDev P, Grid G, const doubl
   double p[3];
   node_xyz(G, r, idx[0], idx[1], idx[2], p);
   const double h = G.h;
+  if constexpr (FAST) {
+    int s;
+    if (one_sided(P, p, h, s)) {
+      double dg = h * h * P.k[s];
+      double known = h * h * (0.0 - rhs_f<double>(P, s, p[0], p[1], p[2]));
+      double wplus[3] = {0.0, 0.0, 0.0};
+      for (int f = 0; f < 6; ++f) {
+        const int ax = f >> 1, sg = (f & 1) ? 1 : -1;
+        int nb[3] = {idx[0], idx[1], idx[2]};
+        nb[ax] += sg;
+        double fc[3] = {p[0], p[1], p[2]};
+        fc[ax] += 0.5 * sg * h;
+        const double wf = mu_at<double>(P, s, fc[0], fc[1], fc[2]);
+        dg += wf;
+        if (nb[ax] == 0 || nb[ax] == G.n)
+          known -= wf * dirichlet_g<double>(P, node_coord(nb[0], h), node_coord(nb[1], h),
+                                            node_coord(nb[2], h));
+        else if (sg > 0) wplus[ax] = wf;
+      }
+      diag[r] = dg;
+      wx[r] = wplus[0];
+      wy[r] = wplus[1];
+      wz[r] = wplus[2];
+      rhs[r] = -known;
+      return;
+    }
+  }
   CellGeo cg;
   cell_geometry_d(P, p, h, cg);
   const int sp = phase_d(P, p);
@@ -164,7 +232,8 @@ __device__ inline void block_partials(T (&v)[NV], double* part, int64_t idx, int
 // scalars[]: 0 rz, 1 pAp, 2 alpha, 3 rz_new, 4 rr, 5 beta (the CG recurrence
 // on the Jacobi-scaled system); 6 ||r|| and 7 1/||r|| (the FP64 residual of the
 // refined solve, unscaled norm), 8 sum d r^2 (= ||r||^2), 9 sum d b^2
-// (= ||b||^2), 12 max |dJ|, 13 max |J| (node jump).  After the sums, POST_ALPHA
+// (= ||b||^2), 12 max |dJ|, 13 max |J| (node jump), 14 iterations and 15 the
+// gave-up mark of k_cg_persist.  After the sums, POST_ALPHA
 // sets alpha = rz / pAp, POST_BETA sets beta = rz_new / rz and rz = rz_new,
 // POST_NORM sets ||r|| and its inverse; POST_SKIP leaves the partials unused.
 enum { POST_SKIP = -1, POST_ALPHA = 1, POST_BETA = 2, POST_NORM = 3 };
@@ -237,6 +306,18 @@ __global__ void __launch_bounds__(kB) k_reduce_parts(const double* part, int npa
   sum_partials(part, nparts, nvec, sc, slot, post, false);
 }
 
+// Row codes of the FP32 operator of a constant-mu problem: away from the
+// interface a row's diagonal, its inverse and its six weights are one of two sets of
+// constants, the plus and the minus side's.  code[r] < 2: row r has set code[r]
+// (cst[3 c ..] = weight, diagonal, inverse diagonal; weights to a node outside the
+// grid do not count), decided by comparing the stored values, so that a coded row
+// computes with the very numbers it does not load; 2: load them.  The HBM-bound FP32
+// iteration then moves 43 bytes per unknown instead of 64.
+struct Coded {
+  const uint8_t* code;
+  const float* cst;
+};
+
 // y = A v on the interior nodes: the Jacobi-scaled operator (UNIT: unit
 // diagonal, `diag` unused) or the unscaled one; v . y summed into sc[1]
 // (post = POST_ALPHA)
@@ -245,14 +326,16 @@ __global__ void __launch_bounds__(kB) k_reduce_parts(const double* part, int npa
 // (i, j) column through the slab, keeping the z neighbours in registers, so
 // node indices need no integer division and each thread reduces once.
 // (FP32: 8 blocks, i.e. 2048 threads, per SM; at most 32 registers)
-template <typename T, bool UNIT>
+// CODED (the FP32 operator of constant-mu problems): see Coded below.
+template <typename T, bool UNIT, bool CODED = false>
 __global__ void __launch_bounds__(kB, sizeof(T) == 4 ? 8 : 6) k_spmv_dot(Grid G, int kz,
                                                  const T* diag,
                                                  const T* wx,
                                                  const T* wy,
                                                  const T* wz,
                                                  const T* v, T* y,
-                                                 double* part, double* sc, int post, int* ticket) {
+                                                 double* part, double* sc, int post, int* ticket,
+                                                 Coded cd) {
   pdl_enter();
   const int i = blockIdx.x * blockDim.x + threadIdx.x, j = blockIdx.y * blockDim.y + threadIdx.y;
   const int k0 = blockIdx.z * kz, k1 = min(k0 + kz, G.m1);
@@ -260,10 +343,36 @@ __global__ void __launch_bounds__(kB, sizeof(T) == 4 ? 8 : 6) k_spmv_dot(Grid G,
   T d[1] = {T(0)};
   if (i < G.m1 && j < G.m1) {
     int64_t r = i + s1 * j + s2 * k0;
-    T vm = k0 > 0 ? v[r - s2] : T(0), wzm = k0 > 0 ? wz[r - s2] : T(0);
+    T vm = k0 > 0 ? v[r - s2] : T(0), wzm = !CODED && k0 > 0 ? wz[r - s2] : T(0);
     T vc = v[r];
+    T cw[2] = {T(0), T(0)}, cg[2] = {T(0), T(0)};
+    if constexpr (CODED) {
+      cw[0] = cd.cst[0];
+      cg[0] = cd.cst[1];
+      cw[1] = cd.cst[3];
+      cg[1] = cd.cst[4];
+    }
     for (int k = k0; k < k1; ++k, r += s2) {
       const T vp = k + 1 < G.m1 ? v[r + s2] : T(0);
+      if constexpr (CODED) {
+        const int c = cd.code[r];
+        if (c < 2) {  // the general row below with its constants (a missing neighbour's v is 0)
+          const T w = c ? cw[1] : cw[0];
+          T acc = (c ? cg[1] : cg[0]) * vc;
+          if (i + 1 < G.m1) acc -= w * v[r + 1];
+          if (i > 0) acc -= w * v[r - 1];
+          if (j + 1 < G.m1) acc -= w * v[r + s1];
+          if (j > 0) acc -= w * v[r - s1];
+          acc -= w * vp;
+          acc -= w * vm;
+          y[r] = acc;
+          d[0] += vc * acc;
+          vm = vc;
+          vc = vp;
+          continue;
+        }
+        wzm = k > 0 ? wz[r - s2] : T(0);
+      }
       const T wzc = wz[r];  // zero on the last interior plane
       T acc = UNIT ? vc : diag[r] * vc;
       if (i + 1 < G.m1) acc -= wx[r] * v[r + 1];
@@ -285,42 +394,51 @@ __global__ void __launch_bounds__(kB, sizeof(T) == 4 ? 8 : 6) k_spmv_dot(Grid G,
   fold_partials(part, nparts, 1, sc, 1, post, ticket);
 }
 
-// x += alpha p; r -= alpha Ap; partials of the recurrence's r.z and of the
-// stopping norm ||r||^2 of the unscaled system.  UNIT (scaled system, dv = D):
-// r.z = r^.r^ and ||r||^2 = sum d r^2.  Otherwise (Jacobi PCG, dv = 1/D):
-// r.z = sum r^2 / d and ||r||^2 = r.r.  The scalars stay FP64 and each thread
-// strides over the nodes, reducing once.
-template <typename T, bool UNIT>
-__global__ void __launch_bounds__(kB) k_update(Grid G, double* sc, const T* dv,
-                                               const T* p,
-                                               const T* Ap, T* x, T* r,
+// r -= alpha Ap; partials of the recurrence's r.z and, with NORM, of the
+// stopping norm ||r||^2 of the unscaled system (the host looks at it every
+// kCheckEvery iterations only).  UNIT (scaled system, dv = D): r.z = r^.r^ and
+// ||r||^2 = sum d r^2.  Otherwise (Jacobi PCG, dv = 1/D): r.z = sum r^2 / d and
+// ||r||^2 = r.r.  The scalars stay FP64 and each thread strides over the nodes,
+// reducing once.
+template <typename T, bool UNIT, bool NORM>
+__global__ void __launch_bounds__(kB) k_update(Grid G, double* sc, const T* dv, const T* Ap, T* r,
                                                double* part, int* ticket) {
   pdl_enter();
-  T acc[2] = {T(0), T(0)};
+  constexpr int NV = NORM ? 2 : 1;
+  T acc[NV];
+#pragma unroll
+  for (int q = 0; q < NV; ++q) acc[q] = T(0);
   const T a = (T)sc[2];
+#pragma unroll 2
   for (int64_t i = (int64_t)blockIdx.x * kB + threadIdx.x; i < G.m; i += (int64_t)gridDim.x * kB) {
-    x[i] += a * p[i];
     const T ri = r[i] - a * Ap[i];
     r[i] = ri;
     const T rr = ri * ri;
     acc[0] += UNIT ? rr : rr * dv[i];
-    acc[1] += UNIT ? dv[i] * rr : rr;
+    if constexpr (NORM) acc[1] += UNIT ? dv[i] * rr : rr;
   }
-  block_partials<T, 2>(acc, part, blockIdx.x, gridDim.x);
-  fold_partials(part, gridDim.x, 2, sc, 3, POST_BETA, ticket);
+  block_partials<T, NV>(acc, part, blockIdx.x, gridDim.x);
+  fold_partials(part, gridDim.x, NV, sc, 3, POST_BETA, ticket);
 }
 
-// p = z + beta p with z = r (UNIT) or r / D (`inv_diag`; Jacobi PCG)
-// (beta = 0: p = z for the first direction)
+// x += alpha p, then p = z + beta p with z = r (UNIT) or r / D (`inv_diag`; Jacobi
+// PCG).  `first`: p = z only (the first direction).  The iterate moves here, where p
+// is read anyway, instead of with the residual: 16 bytes per FP64 unknown less.
 template <typename T, bool UNIT>
 __global__ void __launch_bounds__(kB) k_pupdate(Grid G, const double* sc, int first,
-                                                const T* inv_diag,
-                                                const T* r, T* p) {
+                                                const T* inv_diag, const T* r, T* x, T* p) {
   pdl_enter();
-  const T beta = first ? T(0) : (T)sc[5];
+  const T al = (T)sc[2], beta = (T)sc[5];
+#pragma unroll 2
   for (int64_t i = (int64_t)blockIdx.x * kB + threadIdx.x; i < G.m; i += (int64_t)gridDim.x * kB) {
     const T z = UNIT ? r[i] : r[i] * inv_diag[i];
-    p[i] = first ? z : z + beta * p[i];
+    if (first) {
+      p[i] = z;
+    } else {
+      const T pi = p[i];
+      x[i] += al * pi;
+      p[i] = z + beta * pi;
+    }
   }
 }
 
@@ -364,6 +482,106 @@ __global__ void __launch_bounds__(kB) k_defect(Grid G, const double* d,
   fold_partials(part, gridDim.x, 2, sc, 8, POST_NORM, ticket);
 }
 
+// The two sets of constants from a corner node's row and the middle node's.
+__global__ void k_code_ref(Grid G, const float* d32, const float* idg32, const float* wx32,
+                           float* cst) {
+  pdl_enter();
+  const int64_t c = G.m1 / 2, mid = c + G.m1 * (c + G.m1 * c);
+  cst[0] = wx32[0];
+  cst[1] = d32[0];
+  cst[2] = idg32[0];
+  cst[3] = wx32[mid];
+  cst[4] = d32[mid];
+  cst[5] = idg32[mid];
+}
+
+__global__ void __launch_bounds__(kB) k_code_rows(Grid G, const float* d32, const float* idg32,
+                                                  const float* wx32, const float* wy32,
+                                                  const float* wz32, const float* cst,
+                                                  uint8_t* code) {
+  pdl_enter();
+  const int64_t s1 = G.m1, s2 = (int64_t)G.m1 * G.m1;
+  for (int64_t r = (int64_t)blockIdx.x * kB + threadIdx.x; r < G.m; r += (int64_t)gridDim.x * kB) {
+    const int i = (int)(r % G.m1), j = (int)((r / G.m1) % G.m1), k = (int)(r / s2);
+    int c = 2;
+#pragma unroll
+    for (int t = 0; t < 2; ++t) {
+      const float w = cst[3 * t];
+      if (d32[r] == cst[3 * t + 1] && idg32[r] == cst[3 * t + 2] &&
+          (i + 1 == G.m1 || wx32[r] == w) && (i == 0 || wx32[r - 1] == w) &&
+          (j + 1 == G.m1 || wy32[r] == w) && (j == 0 || wy32[r - s1] == w) &&
+          (k + 1 == G.m1 || wz32[r] == w) && (k == 0 || wz32[r - s2] == w))
+        c = t;
+    }
+    code[r] = (uint8_t)c;
+  }
+}
+
+// Inverse diagonals of the four unknowns from 4 i4 (coded rows).
+__device__ inline float4 inv_diag4(const Coded& cd, const float* idg32, int64_t i4) {
+  const uchar4 c = reinterpret_cast<const uchar4*>(cd.code)[i4];
+  const float a = cd.cst[2], b = cd.cst[5];
+  if ((c.x | c.y | c.z | c.w) < 2)
+    return make_float4(c.x ? b : a, c.y ? b : a, c.z ? b : a, c.w ? b : a);
+  return reinterpret_cast<const float4*>(idg32)[i4];
+}
+
+// k_update<float, false, true> and k_pupdate<float, false> on coded rows, four
+// unknowns per thread and 16-byte access (the last m % 4 by the grid's first thread).
+__global__ void __launch_bounds__(kB) k_update4(Grid G, double* sc, const float* idg32,
+                                                const float* Ap, float* r, double* part,
+                                                Coded cd) {
+  pdl_enter();
+  float acc[2] = {0.f, 0.f};
+  const float a = (float)sc[2];
+  const int64_t m4 = G.m / 4;
+  auto one = [&](float rv, float av, float id) {
+    const float ri = rv - a * av, rr = ri * ri;
+    acc[0] += rr * id;
+    acc[1] += rr;
+    return ri;
+  };
+#pragma unroll 2
+  for (int64_t i = (int64_t)blockIdx.x * kB + threadIdx.x; i < m4; i += (int64_t)gridDim.x * kB) {
+    const float4 av = reinterpret_cast<const float4*>(Ap)[i];
+    const float4 id = inv_diag4(cd, idg32, i);
+    float4 rv = reinterpret_cast<float4*>(r)[i];
+    rv.x = one(rv.x, av.x, id.x);
+    rv.y = one(rv.y, av.y, id.y);
+    rv.z = one(rv.z, av.z, id.z);
+    rv.w = one(rv.w, av.w, id.w);
+    reinterpret_cast<float4*>(r)[i] = rv;
+  }
+  if (blockIdx.x == 0 && threadIdx.x == 0)
+    for (int64_t i = 4 * m4; i < G.m; ++i) r[i] = one(r[i], Ap[i], idg32[i]);
+  block_partials<float, 2>(acc, part, blockIdx.x, gridDim.x);
+}
+
+__global__ void __launch_bounds__(kB) k_pupdate4(Grid G, const double* sc, const float* idg32,
+                                                 const float* r, float* x, float* p, Coded cd) {
+  pdl_enter();
+  const float al = (float)sc[2], beta = (float)sc[5];
+  const int64_t m4 = G.m / 4;
+  auto one = [&](float rv, float id, float& xv, float& pv) {
+    xv += al * pv;
+    pv = rv * id + beta * pv;
+  };
+#pragma unroll 2
+  for (int64_t i = (int64_t)blockIdx.x * kB + threadIdx.x; i < m4; i += (int64_t)gridDim.x * kB) {
+    const float4 rv = reinterpret_cast<const float4*>(r)[i];
+    const float4 id = inv_diag4(cd, idg32, i);
+    float4 xv = reinterpret_cast<float4*>(x)[i], pv = reinterpret_cast<float4*>(p)[i];
+    one(rv.x, id.x, xv.x, pv.x);
+    one(rv.y, id.y, xv.y, pv.y);
+    one(rv.z, id.z, xv.z, pv.z);
+    one(rv.w, id.w, xv.w, pv.w);
+    reinterpret_cast<float4*>(x)[i] = xv;
+    reinterpret_cast<float4*>(p)[i] = pv;
+  }
+  if (blockIdx.x == 0 && threadIdx.x == 0)
+    for (int64_t i = 4 * m4; i < G.m; ++i) one(r[i], idg32[i], x[i], p[i]);
+}
+
 // start of an inner solve (FP32 Jacobi PCG on the unscaled operator) of
 // A e = r / ||r|| with r = D^1/2 r^: e = 0, r32 = r / ||r|| (norm 1),
 // p32 = r32 / D; partials of r32.p32 and r32.r32
@@ -387,6 +605,207 @@ __global__ void __launch_bounds__(kB) k_inner_init(Grid G, double* sc,
   }
   block_partials<float, 2>(acc, part, blockIdx.x, gridDim.x);
   fold_partials(part, gridDim.x, 2, sc, 3, POST_BETA, ticket);
+}
+
+// ---- CG iterations in one launch (small grids) ----
+
+// kPersistT threads per CTA, one CTA per SM; a CTA owns a contiguous range of the
+// unknowns, kPersistN per thread at most.  (16 warps rather than 32: a warp's
+// shuffle sum is 5 FP64 additions on every lane of the narrow FP64 pipe.)
+constexpr int kPersistT = 512;
+constexpr int kPersistN = 28;
+
+// Grid-wide barrier number `seq` (1, 2, ...): every CTA adds 1 to *count (zero at
+// the launch) and waits for seq x gridDim arrivals; bounded, false when the wait
+// gave up.  All CTAs are resident (cooperative launch).
+__device__ inline bool grid_barrier(unsigned* count, unsigned seq, int* gave_up) {
+  __shared__ int ok_s;
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    __threadfence();
+    atomicAdd(count, 1u);
+    const unsigned target = seq * gridDim.x;
+    int ok = 1;
+    const long long t0 = clock64();
+    while (true) {
+      unsigned v;
+      // (relaxed: an acquire per poll would invalidate L1 each time; one fence follows)
+      asm volatile("ld.relaxed.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(count) : "memory");
+      if (v >= target) break;
+      if (clock64() - t0 > 4000000000LL) {
+        *gave_up = 1;
+        ok = 0;
+        break;
+      }
+    }
+    __threadfence();
+    ok_s = ok;
+  }
+  __syncthreads();
+  return ok_s != 0;
+}
+
+// Block sums of NV values by a fixed order into part[v * gridDim.x + blockIdx.x].
+template <typename T, int NV>
+__device__ inline void persist_partials(T (&v)[NV], double* part) {
+  __shared__ double red[NV][kPersistT / 32];
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1)
+#pragma unroll
+    for (int q = 0; q < NV; ++q) v[q] += __shfl_xor_sync(0xffffffffu, v[q], o);
+  if ((threadIdx.x & 31) == 0)
+#pragma unroll
+    for (int q = 0; q < NV; ++q) red[q][threadIdx.x >> 5] = (double)v[q];
+  __syncthreads();
+  if (threadIdx.x < kPersistT / 32) {
+    constexpr unsigned mask = (1u << (kPersistT / 32)) - 1u;
+#pragma unroll
+    for (int q = 0; q < NV; ++q) {
+      double s = red[q][threadIdx.x];
+#pragma unroll
+      for (int o = kPersistT / 64; o > 0; o >>= 1) s += __shfl_xor_sync(mask, s, o);
+      if (threadIdx.x == 0) part[q * (int64_t)gridDim.x + blockIdx.x] = s;
+    }
+  }
+}
+
+// The sum over the CTAs' partials in a fixed order: the same value in every thread
+// of every CTA.
+__device__ inline double persist_sum(const double* part) {
+  __shared__ double tot;
+  if (threadIdx.x < 32) {
+    double s = 0.0;
+    for (int b = threadIdx.x; b < (int)gridDim.x; b += 32) s += __ldcg(part + b);
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+    if (threadIdx.x == 0) tot = s;
+  }
+  __syncthreads();
+  const double v = tot;
+  __syncthreads();
+  return v;
+}
+
+// Up to `steps` CG iterations from iteration `it` (sc[0] = r.z of the residual in
+// r, p the current direction) in one cooperative launch: the SpMV, the residual and
+// the direction update of three launches, with a grid-wide barrier for each of
+// their dependences.  Each CTA keeps its range of r and p (and a row of neighbours
+// on either side) in shared memory and A p in registers; x, the weights and the
+// neighbours a plane away go through L2.  Stops at ||r|| <= stop (looked at every
+// kCheckEvery iterations and at max_iter, as the three-launch path does).  Writes r
+// back, sc[0] = r.z, sc[4] = ||r||^2 of the last look, sc[14] = iterations done, and
+// sc[15] = 1 if a barrier gave up.
+// Bound (FP64): the FP64 pipe's 11 operations per unknown (38 of 58 us per iteration
+// at 128^3), then the three barriers (4 to 8 us each: a fence, an arrival, the polls
+// and the FP64 sums, over two dies).
+template <typename T, bool UNIT>
+__global__ void __launch_bounds__(kPersistT, 1)
+    k_cg_persist(Grid G, const T* diag, const T* dv, const T* wx, const T* wy, const T* wz, T* __restrict__ x,
+                 T* r, T* p, double* part, double* sc, unsigned* count, int it, int steps,
+                 int max_iter, int check_every, double stop) {
+  pdl_enter();
+  constexpr int NT = kPersistT, NPT = kPersistN;
+  extern __shared__ __align__(16) unsigned char cg_smem[];
+  __shared__ int gave_up;
+  const int s1 = G.m1, s2 = G.m1 * G.m1, m = (int)G.m;
+  const int a = (int)((int64_t)m * blockIdx.x / gridDim.x);
+  const int b = (int)((int64_t)m * (blockIdx.x + 1) / gridDim.x), N = b - a;
+  T* ps = reinterpret_cast<T*>(cg_smem) + s1;  // p of a - s1 .. b + s1 - 1
+  T* rs = ps + N + s1;                         // r of a .. b - 1
+  const int tid = threadIdx.x;
+  if (tid == 0) gave_up = 0;
+  auto load_halo = [&](bool own) {
+    for (int i = -s1 + tid; i < N + s1; i += NT)
+      if (own || i < 0 || i >= N) ps[i] = a + i >= 0 && a + i < m ? __ldcg(p + a + i) : T(0);
+  };
+  load_halo(true);
+  for (int i = tid; i < N; i += NT) rs[i] = r[a + i];
+  __syncthreads();
+  double rz = sc[0], rr = sc[4];
+  unsigned seq = 0;
+  bool ok = true;
+  const int end = it + steps < max_iter ? it + steps : max_iter;
+#pragma unroll 1
+  while (it < end) {
+    // A p of this thread's unknowns.  Weights to a node outside the grid are stored
+    // as 0 (a row's last wx, a plane's last wy, the last plane's wz), so only the
+    // ends of the arrays need a test.
+    T Ap[NPT], d[1] = {T(0)};
+#pragma unroll
+    for (int t = 0; t < NPT; ++t) {
+      if (NT * t >= N) break;  // block-uniform: small ranges skip the rest of the code
+      const int i = tid + NT * t, q = a + i;
+      if (i < N) {
+        const T vc = ps[i];
+        T acc = UNIT ? vc : diag[q] * vc;
+        acc -= wx[q] * ps[i + 1];
+        if (q > 0) acc -= wx[q - 1] * ps[i - 1];
+        acc -= wy[q] * ps[i + s1];
+        if (q >= s1) acc -= wy[q - s1] * ps[i - s1];
+        if (q + s2 < m) acc -= wz[q] * __ldcg(p + q + s2);
+        if (q >= s2) acc -= wz[q - s2] * __ldcg(p + q - s2);
+        Ap[t] = acc;
+        d[0] += vc * acc;
+      }
+    }
+    persist_partials<T, 1>(d, part);
+    if (!(ok = grid_barrier(count, ++seq, &gave_up))) break;
+    const double alpha_d = rz / persist_sum(part);
+    const T al = (T)alpha_d;
+    ++it;
+    const bool look = it % check_every == 0 || it == max_iter;
+    // r -= alpha A p and its products (the partials alternate between two places:
+    // another CTA may still be summing the previous ones)
+    T e[1] = {T(0)};
+#pragma unroll
+    for (int t = 0; t < NPT; ++t) {
+      if (NT * t >= N) break;
+      const int i = tid + NT * t;
+      if (i < N) {
+        const T ri = rs[i] - al * Ap[t];
+        rs[i] = ri;
+        e[0] += UNIT ? ri * ri : ri * ri * dv[a + i];
+      }
+    }
+    double* part2 = part + gridDim.x;
+    persist_partials<T, 1>(e, part2);
+    // x += alpha p, on its way through L2 while the barrier completes
+#pragma unroll 8
+    for (int i = tid; i < N; i += NT) x[a + i] += al * ps[i];
+    if (look) {
+      T f[1] = {T(0)};
+      for (int i = tid; i < N; i += NT) f[0] += UNIT ? dv[a + i] * (rs[i] * rs[i]) : rs[i] * rs[i];
+      __syncthreads();
+      persist_partials<T, 1>(f, part2 + gridDim.x);
+    }
+    if (!(ok = grid_barrier(count, ++seq, &gave_up))) break;
+    const double rz_new = persist_sum(part2);
+    if (look) rr = persist_sum(part2 + gridDim.x);
+    const T beta = (T)(rz_new / rz);
+    rz = rz_new;
+    // p = z + beta p (x += alpha p went before the barrier, see above)
+#pragma unroll 4
+    for (int i = tid; i < N; i += NT) {
+      const T pi = ps[i];
+      const T pn = (UNIT ? rs[i] : rs[i] * dv[a + i]) + beta * pi;
+      ps[i] = pn;
+      __stcg(p + a + i, pn);
+    }
+    if (look) {
+      const double rn = sqrt(rr);
+      if (!(rn == rn) || rn <= stop) break;  // the same in every CTA
+    }
+    if (!(ok = grid_barrier(count, ++seq, &gave_up))) break;
+    load_halo(false);
+    __syncthreads();
+  }
+  for (int i = tid; i < N; i += NT) r[a + i] = rs[i];
+  if (blockIdx.x == 0 && tid == 0) {
+    sc[0] = rz;
+    sc[4] = rr;
+    sc[14] = (double)it;
+  }
+  if (tid == 0 && !ok) sc[15] = 1.0;
 }
 
 // ---- extrapolated node jump ----
@@ -625,7 +1044,46 @@ struct CgSetup {
   int nsp;     // SpMV partials
   int64_t nodes;
   bool fold;   // reductions folded into the producing kernels (small grids)
+  int sms;
 };
+
+// Launch of k_cg_persist for this grid: CTAs and shared memory; ctas == 0 when the
+// grid does not fit (kPersistN unknowns per thread, i.e. up to 130 cells per axis on 152
+// SMs; a CTA's range of r and p with its neighbour rows must fit the shared memory)
+// or the device cannot hold one CTA per SM.  Where it fits it is the faster path (whole
+// solves, FP64 / refined, against three launches per iteration): 24^3 2.2 / 2.4 against
+// 2.5 / 3.2 ms, 64^3 7.2 / 7.6 against 9.2 / 9.5, 128^3 34.3 / 28.2 against 46.8 / 29.3.
+// In FP32 twice the unknowns would fit, but there the coded rows of three launches
+// win: 150^3 refined 50.8 against 43.0 ms.
+struct PersistLaunch {
+  int ctas = 0;
+  size_t smem = 0;
+};
+template <typename T, bool UNIT>
+PersistLaunch persist_launch(const CgSetup& S) {
+  PersistLaunch L;
+  const int64_t want = (S.G.m + 511) / 512;  // a thread or two per unknown on small grids
+  const int ctas = (int)(want < S.sms ? want : S.sms);
+  const int64_t per = (S.G.m + ctas - 1) / ctas;
+  const size_t smem = (size_t)(2 * per + 2 * S.G.m1) * sizeof(T);
+  if (per > (int64_t)kPersistT * kPersistN || smem > 230 * 1024 ||
+      3 * (int64_t)ctas > (int64_t)kMaxVec * (S.nu > S.nsp ? S.nu : S.nsp))
+    return L;
+  int dev = 0, coop = 0, fit = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess ||
+      cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, dev) != cudaSuccess || !coop ||
+      cudaFuncSetAttribute(k_cg_persist<T, UNIT>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                           (int)smem) != cudaSuccess ||
+      cudaOccupancyMaxActiveBlocksPerMultiprocessor(&fit, k_cg_persist<T, UNIT>, kPersistT, smem) !=
+          cudaSuccess ||
+      fit < 1) {
+    (void)cudaGetLastError();  // the three-launch path serves
+    return L;
+  }
+  L.ctas = ctas;
+  L.smem = smem;
+  return L;
+}
 
 int cg_setup(nbm_problem* p, int n, double rtol, int max_iter, const double* u_out, const char* who,
              CgSetup& S) {
@@ -667,6 +1125,7 @@ int cg_setup(nbm_problem* p, int n, double rtol, int max_iter, const double* u_o
   S.nsp = (int)(S.sgrid.x * S.sgrid.y * S.sgrid.z);
   S.nodes = (int64_t)(n + 1) * (n + 1) * (n + 1);
   S.fold = G.m <= kFoldMaxUnknowns;
+  S.sms = problem_num_sms(p);
   return NBM_OK;
 }
 
@@ -723,6 +1182,7 @@ namespace {
 
 constexpr double kInnerTol = 1e-5;  // relative residual target of one FP32 inner solve
 constexpr int kCheckEvery = 10;     // inner iterations between host convergence checks
+constexpr int kPersistSteps = 1000;  // iterations of one k_cg_persist launch (50 ms or so)
 constexpr int kMaxStall = 3;        // outer steps in a row that gain less than 10 %
 constexpr int kMaxPasses = 10;      // solves with a lagged jump
 constexpr double kJumpTol = 1e-6;   // max |J_new - J| <= kJumpTol max(1, max |J|)
@@ -745,9 +1205,11 @@ struct GridSolve {
   // weights, right-hand side, iterate x^ = D^1/2 x and residual
   double *diag, *wx, *wy, *wz, *b, *x, *r, *J = nullptr, *part, *sc;
   int* ticket = nullptr;  // last-block counter of the folded reductions
+  unsigned* count = nullptr;  // arrivals at k_cg_persist's barriers
   double *pv = nullptr, *Ap = nullptr;                        // FP64 CG
   float *d32 = nullptr, *idg32 = nullptr, *wx32 = nullptr, *wy32 = nullptr, *wz32 = nullptr,
         *r32 = nullptr, *e32 = nullptr, *p32 = nullptr, *Ap32 = nullptr;  // refined
+  Coded coded = {};  // refined, three launches per iteration, constant mu
   double host_sc[16];
   double rnorm = 0.0, bnorm = 0.0;
   int iters = 0;
@@ -757,6 +1219,39 @@ struct GridSolve {
   void reduce(int nparts, int nvec, int slot, int post) {
     if (!S.fold) launch_pdl(k_reduce_parts, dim3(1),
                             dim3(kB), 0, st, part, nparts, nvec, sc, slot, post);
+  }
+
+  // Iterations from `it` in launches of k_cg_persist until ||r|| <= stop (sets it and
+  // rnorm).  0, or -1 for a CUDA error, or NBM_ERR_DEVICE_TIMEOUT.
+  template <typename T, bool UNIT>
+  int iterate(const PersistLaunch& PL, const T* dg, const T* dv, const T* ax, const T* ay,
+              const T* az, T* xv, T* rv, T* p, int& it, int max_iter, double stop, double& rn,
+              cudaError_t& e) {
+    while (it < max_iter) {
+      if ((e = cudaMemsetAsync(count, 0, sizeof(unsigned), st)) != cudaSuccess) return -1;
+      cudaLaunchConfig_t cfg = {};
+      cfg.gridDim = dim3(PL.ctas);
+      cfg.blockDim = dim3(kPersistT);
+      cfg.dynamicSmemBytes = PL.smem;
+      cfg.stream = st;
+      cudaLaunchAttribute at[1];
+      at[0].id = cudaLaunchAttributeCooperative;
+      at[0].val.cooperative = 1;
+      cfg.attrs = at;
+      cfg.numAttrs = 1;
+      e = cudaLaunchKernelEx(&cfg, k_cg_persist<T, UNIT>, S.G, dg, dv, ax, ay, az, xv, rv, p, part,
+                             sc, count, it, kPersistSteps, max_iter, kCheckEvery, stop);
+      if (e != cudaSuccess || (e = read_sc()) != cudaSuccess) return -1;
+      if (host_sc[15] != 0.0) return NBM_ERR_DEVICE_TIMEOUT;
+      const int done = (int)host_sc[14];
+      const bool looked = done % kCheckEvery == 0 || done == max_iter;
+      it = done;
+      if (looked) {
+        rn = sqrt(host_sc[4]);
+        if (!(rn == rn) || rn <= stop) break;
+      }
+    }
+    return 0;
   }
 
   cudaError_t read_sc() {
@@ -772,7 +1267,7 @@ struct GridSolve {
     cudaMemsetAsync(sc, 0, sizeof(double) * 16, st);
     launch_pdl(k_spmv_dot<double, true>, dim3(S.sgrid),
                dim3(S.sblock), 0, st, G, S.kz, nullptr, wx, wy, wz, x, r, part, sc, POST_SKIP,
-               nullptr);
+               nullptr, Coded{});
     launch_pdl(k_defect, dim3(S.nu), dim3(kB), 0, st, G, diag, b, r, part, sc, tk());
     reduce(S.nu, 2, 8, POST_NORM);
   }
@@ -783,28 +1278,35 @@ struct GridSolve {
   int solve_fp64(double rtol, int max_iter, cudaError_t& e) {
     const Grid& G = S.G;
     defect();
-    cudaMemsetAsync(pv, 0, sizeof(double) * G.m, st);
     cudaMemsetAsync(Ap, 0, sizeof(double) * G.m, st);
     // rz = r^.r^, rr = ||r||^2 (an update with alpha = sc[2] = 0), p = r^
-    launch_pdl(k_update<double, true>, dim3(S.nu), dim3(kB), 0, st, G, sc, diag, pv, Ap, x, r, part,
+    launch_pdl(k_update<double, true, true>, dim3(S.nu), dim3(kB), 0, st, G, sc, diag, Ap, r, part,
                tk());
     reduce(S.nu, 2, 3, POST_BETA);
-    launch_pdl(k_pupdate<double, true>, dim3(S.nu), dim3(kB), 0, st, G, sc, 1, nullptr, r, pv);
+    launch_pdl(k_pupdate<double, true>, dim3(S.nu), dim3(kB), 0, st, G, sc, 1, nullptr, r, x, pv);
     if ((e = read_sc()) != cudaSuccess) return -1;
     bnorm = sqrt(host_sc[9]);
     rnorm = sqrt(host_sc[4]);
     int it = 0;
     bool converged = rnorm <= rtol * bnorm;
+    const PersistLaunch PL = persist_launch<double, true>(S);
+    if (PL.ctas && !converged && it < max_iter && rnorm == rnorm) {
+      if (int rc = iterate<double, true>(PL, nullptr, diag, wx, wy, wz, x, r, pv, it, max_iter,
+                                         rtol * bnorm, rnorm, e))
+        return rc;
+      converged = rnorm <= rtol * bnorm;
+    }
     while (!converged && it < max_iter && rnorm == rnorm) {
       launch_pdl(k_spmv_dot<double, true>, dim3(S.sgrid), dim3(S.sblock), 0, st, G, S.kz, nullptr,
-                 wx, wy, wz, pv, Ap, part, sc, POST_ALPHA, tk());
+                 wx, wy, wz, pv, Ap, part, sc, POST_ALPHA, tk(), Coded{});
       reduce(S.nsp, 1, 1, POST_ALPHA);
-      launch_pdl(k_update<double, true>, dim3(S.nu), dim3(kB), 0, st, G, sc, diag, pv, Ap, x, r,
-                 part, tk());
-      reduce(S.nu, 2, 3, POST_BETA);
-      launch_pdl(k_pupdate<double, true>, dim3(S.nu), dim3(kB), 0, st, G, sc, 0, nullptr, r, pv);
       ++it;
-      if (it % kCheckEvery == 0 || it == max_iter) {
+      const bool look = it % kCheckEvery == 0 || it == max_iter;
+      launch_pdl(look ? k_update<double, true, true> : k_update<double, true, false>, dim3(S.nu),
+                 dim3(kB), 0, st, G, sc, diag, Ap, r, part, tk());
+      reduce(S.nu, look ? 2 : 1, 3, POST_BETA);
+      launch_pdl(k_pupdate<double, true>, dim3(S.nu), dim3(kB), 0, st, G, sc, 0, nullptr, r, x, pv);
+      if (look) {
         if ((e = read_sc()) != cudaSuccess) return -1;
         rnorm = sqrt(host_sc[4]);
         converged = rnorm <= rtol * bnorm;
@@ -823,6 +1325,7 @@ struct GridSolve {
     if ((e = read_sc()) != cudaSuccess) return -1;
     bnorm = sqrt(host_sc[9]);
     rnorm = sqrt(host_sc[8]);
+    const PersistLaunch PL = persist_launch<float, false>(S);
     int it = 0, stall = 0;
     bool converged = rnorm <= rtol * bnorm;
     while (!converged && it < max_iter && rnorm == rnorm && stall < kMaxStall) {
@@ -833,16 +1336,34 @@ struct GridSolve {
       launch_pdl(k_inner_init, dim3(S.nu), dim3(kB), 0, st, G, sc, r, d32, idg32, r32, e32, p32,
                  part, tk());
       reduce(S.nu, 2, 3, POST_BETA);
-      for (int inner = 1; it < max_iter; ++inner) {
-        launch_pdl(k_spmv_dot<float, false>, dim3(S.sgrid), dim3(S.sblock), 0, st, G, S.kz, d32,
-                   wx32, wy32, wz32, p32, Ap32, part, sc, POST_ALPHA, tk());
+      if (PL.ctas) {
+        // the first direction p32 = z is in place: iterations counted from this start
+        double rin = 1.0;
+        int inner = 0;
+        if (int rc = iterate<float, false>(PL, d32, idg32, wx32, wy32, wz32, e32, r32, p32, inner,
+                                           max_iter - it, tau, rin, e))
+          return rc;
+        it += inner;
+      }
+      for (int inner = 1; !PL.ctas && it < max_iter; ++inner) {
+        launch_pdl(coded.code ? k_spmv_dot<float, false, true> : k_spmv_dot<float, false>,
+                   dim3(S.sgrid), dim3(S.sblock), 0, st, G, S.kz, d32, wx32, wy32, wz32, p32, Ap32,
+                   part, sc, POST_ALPHA, tk(), coded);
         reduce(S.nsp, 1, 1, POST_ALPHA);
-        launch_pdl(k_update<float, false>, dim3(S.nu), dim3(kB), 0, st, G, sc, idg32, p32, Ap32,
-                   e32, r32, part, tk());
-        reduce(S.nu, 2, 3, POST_BETA);
-        launch_pdl(k_pupdate<float, false>, dim3(S.nu), dim3(kB), 0, st, G, sc, 0, idg32, r32, p32);
         ++it;
-        if (inner % kCheckEvery == 0 || it == max_iter) {
+        const bool look = inner % kCheckEvery == 0 || it == max_iter;
+        if (coded.code) {
+          launch_pdl(k_update4, dim3(S.nu), dim3(kB), 0, st, G, sc, idg32, Ap32, r32, part, coded);
+          launch_pdl(k_reduce_parts, dim3(1), dim3(kB), 0, st, part, S.nu, 2, sc, 3, POST_BETA);
+          launch_pdl(k_pupdate4, dim3(S.nu), dim3(kB), 0, st, G, sc, idg32, r32, e32, p32, coded);
+        } else {
+        launch_pdl(look ? k_update<float, false, true> : k_update<float, false, false>, dim3(S.nu),
+                   dim3(kB), 0, st, G, sc, idg32, Ap32, r32, part, tk());
+        reduce(S.nu, look ? 2 : 1, 3, POST_BETA);
+        launch_pdl(k_pupdate<float, false>, dim3(S.nu), dim3(kB), 0, st, G, sc, 0, idg32, r32, e32,
+                   p32);
+        }
+        if (look) {
           if ((e = read_sc()) != cudaSuccess) return -1;
           const double rin = sqrt(host_sc[4]);
           if (!(rin == rin) || rin <= tau) break;
@@ -868,7 +1389,8 @@ struct GridSolve {
 
   // the rows of the current jumps, then the scaled system
   void rows() {
-    launch_pdl(k_grid_rows, dim3(S.nb), dim3(kB), 0, st, S.P, S.G, J, diag, wx, wy, wz, b);
+    launch_pdl(f32_signs(S.P) ? k_grid_rows<true> : k_grid_rows<false>, dim3(S.nb), dim3(kB), 0, st,
+               S.P, S.G, J, diag, wx, wy, wz, b);
     launch_pdl(k_scale_rows, dim3(S.nu), dim3(kB), 0, st, S.G, diag, wx, wy, wz, b);
   }
 
@@ -899,6 +1421,8 @@ int grid_solve(nbm_problem* p, int n, double rtol, int max_iter, double* u_out, 
   W.x = B.get<double>(G.m);
   W.r = B.get<double>(G.m);
   if (mode != NBM_JUMP_EXACT) W.J = B.get<double>(G.m);
+  uint8_t* code = nullptr;
+  float* cst = nullptr;
   if (refined) {
     W.d32 = B.get<float>(G.m);
     W.idg32 = B.get<float>(G.m);
@@ -909,6 +1433,12 @@ int grid_solve(nbm_problem* p, int n, double rtol, int max_iter, double* u_out, 
     W.e32 = B.get<float>(G.m);
     W.p32 = B.get<float>(G.m);
     W.Ap32 = B.get<float>(G.m);
+    if (W.S.P.solution == NBM_SOL_BENCH && !persist_launch<float, false>(W.S).ctas) {
+      code = B.get<uint8_t>(G.m);
+      cst = B.get<float>(6);
+      W.coded.code = code;
+      W.coded.cst = cst;
+    }
   } else {
     W.pv = B.get<double>(G.m);
     W.Ap = B.get<double>(G.m);
@@ -916,6 +1446,7 @@ int grid_solve(nbm_problem* p, int n, double rtol, int max_iter, double* u_out, 
   W.part = B.get<double>(kMaxVec * (size_t)(W.S.nu > W.S.nsp ? W.S.nu : W.S.nsp));
   W.sc = B.get<double>(16);
   W.ticket = B.get<int>(1);
+  W.count = B.get<unsigned>(1);
   if (B.err != cudaSuccess) return cg_cuda_fail(W.who, B.err);
 
   cudaStream_t st = W.st;
@@ -930,6 +1461,11 @@ int grid_solve(nbm_problem* p, int n, double rtol, int max_iter, double* u_out, 
     launch_pdl(k_to_f32, dim3(W.S.nu),
                dim3(kB), 0, st, G, W.diag, W.wx, W.wy, W.wz, W.d32, W.idg32, W.wx32, W.wy32,
                W.wz32);
+  if (code) {
+    launch_pdl(k_code_ref, dim3(1), dim3(1), 0, st, G, W.d32, W.idg32, W.wx32, cst);
+    launch_pdl(k_code_rows, dim3(W.S.nu), dim3(kB), 0, st, G, W.d32, W.idg32, W.wx32, W.wy32,
+               W.wz32, cst, code);
+  }
   cudaError_t e = cudaSuccess;
   int status = W.solve(rtol, max_iter, e);
   JumpInfo info;
@@ -958,6 +1494,10 @@ int grid_solve(nbm_problem* p, int n, double rtol, int max_iter, double* u_out, 
     }
   }
   if (status < 0) return cg_cuda_fail(W.who, e);
+  if (status == NBM_ERR_DEVICE_TIMEOUT) {
+    set_error_message("grid solve: a bounded device wait gave up");
+    return status;
+  }
   launch_pdl(k_write_nodes, dim3((int)((W.S.nodes + kB - 1) / kB)),
              dim3(kB), 0, st, W.S.P, G, W.x, W.diag, u_out);
   e = cudaGetLastError();

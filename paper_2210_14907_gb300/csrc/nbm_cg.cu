@@ -97,50 +97,13 @@ __device__ inline bool one_sided(const ProbDev& P, const double p[3], double h, 
 // Rows of every interior node.  Jn (interior-node array) holds the node jump
 // J = u+ - u- carried to each node; NULL takes the manufactured pair's own
 // u+(x) - u-(x) (the exact jump).
-// FAST: a node whose cell and neighbours are on one side (FP32 decides) takes
-// its row without cell geometry and node jumps: every term left out is a product
-// with an exact 0, and the rest is summed in the same order, so the rows are the
-// same to the last bit.  The FP64 pipe bounds the full row (15 level-set values
-// and 7 exact jumps per node): 256^3 took 35 ms, and only the few per cent of
-// nodes about the interface still pay for it.
-template <bool FAST>
-__global__ void __launch_bounds__(kB) k_grid_rows(ProbDev P, Grid G, const double* Jn,
-                                                  double* diag, double* wx, double* wy, double* wz,
-                                                  double* rhs) {
-  pdl_enter();
-  const int64_t r = (int64_t)blockIdx.x * kB + threadIdx.x;
-  if (r >= G.m) return;
+__device__ __forceinline__ void grid_row(const ProbDev& P, const Grid& G, const double* Jn,
+                                         int64_t r, double* diag, double* wx, double* wy,
+                                         double* wz, double* rhs) {
   int idx[3];
   double p[3];
   node_xyz(G, r, idx[0], idx[1], idx[2], p);
   const double h = G.h;
-  if constexpr (FAST) {
-    int s;
-    if (one_sided(P, p, h, s)) {
-      double dg = h * h * P.k[s];
-      double known = h * h * (0.0 - rhs_f<double>(P, s, p[0], p[1], p[2]));
-      double wplus[3] = {0.0, 0.0, 0.0};
-      for (int f = 0; f < 6; ++f) {
-        const int ax = f >> 1, sg = (f & 1) ? 1 : -1;
-        int nb[3] = {idx[0], idx[1], idx[2]};
-        nb[ax] += sg;
-        double fc[3] = {p[0], p[1], p[2]};
-        fc[ax] += 0.5 * sg * h;
-        const double wf = mu_at<double>(P, s, fc[0], fc[1], fc[2]);
-        dg += wf;
-        if (nb[ax] == 0 || nb[ax] == G.n)
-          known -= wf * dirichlet_g<double>(P, node_coord(nb[0], h), node_coord(nb[1], h),
-                                            node_coord(nb[2], h));
-        else if (sg > 0) wplus[ax] = wf;
-      }
-      diag[r] = dg;
-      wx[r] = wplus[0];
-      wy[r] = wplus[1];
-      wz[r] = wplus[2];
-      rhs[r] = -known;
-      return;
-    }
-  }
   CellGeo cg;
   cell_geometry_d(P, p, h, cg);
   const int sp = phase_d(P, p);
@@ -180,6 +143,70 @@ __global__ void __launch_bounds__(kB) k_grid_rows(ProbDev P, Grid G, const doubl
     else if (sg > 0) wplus[ax] = wf;
   }
   if (cg.cut && cg.has_jump) known += h * cg.S * beta_d(P, cg.xg);
+  diag[r] = dg;
+  wx[r] = wplus[0];
+  wy[r] = wplus[1];
+  wz[r] = wplus[2];
+  rhs[r] = -known;
+}
+
+// Every row in full, or (list != nullptr) those of the listed nodes.
+__global__ void __launch_bounds__(kB) k_grid_rows(ProbDev P, Grid G, const double* Jn,
+                                                  double* diag, double* wx, double* wy, double* wz,
+                                                  double* rhs, const int64_t* list,
+                                                  const unsigned long long* count) {
+  pdl_enter();
+  const int64_t m = list ? (int64_t)*count : G.m;
+  for (int64_t e = (int64_t)blockIdx.x * kB + threadIdx.x; e < m; e += (int64_t)gridDim.x * kB)
+    grid_row(P, G, Jn, list ? list[e] : e, diag, wx, wy, wz, rhs);
+}
+
+// The rows of the nodes whose cell and neighbours are on one side (FP32 decides),
+// without cell geometry and node jumps: every term left out is a product with an
+// exact 0, and the rest is summed in the same order, so the rows are the same to
+// the last bit.  The other nodes' numbers go to the list, for k_grid_rows.  The
+// FP64 pipe bounds the full row (15 level-set values and 7 exact jumps per node):
+// in full, 256^3 took 35 ms; with the nodes about the interface in the same kernel
+// (a full row in one lane holds up its warp) 11.7 ms; listed 2.7 ms.
+__global__ void __launch_bounds__(kB) k_grid_rows_clear(ProbDev P, Grid G, double* diag, double* wx,
+                                                        double* wy, double* wz, double* rhs,
+                                                        int64_t* list, unsigned long long* count) {
+  pdl_enter();
+  const int64_t r = (int64_t)blockIdx.x * kB + threadIdx.x;
+  const double h = G.h;
+  int idx[3], s = 0;
+  double p[3];
+  bool clear = true;
+  if (r < G.m) {
+    node_xyz(G, r, idx[0], idx[1], idx[2], p);
+    clear = one_sided(P, p, h, s);
+  }
+  const unsigned open = __ballot_sync(0xffffffffu, !clear);
+  if (open) {
+    const int lane = threadIdx.x & 31;
+    unsigned long long at = 0;
+    if (lane == 0) at = atomicAdd(count, (unsigned long long)__popc(open));
+    at = __shfl_sync(0xffffffffu, at, 0);
+    if (!clear) list[at + __popc(open & ((1u << lane) - 1u))] = r;
+  }
+  if (r >= G.m || !clear) return;
+  double dg = h * h * P.k[s];
+  double known = h * h * (0.0 - rhs_f<double>(P, s, p[0], p[1], p[2]));
+  double wplus[3] = {0.0, 0.0, 0.0};
+#pragma unroll
+  for (int f = 0; f < 6; ++f) {
+    const int ax = f >> 1, sg = (f & 1) ? 1 : -1;
+    int nb[3] = {idx[0], idx[1], idx[2]};
+    nb[ax] += sg;
+    double fc[3] = {p[0], p[1], p[2]};
+    fc[ax] += 0.5 * sg * h;
+    const double wf = mu_at<double>(P, s, fc[0], fc[1], fc[2]);
+    dg += wf;
+    if (nb[ax] == 0 || nb[ax] == G.n)
+      known -= wf * dirichlet_g<double>(P, node_coord(nb[0], h), node_coord(nb[1], h),
+                                        node_coord(nb[2], h));
+    else if (sg > 0) wplus[ax] = wf;
+  }
   diag[r] = dg;
   wx[r] = wplus[0];
   wy[r] = wplus[1];
@@ -328,7 +355,7 @@ struct Coded {
 // (FP32: 8 blocks, i.e. 2048 threads, per SM; at most 32 registers)
 // CODED (the FP32 operator of constant-mu problems): see Coded below.
 template <typename T, bool UNIT, bool CODED = false>
-__global__ void __launch_bounds__(kB, sizeof(T) == 4 ? 8 : 6) k_spmv_dot(Grid G, int kz,
+__global__ void __launch_bounds__(kB, sizeof(T) == 4 && !CODED ? 8 : 6) k_spmv_dot(Grid G, int kz,
                                                  const T* diag,
                                                  const T* wx,
                                                  const T* wy,
@@ -352,17 +379,24 @@ __global__ void __launch_bounds__(kB, sizeof(T) == 4 ? 8 : 6) k_spmv_dot(Grid G,
       cw[1] = cd.cst[3];
       cg[1] = cd.cst[4];
     }
+    // (CODED: the plane above and its code are requested a plane ahead)
+    T vnext = CODED && k0 + 1 < G.m1 ? v[r + s2] : T(0);
+    int cnext = CODED ? cd.code[r] : 2;
     for (int k = k0; k < k1; ++k, r += s2) {
-      const T vp = k + 1 < G.m1 ? v[r + s2] : T(0);
+      const T vp = CODED ? vnext : k + 1 < G.m1 ? v[r + s2] : T(0);
       if constexpr (CODED) {
-        const int c = cd.code[r];
+        const T ve = i + 1 < G.m1 ? v[r + 1] : T(0), vw = i > 0 ? v[r - 1] : T(0);
+        const T vn = j + 1 < G.m1 ? v[r + s1] : T(0), vs = j > 0 ? v[r - s1] : T(0);
+        const int c = cnext;
+        vnext = k + 2 < G.m1 ? v[r + 2 * s2] : T(0);
+        if (k + 1 < k1) cnext = cd.code[r + s2];
         if (c < 2) {  // the general row below with its constants (a missing neighbour's v is 0)
           const T w = c ? cw[1] : cw[0];
           T acc = (c ? cg[1] : cg[0]) * vc;
-          if (i + 1 < G.m1) acc -= w * v[r + 1];
-          if (i > 0) acc -= w * v[r - 1];
-          if (j + 1 < G.m1) acc -= w * v[r + s1];
-          if (j > 0) acc -= w * v[r - s1];
+          acc -= w * ve;
+          acc -= w * vw;
+          acc -= w * vn;
+          acc -= w * vs;
           acc -= w * vp;
           acc -= w * vm;
           y[r] = acc;
@@ -1110,11 +1144,11 @@ int cg_setup(nbm_problem* p, int n, double rtol, int max_iter, const double* u_o
   S.nb = (int)((G.m + kB - 1) / kB);
   const int resident = 8 * problem_num_sms(p);  // 2048 threads per SM
   S.nu = S.nb < resident ? S.nb : resident;
-  // SpMV blocks: a power-of-two run of a row (32 ... kB nodes) times kB / run
-  // rows; slabs of kz planes, kz chosen to keep about two threads per
-  // resident thread slot (2048 per SM), between 2 and 16 planes
-  int run = 32;  // a power of two, so that run x (kB / run) is exactly kB threads
-  while (run < G.m1 && run < kB) run *= 2;
+  // SpMV blocks: runs of 64 (small grids: 32) nodes of 4 (8) neighbouring rows, so
+  // that most of a node's row neighbours are in its block's L1 (a block of one
+  // 256-node row read them from L2); slabs of kz planes, kz chosen to keep about two
+  // threads per resident thread slot (2048 per SM), between 2 and 16 planes
+  const int run = G.m1 > 48 ? 64 : 32;
   S.sblock = dim3((unsigned)run, (unsigned)(kB / run), 1);
   const int gx = (G.m1 + run - 1) / run, gy = (G.m1 + (int)S.sblock.y - 1) / (int)S.sblock.y;
   const int64_t threads_per_plane = (int64_t)gx * run * gy * S.sblock.y;
@@ -1131,7 +1165,7 @@ int cg_setup(nbm_problem* p, int n, double rtol, int max_iter, const double* u_o
 
 // device buffers of one solve, freed together
 struct CgBuffers {
-  void* ptr[24] = {};
+  void* ptr[28] = {};
   int n = 0;
   cudaError_t err = cudaSuccess;
   template <typename T>
@@ -1206,6 +1240,7 @@ struct GridSolve {
   double *diag, *wx, *wy, *wz, *b, *x, *r, *J = nullptr, *part, *sc;
   int* ticket = nullptr;  // last-block counter of the folded reductions
   unsigned* count = nullptr;  // arrivals at k_cg_persist's barriers
+  unsigned long long* list_n = nullptr;  // nodes on the rows' list
   double *pv = nullptr, *Ap = nullptr;                        // FP64 CG
   float *d32 = nullptr, *idg32 = nullptr, *wx32 = nullptr, *wy32 = nullptr, *wz32 = nullptr,
         *r32 = nullptr, *e32 = nullptr, *p32 = nullptr, *Ap32 = nullptr;  // refined
@@ -1389,8 +1424,18 @@ struct GridSolve {
 
   // the rows of the current jumps, then the scaled system
   void rows() {
-    launch_pdl(f32_signs(S.P) ? k_grid_rows<true> : k_grid_rows<false>, dim3(S.nb), dim3(kB), 0, st,
-               S.P, S.G, J, diag, wx, wy, wz, b);
+    if (f32_signs(S.P)) {
+      // r is free between solves: it holds the list
+      int64_t* list = reinterpret_cast<int64_t*>(r);
+      cudaMemsetAsync(list_n, 0, sizeof(unsigned long long), st);
+      launch_pdl(k_grid_rows_clear, dim3(S.nb), dim3(kB), 0, st, S.P, S.G, diag, wx, wy, wz, b, list,
+                 list_n);
+      launch_pdl(k_grid_rows, dim3(S.nu), dim3(kB), 0, st, S.P, S.G, J, diag, wx, wy, wz, b, list,
+                 list_n);
+    } else {
+      launch_pdl(k_grid_rows, dim3(S.nb), dim3(kB), 0, st, S.P, S.G, J, diag, wx, wy, wz, b,
+                 nullptr, nullptr);
+    }
     launch_pdl(k_scale_rows, dim3(S.nu), dim3(kB), 0, st, S.G, diag, wx, wy, wz, b);
   }
 
@@ -1447,6 +1492,7 @@ int grid_solve(nbm_problem* p, int n, double rtol, int max_iter, double* u_out, 
   W.sc = B.get<double>(16);
   W.ticket = B.get<int>(1);
   W.count = B.get<unsigned>(1);
+  W.list_n = B.get<unsigned long long>(1);
   if (B.err != cudaSuccess) return cg_cuda_fail(W.who, B.err);
 
   cudaStream_t st = W.st;

@@ -190,6 +190,8 @@ cudaError_t launch_prep_weights(const ProbDev& P, const float* params, int prec,
                                 cudaStream_t st);
 cudaError_t launch_step_fp32(const ProbDev& P, const StepArgs& a, int grid, cudaStream_t st);
 cudaError_t launch_step_small(const ProbDev& P, const StepArgs& a, int grid, cudaStream_t st);
+// MODE_RESIDUAL and MODE_CUT_FWD of the tensor-core path (launch_step_tc calls it)
+cudaError_t launch_fwd_tc(const ProbDev& P, const StepArgs& a, int grid, cudaStream_t st);
 cudaError_t launch_step_tc(const ProbDev& P, const StepArgs& a, int grid, int prec, cudaStream_t st);
 cudaError_t launch_finish(const ProbDev& P, int64_t n, int grid, bool adam, bool want_grad,
                           float* params, float* m, float* v, float* grad_out, float lr, float b1,

@@ -28,12 +28,10 @@
 // Every wait is bounded.  The group barrier that ends each phase agrees on an
 // abort; an aborted CTA gives its MMAs and copies in flight a short bounded
 // wait before it frees TMEM.
-#include <cuda_bf16.h>
-#include <cuda_fp16.h>
-
 #include "nbm_device.cuh"
-#include "nbm_tc_ptx.cuh"
 #include "nbm_f32x2.cuh"
+#include "nbm_tc_layer.cuh"
+#include "nbm_tc_ptx.cuh"
 
 namespace nbm {
 
@@ -41,144 +39,8 @@ using namespace tc;
 
 namespace {
 
-constexpr int kHP = 8;        // points per half-tile (one warp group)
-constexpr int kImg = 32768;   // 128 x 128 16-bit weight image
-constexpr int kImgH = 16384;  // 128 x 64 16-bit operand image of a half-tile
 constexpr int kMisc = 2048;
 constexpr int kPrefetchT = 224;  // rank in the group of the thread that fetches tile records
-
-template <bool BF>
-struct F16T;
-template <>
-struct F16T<true> {
-  static __device__ __forceinline__ uint32_t pack(float a, float b) {
-    __nv_bfloat162 v = __floats2bfloat162_rn(a, b);
-    return *reinterpret_cast<uint32_t*>(&v);
-  }
-  static __device__ __forceinline__ float2 unpack(uint32_t u) {
-    __nv_bfloat162 v = *reinterpret_cast<__nv_bfloat162*>(&u);
-    return __bfloat1622float2(v);
-  }
-};
-template <>
-struct F16T<false> {
-  static __device__ __forceinline__ uint32_t pack(float a, float b) {
-    __half2 v = __floats2half2_rn(a, b);
-    return *reinterpret_cast<uint32_t*>(&v);
-  }
-  static __device__ __forceinline__ float2 unpack(uint32_t u) {
-    __half2 v = *reinterpret_cast<__half2*>(&u);
-    return __half22float2(v);
-  }
-};
-
-template <bool BF>
-__device__ __forceinline__ void store8o(unsigned char* img, uint32_t off, const float* o) {
-  uint4 pk;
-  pk.x = F16T<BF>::pack(o[0], o[1]);
-  pk.y = F16T<BF>::pack(o[2], o[3]);
-  pk.z = F16T<BF>::pack(o[4], o[5]);
-  pk.w = F16T<BF>::pack(o[6], o[7]);
-  *reinterpret_cast<uint4*>(img + off) = pk;
-}
-template <bool BF>
-__device__ __forceinline__ void load8o(const unsigned char* img, uint32_t off, float* o) {
-  const uint4 pk = *reinterpret_cast<const uint4*>(img + off);
-  float2 a = F16T<BF>::unpack(pk.x), b = F16T<BF>::unpack(pk.y), c = F16T<BF>::unpack(pk.z),
-         d = F16T<BF>::unpack(pk.w);
-  o[0] = a.x; o[1] = a.y; o[2] = b.x; o[3] = b.y;
-  o[4] = c.x; o[5] = c.y; o[6] = d.x; o[7] = d.y;
-}
-template <bool BF>
-__device__ __forceinline__ void store8(unsigned char* img, int row, int col0, const float* o) {
-  uint4 pk;
-  pk.x = F16T<BF>::pack(o[0], o[1]);
-  pk.y = F16T<BF>::pack(o[2], o[3]);
-  pk.z = F16T<BF>::pack(o[4], o[5]);
-  pk.w = F16T<BF>::pack(o[6], o[7]);
-  *reinterpret_cast<uint4*>(img + img_off(row, col0)) = pk;
-}
-template <bool BF>
-__device__ __forceinline__ void load8(const unsigned char* img, int row, int col0, float* o) {
-  const uint4 pk = *reinterpret_cast<const uint4*>(img + img_off(row, col0));
-  float2 a = F16T<BF>::unpack(pk.x), b = F16T<BF>::unpack(pk.y), c = F16T<BF>::unpack(pk.z),
-         d = F16T<BF>::unpack(pk.w);
-  o[0] = a.x; o[1] = a.y; o[2] = b.x; o[3] = b.y;
-  o[4] = c.x; o[5] = c.y; o[6] = d.x; o[7] = d.y;
-}
-
-// Sum of wo * x[0..31] over the 32 lanes of the warp: on return lane l holds
-// the sum of column l (recursive halving, one exchange per value; the scaling
-// is folded into the first halving so that x stays intact for the backward).
-__device__ __forceinline__ void warp_transpose_reduce32(const float (&x)[32], float wo, int lane,
-                                                        float& s) {
-  float v[16];
-#pragma unroll
-  for (int i = 0; i < 16; ++i) {
-    const bool hi = lane & 16;
-    const float keep = wo * (hi ? x[16 + i] : x[i]), send = wo * (hi ? x[i] : x[16 + i]);
-    v[i] = keep + __shfl_xor_sync(0xffffffffu, send, 16);
-  }
-#pragma unroll
-  for (int i = 0; i < 8; ++i) {
-    const bool hi = lane & 8;
-    const float keep = hi ? v[8 + i] : v[i], send = hi ? v[i] : v[8 + i];
-    v[i] = keep + __shfl_xor_sync(0xffffffffu, send, 8);
-  }
-#pragma unroll
-  for (int i = 0; i < 4; ++i) {
-    const bool hi = lane & 4;
-    const float keep = hi ? v[4 + i] : v[i], send = hi ? v[i] : v[4 + i];
-    v[i] = keep + __shfl_xor_sync(0xffffffffu, send, 4);
-  }
-#pragma unroll
-  for (int i = 0; i < 2; ++i) {
-    const bool hi = lane & 2;
-    const float keep = hi ? v[2 + i] : v[i], send = hi ? v[i] : v[2 + i];
-    v[i] = keep + __shfl_xor_sync(0xffffffffu, send, 2);
-  }
-  {
-    const bool hi = lane & 1;
-    const float keep = hi ? v[1] : v[0], send = hi ? v[0] : v[1];
-    s = keep + __shfl_xor_sync(0xffffffffu, send, 1);
-  }
-}
-
-// Two points' tanh stencil layer on packed FP32 pairs (unscaled columns, every
-// lane's symmetric increments small): the arithmetic of tanh_stencil_fwd's
-// series path, operation for operation.
-template <bool FAST>
-__device__ __forceinline__ void tanh_stencil_fwd_pair(F2 T, F2 NT, F2 S0, F2 MU, F2 DE, F2& M,
-                                                      F2& D, bool small_de = false) {
-  const bool sde = !FAST && small_de;  // the series of tanh d and 1/(1-x) (accurate path)
-  F2 TD;
-  if (sde) {
-    const F2 d2 = mul2(DE, DE);
-    TD = mul2(DE, fma2(d2, fma2(d2, f2s(2.0f / 15.0f), f2s(-1.0f / 3.0f)), f2s(1.0f)));
-  } else {
-    float dA, dB;
-    f2get(DE, dA, dB);
-    TD = f2(act_tanh<FAST>(dA), act_tanh<FAST>(dB));
-  }
-  const F2 poly = fma2(fma2(T, T, f2s(-1.0f / 3.0f)), mul2(MU, MU), fma2(NT, MU, f2s(1.0f)));
-  const F2 dm = mul2(mul2(S0, MU), poly);
-  const F2 tw = add2(T, dm);
-  const F2 ntw = mul2(tw, f2s(-1.0f));
-  const F2 sw = fma2(ntw, tw, f2s(1.0f));
-  const F2 td2 = mul2(TD, TD);
-  F2 r2;
-  if (sde) {
-    const F2 x = mul2(mul2(tw, tw), td2);  // 1/(1-x) = 1 + x (1 + x (1 + x))
-    r2 = fma2(x, fma2(x, add2(x, f2s(1.0f)), f2s(1.0f)), f2s(1.0f));
-  } else {
-    float eA, eB;
-    f2get(fma2(add2(sw, f2s(-1.0f)), td2, f2s(1.0f)), eA, eB);
-    r2 = f2(rcp<FAST>(eA), rcp<FAST>(eB));
-  }
-  const F2 k = mul2(sw, r2);
-  M = fma2(mul2(ntw, td2), k, dm);
-  D = mul2(k, TD);
-}
 
 // Two points' adjoint of one stencil axis (unscaled columns): the arithmetic of
 // tanh_stencil_bwd on packed pairs.
@@ -198,12 +60,10 @@ __device__ __forceinline__ F2 tanh_stencil_bwd_pair(F2 T, F2 S0, F2 MO, F2 DO, F
 size_t tc_smem_bytes(int L) { return (size_t)(2 * L - 1) * kImg + 1024 + kMisc; }
 int tc_supported(int H, int L) { return H == 128 && L >= 2 && L <= 4; }
 
-// Column convention.  SCALED: the difference columns hold mt = mu/h^2 and
-// dt = del/h (keeps FP16 operands out of the subnormal range).  Unscaled (BF16,
-// whose exponent range is that of FP32): they hold mu and del themselves,
-// which saves the rescaling in every epilogue; the output stage converts to
-// the scaled convention of the residual rows.
-template <int L, bool BF, bool FAST, bool SCALED>
+// Column convention: the difference columns hold mu and del themselves (BF16 has
+// the exponent range of FP32); the output stage converts to the scaled convention
+// of the residual rows (mu/h^2, del/h).
+template <int L, bool FAST>
 __global__ void __launch_bounds__(512, 1) k_step_tc(ProbDev P, StepArgs a) {
   pdl_enter();
   constexpr int H = 128;
@@ -242,12 +102,9 @@ __global__ void __launch_bounds__(512, 1) k_step_tc(ProbDev P, StepArgs a) {
   const uint32_t row_off = (uint32_t)((u >> 3) * 1024 + (u & 7) * 128);
   const uint32_t pbase = (uint32_t)(cgl << 2), uxor = (uint32_t)(u & 7);
   auto poff = [&](int j) -> uint32_t { return row_off + ((((pbase + j) ^ uxor) & 7u) << 4); };
-  const bool train = a.mode == MODE_TRAIN;
-  const float hs = SCALED ? P.hf : 1.f, h2s = SCALED ? P.h2f : 1.f;
-  const float ihs = SCALED ? P.inv_hf : 1.f, ih2s = SCALED ? P.inv_h2f : 1.f;
-  const uint32_t id_fwd = idesc_f16_n(BF, false, true, kHP * 8);
-  const uint32_t id_dgr = idesc_f16_n(BF, true, true, kHP * 8);
-  const uint32_t id_wgr = idesc_f16_n(BF, false, false, 128);
+  const uint32_t id_fwd = idesc_f16_n(true, false, true, kHP * 8);
+  const uint32_t id_dgr = idesc_f16_n(true, true, true, kHP * 8);
+  const uint32_t id_wgr = idesc_f16_n(true, false, false, 128);
 
   if (tid == 0) {
     mbar_init(smem_u32(bar_w), 1);
@@ -268,19 +125,16 @@ __global__ void __launch_bounds__(512, 1) k_step_tc(ProbDev P, StepArgs a) {
   uint32_t ph_w = 0, ph_mma = 0, ph_p = 0;
   bool aborted = false;
 
-  // half-tiles of 8 points: net 0 (or the cut list for net 0), then net 1
-  const int nm = a.counters[0], np = a.counters[1], nc = a.counters[2];
-  const bool cutfwd = a.mode == MODE_CUT_FWD;
-  const int T0 = cutfwd ? (nc + kHP - 1) / kHP : (nm + kHP - 1) / kHP;
-  const int T = cutfwd ? 2 * T0 : T0 + (np + kHP - 1) / kHP;
+  // half-tiles of 8 points: net 0, then net 1
+  const int nm = a.counters[0], np = a.counters[1];
+  const int T0 = (nm + kHP - 1) / kHP, T = T0 + (np + kHP - 1) / kHP;
   const int tb = (int)((int64_t)blockIdx.x * T / gridDim.x);
   const int te = (int)((int64_t)(blockIdx.x + 1) * T / gridDim.x);
 
   // tile records: one 256-byte bulk copy per half-tile, fetched a tile ahead
   auto prefetch = [&](int tau, int buf) {
     // the record lists are padded to 16 per list; net 1 starts after net 0's padding
-    const PRec* src = cutfwd ? a.rec_cut + (int64_t)kHP * (tau < T0 ? tau : tau - T0)
-                    : tau < T0 ? a.rec + (int64_t)kHP * tau
+    const PRec* src = tau < T0 ? a.rec + (int64_t)kHP * tau
                                : a.rec + 16 * (int64_t)((nm + 15) / 16) + (int64_t)kHP * (tau - T0);
     fence_proxy_async();
     mbar_expect_tx(smem_u32(bar_p), kHP * sizeof(PRec));
@@ -473,81 +327,25 @@ __global__ void __launch_bounds__(512, 1) k_step_tc(ProbDev P, StepArgs a) {
       const PRec* pr = pbuf + kHP * (kk & 1);
       // seeds of cut points (from the cut-row kernel): copied into the seed
       // buffer now (asynchronously), used after the forward
-      if (train && gtid < 8 * kHP) {
+      if (gtid < 8 * kHP) {
         const PRec& pc = pr[gtid >> 3];
         if (pc.pt >= 0 && pc.cutj >= 0)
           cp_async4(smem_u32(seeds + gtid),
                     a.cut_seed + (int64_t)(pc.cutj >> 1) * 16 + net * 8 + (gtid & 7));
       }
 
-      // ---- layer 1 (3 -> H) in FP32; exact increments mu = 0, del_i = h W1[u][i]
+      // ---- layer 1 (3 -> H) in FP32, two points per packed FP32 instruction
       {
-        const float dl1[3] = {SCALED ? w1[0] : w1[0] * P.hf, SCALED ? w1[1] : w1[1] * P.hf,
-                              SCALED ? w1[2] : w1[2] * P.hf};
-        if constexpr (!SCALED) {
-          // two points per packed FP32 instruction; tanh(h W1[u][i]) depends on the
-          // unit only
-          float Td[3];
-          // accurate path with small increments h W1[u][i] in every lane: the series
-          bool sd1 = false;
-          if constexpr (!FAST)
-            sd1 = __all_sync(0xffffffffu, fmaxf(fabsf(dl1[0]), fmaxf(fabsf(dl1[1]), fabsf(dl1[2]))) <=
-                                              kSmallDelAccurate);
+        float Td[3];
+        bool sd1;
+        layer1_increments<FAST>(w1, P.hf, Td, sd1);
 #pragma unroll
-          for (int i = 0; i < 3; ++i) Td[i] = sd1 ? tanh_small(dl1[i]) : act_tanh<FAST>(dl1[i]);
-#pragma unroll
-          for (int pp = 0; pp < kPPT; pp += 2) {
-            const PRec pa = pr[4 * cgl + pp], pb = pr[4 * cgl + pp + 1];
-            const F2 W0 = f2s(w1[0]), W1 = f2s(w1[1]), W2 = f2s(w1[2]), B1 = f2s(b1);
-            float zA, zB;
-            f2get(fma2(W0, f2(pa.x, pb.x), fma2(W1, f2(pa.y, pb.y), fma2(W2, f2(pa.z, pb.z), B1))),
-                  zA, zB);
-            const F2 T = f2(act_tanh<FAST>(zA), act_tanh<FAST>(zB));
-            const F2 NT = mul2(T, f2s(-1.0f));
-            const F2 SW = fma2(NT, T, f2s(1.0f));
-            const F2 NTT = mul2(NT, T);
-            const F2 NTS = mul2(NT, SW);
-            float oA[8], oB[8];
-            f2get(T, oA[0], oB[0]);
-#pragma unroll
-            for (int i = 0; i < 3; ++i) {
-              const F2 TD = f2s(Td[i]), TD2 = mul2(TD, TD);
-              F2 R2;
-              if (sd1) {  // 1 / (1 - t^2 Td^2) by its series
-                const F2 x = mul2(mul2(T, T), TD2);
-                R2 = fma2(x, fma2(x, add2(x, f2s(1.0f)), f2s(1.0f)), f2s(1.0f));
-              } else {
-                float eA, eB;
-                f2get(fma2(NTT, TD2, f2s(1.0f)), eA, eB);
-                R2 = f2(rcp<FAST>(eA), rcp<FAST>(eB));
-              }
-              f2get(mul2(mul2(NTS, TD2), R2), oA[1 + i], oB[1 + i]);
-              f2get(mul2(mul2(SW, TD), R2), oA[4 + i], oB[4 + i]);
-            }
-            const bool ja = pa.cutj >= 0 && (pa.cutj & 1), jb = pb.cutj >= 0 && (pb.cutj & 1);
-            oA[7] = ja ? act_tanh<FAST>(fmaf(w1[0], pa.gx, fmaf(w1[1], pa.gy, fmaf(w1[2], pa.gz, b1))))
-                       : 0.f;
-            oB[7] = jb ? act_tanh<FAST>(fmaf(w1[0], pb.gx, fmaf(w1[1], pb.gy, fmaf(w1[2], pb.gz, b1))))
-                       : 0.f;
-            store8o<BF>(Aimg, poff(pp), oA);
-            store8o<BF>(Aimg, poff(pp + 1), oB);
-          }
-        } else {
-#pragma unroll
-        for (int pp = 0; pp < kPPT; ++pp) {
-          const int p = 4 * cgl + pp;
-          const PRec pi = pr[p];
-          const float z = fmaf(w1[0], pi.x, fmaf(w1[1], pi.y, fmaf(w1[2], pi.z, b1)));
-          const float t = act_tanh<FAST>(z);
-          float o[8];
-          o[0] = t;
-#pragma unroll
-          for (int i = 0; i < 3; ++i) tanh_stencil_fwd0<FAST>(t, dl1[i], hs, ihs, ih2s, o[1 + i], o[4 + i]);
-          const bool jump = pi.cutj >= 0 && (pi.cutj & 1);
-          o[7] = jump ? act_tanh<FAST>(fmaf(w1[0], pi.gx, fmaf(w1[1], pi.gy, fmaf(w1[2], pi.gz, b1))))
-                      : 0.f;
-          store8o<BF>(Aimg, poff(pp), o);
-        }
+        for (int pp = 0; pp < kPPT; pp += 2) {
+          const PRec pa = pr[4 * cgl + pp], pb = pr[4 * cgl + pp + 1];
+          float oA[8], oB[8];
+          layer1_pair<FAST>(w1, b1, Td, sd1, pa, pb, oA, oB);
+          store8o<true>(Aimg, poff(pp), oA);
+          store8o<true>(Aimg, poff(pp + 1), oB);
         }
       }
       fence_proxy_async();
@@ -577,96 +375,21 @@ __global__ void __launch_bounds__(512, 1) k_step_tc(ProbDev P, StepArgs a) {
         const bool ok_w = wait_mma();
         float acc[32];
         tmem_ld32(d_tm + lane_base + col0, acc);
-        if constexpr (!SCALED) {
-          // two points per packed FP32 instruction
-          constexpr float kSmall = FAST ? kSmallMu : kSmallMuAccurate;
 #pragma unroll
-          for (int jp = 0; jp < kPPT; jp += 2) {
-            const float* cA = acc + 8 * jp;
-            const float* cB = cA + 8;
-            float oA[8], oB[8];
-            const float tA = act_tanh<FAST>(cA[0] + bb), tB = act_tanh<FAST>(cB[0] + bb);
-            oA[0] = tA;
-            oB[0] = tB;
-            const bool smA = __all_sync(
-                0xffffffffu, fmaxf(fabsf(cA[1]), fmaxf(fabsf(cA[2]), fabsf(cA[3]))) <= kSmall);
-            const bool smB = __all_sync(
-                0xffffffffu, fmaxf(fabsf(cB[1]), fmaxf(fabsf(cB[2]), fabsf(cB[3]))) <= kSmall);
-            // accurate path: antisymmetric increments small in every lane (their series)
-            bool sdA = false, sdB = false;
-            if constexpr (!FAST) {
-              sdA = __all_sync(0xffffffffu, fmaxf(fabsf(cA[4]), fmaxf(fabsf(cA[5]), fabsf(cA[6]))) <=
-                                                kSmallDelAccurate);
-              sdB = __all_sync(0xffffffffu, fmaxf(fabsf(cB[4]), fmaxf(fabsf(cB[5]), fabsf(cB[6]))) <=
-                                                kSmallDelAccurate);
-            }
-            if (smA && smB) {
-              const F2 T = f2(tA, tB), NT = mul2(T, f2s(-1.0f));
-              const F2 S0 = fma2(NT, T, f2s(1.0f));
-#pragma unroll
-              for (int i = 0; i < 3; ++i) {
-                F2 M, D;
-                tanh_stencil_fwd_pair<FAST>(T, NT, S0, f2(cA[1 + i], cB[1 + i]),
-                                            f2(cA[4 + i], cB[4 + i]), M, D, sdA && sdB);
-                f2get(M, oA[1 + i], oB[1 + i]);
-                f2get(D, oA[4 + i], oB[4 + i]);
-              }
-            } else {
-#pragma unroll
-              for (int i = 0; i < 3; ++i) {
-                tanh_stencil_fwd<FAST>(tA, cA[1 + i], cA[4 + i], 1.f, 1.f, 1.f, 1.f, oA[1 + i],
-                                       oA[4 + i], smA, sdA);
-                tanh_stencil_fwd<FAST>(tB, cB[1 + i], cB[4 + i], 1.f, 1.f, 1.f, 1.f, oB[1 + i],
-                                       oB[4 + i], smB, sdB);
-              }
-            }
-            // column 7 (the interface point) only matters for cut cells with a jump
-            // row; elsewhere its seeds are 0.  The accurate path skips its tanh there
-            // (0, as layer 1 leaves it); in the SFU path the test cost more than it
-            // saved (C2 6 % slower), so that path keeps computing it.
-            if constexpr (FAST) {
-              oA[7] = act_tanh<FAST>(cA[7] + bb);
-              oB[7] = act_tanh<FAST>(cB[7] + bb);
-            } else {
-              const PRec& qa = pr[4 * cgl + jp];
-              const PRec& qb = pr[4 * cgl + jp + 1];
-              oA[7] = (qa.cutj >= 0 && (qa.cutj & 1)) ? act_tanh<FAST>(cA[7] + bb) : 0.f;
-              oB[7] = (qb.cutj >= 0 && (qb.cutj & 1)) ? act_tanh<FAST>(cB[7] + bb) : 0.f;
-            }
-            if (g < NG) {
-              store8o<BF>(Aimg + g * kImgH, poff(jp), oA);
-              store8o<BF>(Aimg + g * kImgH, poff(jp + 1), oB);
-            } else {
-#pragma unroll
-              for (int c2 = 0; c2 < 8; ++c2) {
-                last[8 * jp + c2] = oA[c2];
-                last[8 * jp + 8 + c2] = oB[c2];
-              }
-            }
-          }
-        } else {
-#pragma unroll
-        for (int j = 0; j < kPPT; ++j) {
-          const float* c = acc + 8 * j;
-          float o[8];
-          const float t = act_tanh<FAST>(c[0] + bb);
-          o[0] = t;
-          // symmetric increments small in every lane: their series (see tanh_stencil_fwd)
-          const bool small_mu =
-              FAST && __all_sync(0xffffffffu,
-                                 fmaxf(fabsf(c[1]), fmaxf(fabsf(c[2]), fabsf(c[3]))) * h2s <= kSmallMu);
-#pragma unroll
-          for (int i = 0; i < 3; ++i)
-            tanh_stencil_fwd<FAST>(t, c[1 + i], c[4 + i], hs, h2s, ihs, ih2s, o[1 + i], o[4 + i],
-                                   small_mu);
-          o[7] = act_tanh<FAST>(c[7] + bb);
+        for (int jp = 0; jp < kPPT; jp += 2) {
+          float oA[8], oB[8];
+          hidden_pair<FAST>(acc + 8 * jp, acc + 8 * jp + 8, bb, pr + 4 * cgl + jp,
+                            pr + 4 * cgl + jp + 1, oA, oB);
           if (g < NG) {
-            store8o<BF>(Aimg + g * kImgH, poff(j), o);
+            store8o<true>(Aimg + g * kImgH, poff(jp), oA);
+            store8o<true>(Aimg + g * kImgH, poff(jp + 1), oB);
           } else {
 #pragma unroll
-            for (int c2 = 0; c2 < 8; ++c2) last[8 * j + c2] = o[c2];
+            for (int c2 = 0; c2 < 8; ++c2) {
+              last[8 * jp + c2] = oA[c2];
+              last[8 * jp + 8 + c2] = oB[c2];
+            }
           }
-        }
         }
         if (!end_phase(ok_w)) {
           aborted = true;
@@ -682,7 +405,7 @@ __global__ void __launch_bounds__(512, 1) k_step_tc(ProbDev P, StepArgs a) {
         warp_transpose_reduce32(last, wo, lane, s);  // lane l: column col0 + l
         red[q * 64 + col0 + lane] = s;
       }
-      if (train && gtid < 8 * kHP) cp_async_wait_all();
+      if (gtid < 8 * kHP) cp_async_wait_all();
       named_sync(gbar, 256);
       // ---- output columns and residual rows: lane c of the 8 lanes
       // gtid = 8 p + c of the group's first two warps takes column c of point
@@ -700,8 +423,7 @@ __global__ void __launch_bounds__(512, 1) k_step_tc(ProbDev P, StepArgs a) {
 #pragma unroll
         for (int qq = 1; qq < 4; ++qq) oc += red[64 * qq + 8 * p + c];
         if (c == 0 || c == 7) oc += bo;
-        const float csc = SCALED ? 1.f : (c >= 1 && c <= 3) ? P.inv_h2f
-                                       : (c >= 4 && c <= 6) ? P.inv_hf : 1.f;
+        const float csc = (c >= 1 && c <= 3) ? P.inv_h2f : (c >= 4 && c <= 6) ? P.inv_hf : 1.f;
         oc *= csc;  // the scaled convention of the rows: U, Mt_i = M_i/h^2, Dt_i = D_i/h
         // U and the Mt, Dt columns of this lane's face axis (c / 2)
         const float Uc = __shfl_sync(gmask, oc, 0, 8);
@@ -710,9 +432,7 @@ __global__ void __launch_bounds__(512, 1) k_step_tc(ProbDev P, StepArgs a) {
         const PRec pi = pr[p];
         const bool valid = pi.pt >= 0, is_cut = pi.cutj >= 0;
         float* sdp = seeds + 8 * p;
-        if (cutfwd) {
-          if (valid) a.cut_out[(int64_t)(pi.cutj >> 1) * 16 + net * 8 + c] = oc;
-        } else if (valid && !is_cut) {
+        if (valid && !is_cut) {
           float sdc, r2;
           bool rows64 = false;
           if constexpr (!FAST) rows64 = P.fp64;
@@ -727,9 +447,8 @@ __global__ void __launch_bounds__(512, 1) k_step_tc(ProbDev P, StepArgs a) {
                                              a.scale, c, gmask, sdc);
             if (c == 0) loss_acc += r2;
           }
-          if (c == 0 && a.r2_out) a.r2_out[pi.pt] = (P.level ? a.r2_out[pi.pt] : 0.f) + r2;
           sdp[c] = sdc * csc;  // seeds in this kernel's column convention
-        } else if (valid && train) {
+        } else if (valid) {
           sdp[c] *= csc;  // cut point: the seeds copied at the start of the tile, rescaled
         } else {
           sdp[c] = 0.f;
@@ -750,55 +469,40 @@ __global__ void __launch_bounds__(512, 1) k_step_tc(ProbDev P, StepArgs a) {
           o[0] = lo.x + bo; o[1] = lo.y; o[2] = lo.z; o[3] = lo.w;
           o[4] = hi.x; o[5] = hi.y; o[6] = hi.z; o[7] = hi.w + bo;
         }
-        if (!SCALED) {
 #pragma unroll
-          for (int i = 0; i < 3; ++i) {
-            o[1 + i] *= P.inv_h2f;
-            o[4 + i] *= P.inv_hf;
-          }
+        for (int i = 0; i < 3; ++i) {
+          o[1 + i] *= P.inv_h2f;
+          o[4 + i] *= P.inv_hf;
         }
         const PRec pi = pr[p];
         const bool valid = pi.pt >= 0, is_cut = pi.cutj >= 0;
         float4* sd4 = reinterpret_cast<float4*>(seeds + 8 * p);
-        if (cutfwd) {
-          if (valid) {
-            float4* co = reinterpret_cast<float4*>(a.cut_out + (int64_t)(pi.cutj >> 1) * 16 + net * 8);
-            co[0] = make_float4(o[0], o[1], o[2], o[3]);
-            co[1] = make_float4(o[4], o[5], o[6], o[7]);
-          }
-        } else if (valid && !is_cut) {
+        if (valid && !is_cut) {
           float sd[8];
           const float r2 = uncut_residual_pt<float>(P, net, pi.x, pi.y, pi.z, pi.gx, o, a.scale, sd);
           loss_acc += r2;
-          if (a.r2_out) a.r2_out[pi.pt] = (P.level ? a.r2_out[pi.pt] : 0.f) + r2;
-          if (!SCALED) {
 #pragma unroll
-            for (int i = 0; i < 3; ++i) {
-              sd[1 + i] *= P.inv_h2f;
-              sd[4 + i] *= P.inv_hf;
-            }
+          for (int i = 0; i < 3; ++i) {
+            sd[1 + i] *= P.inv_h2f;
+            sd[4 + i] *= P.inv_hf;
           }
           sd4[0] = make_float4(sd[0], sd[1], sd[2], sd[3]);
           sd4[1] = make_float4(sd[4], sd[5], sd[6], sd[7]);
-        } else if (valid && train) {
+        } else if (valid) {
           // cut point: the seeds copied at the start of the tile, rescaled
-          if (!SCALED) {
-            float4 lo = sd4[0], hi = sd4[1];
-            lo.y *= P.inv_h2f; lo.z *= P.inv_h2f; lo.w *= P.inv_h2f;
-            hi.x *= P.inv_hf; hi.y *= P.inv_hf; hi.z *= P.inv_hf;
-            sd4[0] = lo;
-            sd4[1] = hi;
-          }
+          float4 lo = sd4[0], hi = sd4[1];
+          lo.y *= P.inv_h2f; lo.z *= P.inv_h2f; lo.w *= P.inv_h2f;
+          hi.x *= P.inv_hf; hi.y *= P.inv_hf; hi.z *= P.inv_hf;
+          sd4[0] = lo;
+          sd4[1] = hi;
         } else {
           sd4[0] = make_float4(0.f, 0.f, 0.f, 0.f);
           sd4[1] = make_float4(0.f, 0.f, 0.f, 0.f);
         }
       }
       named_sync(gbar, 256);
-      if (!train) continue;
-
       // ---- backward: adjoint of the last tanh layer (FP32 state in registers)
-      if constexpr (!SCALED) {
+      {
         // two points per packed FP32 instruction
 #pragma unroll
         for (int pp = 0; pp < kPPT; pp += 2) {
@@ -843,37 +547,9 @@ __global__ void __launch_bounds__(512, 1) k_step_tc(ProbDev P, StepArgs a) {
                 gB[7]);
           gbh[NG - 1] += gA[0] + gA[7];
           gbh[NG - 1] += gB[0] + gB[7];
-          store8o<BF>(Aimg + (L - 1) * kImgH, poff(pp), gA);
-          store8o<BF>(Aimg + (L - 1) * kImgH, poff(pp + 1), gB);
+          store8o<true>(Aimg + (L - 1) * kImgH, poff(pp), gA);
+          store8o<true>(Aimg + (L - 1) * kImgH, poff(pp + 1), gB);
         }
-      } else {
-#pragma unroll
-      for (int pp = 0; pp < kPPT; ++pp) {
-        const int p = 4 * cgl + pp;
-        float sd[8];
-        {
-          const float4 lo = *reinterpret_cast<const float4*>(seeds + 8 * p);
-          const float4 hi = *reinterpret_cast<const float4*>(seeds + 8 * p + 4);
-          sd[0] = lo.x; sd[1] = lo.y; sd[2] = lo.z; sd[3] = lo.w;
-          sd[4] = hi.x; sd[5] = hi.y; sd[6] = hi.z; sd[7] = hi.w;
-        }
-        const float* st = last + 8 * pp;
-        float s = 0.f;
-#pragma unroll
-        for (int c = 0; c < 8; ++c) s = fmaf(sd[c], st[c], s);
-        gwo += s;
-        const float t = st[0], s0 = fmaf(-t, t, 1.f);
-        float gz[8];
-        float gzc = s0 * (wo * sd[0]);
-#pragma unroll
-        for (int i = 0; i < 3; ++i)
-          gzc += tanh_stencil_bwd(t, s0, st[1 + i], st[4 + i], wo * sd[1 + i], wo * sd[4 + i], hs,
-                                  h2s, ihs, ih2s, gz[1 + i], gz[4 + i]);
-        gz[0] = gzc;
-        gz[7] = fmaf(-st[7], st[7], 1.f) * (wo * sd[7]);
-        gbh[NG - 1] += gz[0] + gz[7];
-        store8o<BF>(Aimg + (L - 1) * kImgH, poff(pp), gz);
-      }
       }
       if (gtid == 0) {
         float s = 0.f;
@@ -916,13 +592,13 @@ __global__ void __launch_bounds__(512, 1) k_step_tc(ProbDev P, StepArgs a) {
           if ((j & 1) == 0) tmem_ld16(d_tm + lane_base + col0 + 8 * j, G);
           const int p = 4 * cgl + j;
           float st[8];
-          load8o<BF>(img, poff(j), st);
+          load8o<true>(img, poff(j), st);
           float gz[8];
-          if constexpr (!SCALED) {
+          {
             if ((j & 1) == 0) {
               // this point and the next one on packed FP32 pairs
               float sB[8];
-              load8o<BF>(img, poff(j + 1), sB);
+              load8o<true>(img, poff(j + 1), sB);
               const F2 T = f2(st[0], sB[0]);
               const F2 S0 = fma2(mul2(T, f2s(-1.0f)), T, f2s(1.0f));
               F2 gzc = mul2(S0, f2(G[0], G[8]));
@@ -943,26 +619,16 @@ __global__ void __launch_bounds__(512, 1) k_step_tc(ProbDev P, StepArgs a) {
 #pragma unroll
               for (int c2 = 0; c2 < 8; ++c2) gz[c2] = gzP[c2];
             }
-          } else {
-          const float* Gp = G + 8 * (j & 1);
-          const float t = st[0], s0 = fmaf(-t, t, 1.f);
-          float gzc = s0 * Gp[0];
-#pragma unroll
-          for (int i = 0; i < 3; ++i)
-            gzc += tanh_stencil_bwd(t, s0, st[1 + i], st[4 + i], Gp[1 + i], Gp[4 + i], hs, h2s,
-                                    ihs, ih2s, gz[1 + i], gz[4 + i]);
-          gz[0] = gzc;
-          gz[7] = fmaf(-st[7], st[7], 1.f) * Gp[7];
           }
           if (g > 1) {
             const float gsum = gz[0] + gz[7];
 #pragma unroll
             for (int i = 0; i < NG; ++i) gbh[i] += (g - 2 == i) ? gsum : 0.f;
-            store8o<BF>(img, poff(j), gz);
+            store8o<true>(img, poff(j), gz);
           } else {
-            // d del_i / d W1[u][i] = h (unscaled columns) or 1 (scaled)
+            // d del_i / d W1[u][i] = h
             const PRec pi = pr[p];
-            const float dd = SCALED ? 1.f : P.hf;
+            const float dd = P.hf;
             gW1[0] += fmaf(gz[0], pi.x, fmaf(gz[7], pi.gx, gz[4] * dd));
             gW1[1] += fmaf(gz[0], pi.y, fmaf(gz[7], pi.gy, gz[5] * dd));
             gW1[2] += fmaf(gz[0], pi.z, fmaf(gz[7], pi.gz, gz[6] * dd));
@@ -982,7 +648,7 @@ __global__ void __launch_bounds__(512, 1) k_step_tc(ProbDev P, StepArgs a) {
       break;
     }
     fence_after_sync();
-    if (train) flush(net);
+    flush(net);
   }
 
   double lsum = (double)loss_acc + loss_acc_d;
@@ -994,11 +660,9 @@ __global__ void __launch_bounds__(512, 1) k_step_tc(ProbDev P, StepArgs a) {
   if (tid == 0) {
     double s = 0.0;
     for (int ww = 0; ww < 16; ++ww) s += loss_red[ww];
-    if (!cutfwd) a.loss_part[blockIdx.x] = s;
-    if (train) {
-      a.gpart_flag[2 * blockIdx.x] = aborted ? 0 : wrote0;
-      a.gpart_flag[2 * blockIdx.x + 1] = aborted ? 0 : wrote1;
-    }
+    a.loss_part[blockIdx.x] = s;
+    a.gpart_flag[2 * blockIdx.x] = aborted ? 0 : wrote0;
+    a.gpart_flag[2 * blockIdx.x + 1] = aborted ? 0 : wrote1;
   }
   if (aborted) {
     // an MMA or record copy of this group may still be in flight: give it a
@@ -1034,33 +698,26 @@ cudaError_t launch_selftest_wait(long long budget, int* out, cudaStream_t st) {
   return cudaGetLastError();
 }
 
-template <int L, bool BF, bool FAST>
+template <int L, bool FAST>
 static cudaError_t launch_tc_t(const ProbDev& P, const StepArgs& a, int grid, cudaStream_t st) {
-  constexpr bool SCALED = !BF;  // FP16 operands need the 1/h^2, 1/h column scaling
   const size_t smem = tc_smem_bytes(L);
-  cudaError_t e = cudaFuncSetAttribute(k_step_tc<L, BF, FAST, SCALED>,
+  cudaError_t e = cudaFuncSetAttribute(k_step_tc<L, FAST>,
                                        cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;
-  return launch_pdl(k_step_tc<L, BF, FAST, SCALED>, dim3(grid), dim3(512), smem, st, P, a);
+  return launch_pdl(k_step_tc<L, FAST>, dim3(grid), dim3(512), smem, st, P, a);
 }
 
 cudaError_t launch_step_tc(const ProbDev& P, const StepArgs& a, int grid, int prec, cudaStream_t st) {
-  if (P.H != 128) return cudaErrorInvalidValue;
+  if (P.H != 128 || prec != NBM_PREC_BF16) return cudaErrorInvalidValue;
+  if (a.mode != MODE_TRAIN) return launch_fwd_tc(P, a, grid, st);
   // The tanh/reciprocal of the epilogue run on the SFU (tanh.approx, rcp.approx,
   // relative error ~2^-11): every value they produce is rounded to BF16
   // (2^-9) before the next GEMM, so they do not add an error class.  The
   // fine-h mode (FP64 rows) keeps the accurate functions: there the BF16
   // rounding alone already uses most of the gradient tolerance.
-  if (prec == NBM_PREC_BF16 && !P.fp64) {
-    if (P.L == 2) return launch_tc_t<2, true, true>(P, a, grid, st);
-    if (P.L == 3) return launch_tc_t<3, true, true>(P, a, grid, st);
-    if (P.L == 4) return launch_tc_t<4, true, true>(P, a, grid, st);
-  }
-  if (prec == NBM_PREC_BF16) {
-    if (P.L == 2) return launch_tc_t<2, true, false>(P, a, grid, st);
-    if (P.L == 3) return launch_tc_t<3, true, false>(P, a, grid, st);
-    if (P.L == 4) return launch_tc_t<4, true, false>(P, a, grid, st);
-  }
+  if (P.L == 2) return P.fp64 ? launch_tc_t<2, false>(P, a, grid, st) : launch_tc_t<2, true>(P, a, grid, st);
+  if (P.L == 3) return P.fp64 ? launch_tc_t<3, false>(P, a, grid, st) : launch_tc_t<3, true>(P, a, grid, st);
+  if (P.L == 4) return P.fp64 ? launch_tc_t<4, false>(P, a, grid, st) : launch_tc_t<4, true>(P, a, grid, st);
   return cudaErrorInvalidValue;
 }
 

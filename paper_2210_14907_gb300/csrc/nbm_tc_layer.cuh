@@ -1,0 +1,255 @@
+// nbm_tc_layer.cuh -- the pieces that the tensor-core step kernels share: 16-bit
+// operand images, the output layer's warp reduction, and the forward tanh stencil
+// layers of two points on packed FP32 pairs (unscaled difference columns).
+#pragma once
+
+#include <cuda_bf16.h>
+#include <cuda_fp16.h>
+
+#include "nbm_device.cuh"
+#include "nbm_f32x2.cuh"
+#include "nbm_tc_ptx.cuh"
+
+namespace nbm {
+
+constexpr int kHP = 8;        // points per half-tile (one warp group)
+constexpr int kImg = 32768;   // 128 x 128 16-bit weight image
+constexpr int kImgH = 16384;  // 128 x 64 16-bit operand image of a half-tile
+
+template <bool BF>
+struct F16T;
+template <>
+struct F16T<true> {
+  static __device__ __forceinline__ uint32_t pack(float a, float b) {
+    __nv_bfloat162 v = __floats2bfloat162_rn(a, b);
+    return *reinterpret_cast<uint32_t*>(&v);
+  }
+  static __device__ __forceinline__ float2 unpack(uint32_t u) {
+    __nv_bfloat162 v = *reinterpret_cast<__nv_bfloat162*>(&u);
+    return __bfloat1622float2(v);
+  }
+};
+template <>
+struct F16T<false> {
+  static __device__ __forceinline__ uint32_t pack(float a, float b) {
+    __half2 v = __floats2half2_rn(a, b);
+    return *reinterpret_cast<uint32_t*>(&v);
+  }
+  static __device__ __forceinline__ float2 unpack(uint32_t u) {
+    __half2 v = *reinterpret_cast<__half2*>(&u);
+    return __half22float2(v);
+  }
+};
+
+template <bool BF>
+__device__ __forceinline__ void store8o(unsigned char* img, uint32_t off, const float* o) {
+  uint4 pk;
+  pk.x = F16T<BF>::pack(o[0], o[1]);
+  pk.y = F16T<BF>::pack(o[2], o[3]);
+  pk.z = F16T<BF>::pack(o[4], o[5]);
+  pk.w = F16T<BF>::pack(o[6], o[7]);
+  *reinterpret_cast<uint4*>(img + off) = pk;
+}
+template <bool BF>
+__device__ __forceinline__ void load8o(const unsigned char* img, uint32_t off, float* o) {
+  const uint4 pk = *reinterpret_cast<const uint4*>(img + off);
+  float2 a = F16T<BF>::unpack(pk.x), b = F16T<BF>::unpack(pk.y), c = F16T<BF>::unpack(pk.z),
+         d = F16T<BF>::unpack(pk.w);
+  o[0] = a.x; o[1] = a.y; o[2] = b.x; o[3] = b.y;
+  o[4] = c.x; o[5] = c.y; o[6] = d.x; o[7] = d.y;
+}
+template <bool BF>
+__device__ __forceinline__ void store8(unsigned char* img, int row, int col0, const float* o) {
+  uint4 pk;
+  pk.x = F16T<BF>::pack(o[0], o[1]);
+  pk.y = F16T<BF>::pack(o[2], o[3]);
+  pk.z = F16T<BF>::pack(o[4], o[5]);
+  pk.w = F16T<BF>::pack(o[6], o[7]);
+  *reinterpret_cast<uint4*>(img + tc::img_off(row, col0)) = pk;
+}
+template <bool BF>
+__device__ __forceinline__ void load8(const unsigned char* img, int row, int col0, float* o) {
+  const uint4 pk = *reinterpret_cast<const uint4*>(img + tc::img_off(row, col0));
+  float2 a = F16T<BF>::unpack(pk.x), b = F16T<BF>::unpack(pk.y), c = F16T<BF>::unpack(pk.z),
+         d = F16T<BF>::unpack(pk.w);
+  o[0] = a.x; o[1] = a.y; o[2] = b.x; o[3] = b.y;
+  o[4] = c.x; o[5] = c.y; o[6] = d.x; o[7] = d.y;
+}
+
+// Sum of wo * x[0..31] over the 32 lanes of the warp: on return lane l holds
+// the sum of column l (recursive halving, one exchange per value; the scaling
+// is folded into the first halving so that x stays intact for the backward).
+__device__ __forceinline__ void warp_transpose_reduce32(const float (&x)[32], float wo, int lane,
+                                                        float& s) {
+  float v[16];
+#pragma unroll
+  for (int i = 0; i < 16; ++i) {
+    const bool hi = lane & 16;
+    const float keep = wo * (hi ? x[16 + i] : x[i]), send = wo * (hi ? x[i] : x[16 + i]);
+    v[i] = keep + __shfl_xor_sync(0xffffffffu, send, 16);
+  }
+#pragma unroll
+  for (int i = 0; i < 8; ++i) {
+    const bool hi = lane & 8;
+    const float keep = hi ? v[8 + i] : v[i], send = hi ? v[i] : v[8 + i];
+    v[i] = keep + __shfl_xor_sync(0xffffffffu, send, 8);
+  }
+#pragma unroll
+  for (int i = 0; i < 4; ++i) {
+    const bool hi = lane & 4;
+    const float keep = hi ? v[4 + i] : v[i], send = hi ? v[i] : v[4 + i];
+    v[i] = keep + __shfl_xor_sync(0xffffffffu, send, 4);
+  }
+#pragma unroll
+  for (int i = 0; i < 2; ++i) {
+    const bool hi = lane & 2;
+    const float keep = hi ? v[2 + i] : v[i], send = hi ? v[i] : v[2 + i];
+    v[i] = keep + __shfl_xor_sync(0xffffffffu, send, 2);
+  }
+  {
+    const bool hi = lane & 1;
+    const float keep = hi ? v[1] : v[0], send = hi ? v[0] : v[1];
+    s = keep + __shfl_xor_sync(0xffffffffu, send, 1);
+  }
+}
+
+// Two points' tanh stencil layer on packed FP32 pairs (unscaled columns, every
+// lane's symmetric increments small): the arithmetic of tanh_stencil_fwd's
+// series path, operation for operation.
+template <bool FAST>
+__device__ __forceinline__ void tanh_stencil_fwd_pair(F2 T, F2 NT, F2 S0, F2 MU, F2 DE, F2& M,
+                                                      F2& D, bool small_de = false) {
+  const bool sde = !FAST && small_de;  // the series of tanh d and 1/(1-x) (accurate path)
+  F2 TD;
+  if (sde) {
+    const F2 d2 = mul2(DE, DE);
+    TD = mul2(DE, fma2(d2, fma2(d2, f2s(2.0f / 15.0f), f2s(-1.0f / 3.0f)), f2s(1.0f)));
+  } else {
+    float dA, dB;
+    f2get(DE, dA, dB);
+    TD = f2(act_tanh<FAST>(dA), act_tanh<FAST>(dB));
+  }
+  const F2 poly = fma2(fma2(T, T, f2s(-1.0f / 3.0f)), mul2(MU, MU), fma2(NT, MU, f2s(1.0f)));
+  const F2 dm = mul2(mul2(S0, MU), poly);
+  const F2 tw = add2(T, dm);
+  const F2 ntw = mul2(tw, f2s(-1.0f));
+  const F2 sw = fma2(ntw, tw, f2s(1.0f));
+  const F2 td2 = mul2(TD, TD);
+  F2 r2;
+  if (sde) {
+    const F2 x = mul2(mul2(tw, tw), td2);  // 1/(1-x) = 1 + x (1 + x (1 + x))
+    r2 = fma2(x, fma2(x, add2(x, f2s(1.0f)), f2s(1.0f)), f2s(1.0f));
+  } else {
+    float eA, eB;
+    f2get(fma2(add2(sw, f2s(-1.0f)), td2, f2s(1.0f)), eA, eB);
+    r2 = f2(rcp<FAST>(eA), rcp<FAST>(eB));
+  }
+  const F2 k = mul2(sw, r2);
+  M = fma2(mul2(ntw, td2), k, dm);
+  D = mul2(k, TD);
+}
+
+// Layer 1 (3 -> H) of two points in one unit: exact increments mu = 0, del_i = h
+// W1[u][i]; Td[i] = tanh(del_i), sd1: the series of 1/(1-x) (accurate path).
+template <bool FAST>
+__device__ __forceinline__ void layer1_pair(const float (&w1)[3], float b1, const float (&Td)[3],
+                                            bool sd1, const PRec& pa, const PRec& pb, float (&oA)[8],
+                                            float (&oB)[8]) {
+  const F2 W0 = f2s(w1[0]), W1 = f2s(w1[1]), W2 = f2s(w1[2]), B1 = f2s(b1);
+  float zA, zB;
+  f2get(fma2(W0, f2(pa.x, pb.x), fma2(W1, f2(pa.y, pb.y), fma2(W2, f2(pa.z, pb.z), B1))), zA, zB);
+  const F2 T = f2(act_tanh<FAST>(zA), act_tanh<FAST>(zB));
+  const F2 NT = mul2(T, f2s(-1.0f));
+  const F2 SW = fma2(NT, T, f2s(1.0f));
+  const F2 NTT = mul2(NT, T);
+  const F2 NTS = mul2(NT, SW);
+  f2get(T, oA[0], oB[0]);
+#pragma unroll
+  for (int i = 0; i < 3; ++i) {
+    const F2 TD = f2s(Td[i]), TD2 = mul2(TD, TD);
+    F2 R2;
+    if (sd1) {  // 1 / (1 - t^2 Td^2) by its series
+      const F2 x = mul2(mul2(T, T), TD2);
+      R2 = fma2(x, fma2(x, add2(x, f2s(1.0f)), f2s(1.0f)), f2s(1.0f));
+    } else {
+      float eA, eB;
+      f2get(fma2(NTT, TD2, f2s(1.0f)), eA, eB);
+      R2 = f2(rcp<FAST>(eA), rcp<FAST>(eB));
+    }
+    f2get(mul2(mul2(NTS, TD2), R2), oA[1 + i], oB[1 + i]);
+    f2get(mul2(mul2(SW, TD), R2), oA[4 + i], oB[4 + i]);
+  }
+  const bool ja = pa.cutj >= 0 && (pa.cutj & 1), jb = pb.cutj >= 0 && (pb.cutj & 1);
+  oA[7] = ja ? act_tanh<FAST>(fmaf(w1[0], pa.gx, fmaf(w1[1], pa.gy, fmaf(w1[2], pa.gz, b1)))) : 0.f;
+  oB[7] = jb ? act_tanh<FAST>(fmaf(w1[0], pb.gx, fmaf(w1[1], pb.gy, fmaf(w1[2], pb.gz, b1)))) : 0.f;
+}
+
+// tanh(h W1[u][i]) of the first layer (it depends on the unit only); sd1: every
+// lane's increments are small and their series serves (accurate path)
+template <bool FAST>
+__device__ __forceinline__ void layer1_increments(const float (&w1)[3], float h, float (&Td)[3],
+                                                  bool& sd1) {
+  const float d[3] = {w1[0] * h, w1[1] * h, w1[2] * h};
+  sd1 = false;
+  if constexpr (!FAST)
+    sd1 = __all_sync(0xffffffffu,
+                     fmaxf(fabsf(d[0]), fmaxf(fabsf(d[1]), fabsf(d[2]))) <= kSmallDelAccurate);
+#pragma unroll
+  for (int i = 0; i < 3; ++i) Td[i] = sd1 ? tanh_small(d[i]) : act_tanh<FAST>(d[i]);
+}
+
+// A hidden layer's outputs of two points in one unit from the GEMM's columns cA, cB
+// and the bias.  Column 7 (the interface point) only matters for cut cells with a
+// jump row; elsewhere its seeds are 0.  The accurate path skips its tanh there (0,
+// as layer 1 leaves it); in the SFU path the test cost more than it saved (C2 6 %
+// slower), so that path keeps computing it.
+template <bool FAST>
+__device__ __forceinline__ void hidden_pair(const float* cA, const float* cB, float bb,
+                                            const PRec* pa, const PRec* pb, float (&oA)[8],
+                                            float (&oB)[8]) {
+  constexpr float kSmall = FAST ? kSmallMu : kSmallMuAccurate;
+  const float tA = act_tanh<FAST>(cA[0] + bb), tB = act_tanh<FAST>(cB[0] + bb);
+  oA[0] = tA;
+  oB[0] = tB;
+  const bool smA = __all_sync(0xffffffffu,
+                              fmaxf(fabsf(cA[1]), fmaxf(fabsf(cA[2]), fabsf(cA[3]))) <= kSmall);
+  const bool smB = __all_sync(0xffffffffu,
+                              fmaxf(fabsf(cB[1]), fmaxf(fabsf(cB[2]), fabsf(cB[3]))) <= kSmall);
+  // accurate path: antisymmetric increments small in every lane (their series)
+  bool sdA = false, sdB = false;
+  if constexpr (!FAST) {
+    sdA = __all_sync(0xffffffffu, fmaxf(fabsf(cA[4]), fmaxf(fabsf(cA[5]), fabsf(cA[6]))) <=
+                                      kSmallDelAccurate);
+    sdB = __all_sync(0xffffffffu, fmaxf(fabsf(cB[4]), fmaxf(fabsf(cB[5]), fabsf(cB[6]))) <=
+                                      kSmallDelAccurate);
+  }
+  if (smA && smB) {
+    const F2 T = f2(tA, tB), NT = mul2(T, f2s(-1.0f));
+    const F2 S0 = fma2(NT, T, f2s(1.0f));
+#pragma unroll
+    for (int i = 0; i < 3; ++i) {
+      F2 M, D;
+      tanh_stencil_fwd_pair<FAST>(T, NT, S0, f2(cA[1 + i], cB[1 + i]), f2(cA[4 + i], cB[4 + i]), M,
+                                  D, sdA && sdB);
+      f2get(M, oA[1 + i], oB[1 + i]);
+      f2get(D, oA[4 + i], oB[4 + i]);
+    }
+  } else {
+#pragma unroll
+    for (int i = 0; i < 3; ++i) {
+      tanh_stencil_fwd<FAST>(tA, cA[1 + i], cA[4 + i], 1.f, 1.f, 1.f, 1.f, oA[1 + i], oA[4 + i],
+                             smA, sdA);
+      tanh_stencil_fwd<FAST>(tB, cB[1 + i], cB[4 + i], 1.f, 1.f, 1.f, 1.f, oB[1 + i], oB[4 + i],
+                             smB, sdB);
+    }
+  }
+  if constexpr (FAST) {
+    oA[7] = act_tanh<FAST>(cA[7] + bb);
+    oB[7] = act_tanh<FAST>(cB[7] + bb);
+  } else {
+    oA[7] = (pa->cutj >= 0 && (pa->cutj & 1)) ? act_tanh<FAST>(cA[7] + bb) : 0.f;
+    oB[7] = (pb->cutj >= 0 && (pb->cutj & 1)) ? act_tanh<FAST>(cB[7] + bb) : 0.f;
+  }
+}
+
+}  // namespace nbm

@@ -412,11 +412,8 @@ __global__ void __launch_bounds__(512, 1) k_step_tc(ProbDev P, StepArgs a) {
       // p, and the point's row is spread over its 8 lanes
       // (uncut_residual_lanes: one face per lane, sums by shuffles), so the
       // row's dependency chain runs on 8 lanes instead of 1.  FP64 rows only
-      // occur in the accurate (!FAST) instances.  The fast four-layer
-      // instance keeps one thread per point (uncut_residual_pt): there the
-      // lane rows cost registers elsewhere and made the kernel 4 % slower.
-      constexpr bool kLaneRows = !FAST || L <= 3;
-      if (kLaneRows && gtid < 8 * kHP) {
+      // occur in the accurate (!FAST) instances.
+      if (gtid < 8 * kHP) {
         const int p = gtid >> 3, c = gtid & 7;
         const unsigned gmask = 0xFFu << (gtid & 24);
         float oc = red[8 * p + c];
@@ -452,52 +449,6 @@ __global__ void __launch_bounds__(512, 1) k_step_tc(ProbDev P, StepArgs a) {
           sdp[c] *= csc;  // cut point: the seeds copied at the start of the tile, rescaled
         } else {
           sdp[c] = 0.f;
-        }
-      } else if (!kLaneRows && gtid < kHP) {
-        // one thread per point (FP32 rows)
-        const int p = gtid;
-        float o[8];
-        {
-          const float4* r4 = reinterpret_cast<const float4*>(red) + 2 * p;
-          float4 lo = r4[0], hi = r4[1];
-#pragma unroll
-          for (int qq = 1; qq < 4; ++qq) {
-            const float4 l2 = r4[16 * qq], h2 = r4[16 * qq + 1];
-            lo.x += l2.x; lo.y += l2.y; lo.z += l2.z; lo.w += l2.w;
-            hi.x += h2.x; hi.y += h2.y; hi.z += h2.z; hi.w += h2.w;
-          }
-          o[0] = lo.x + bo; o[1] = lo.y; o[2] = lo.z; o[3] = lo.w;
-          o[4] = hi.x; o[5] = hi.y; o[6] = hi.z; o[7] = hi.w + bo;
-        }
-#pragma unroll
-        for (int i = 0; i < 3; ++i) {
-          o[1 + i] *= P.inv_h2f;
-          o[4 + i] *= P.inv_hf;
-        }
-        const PRec pi = pr[p];
-        const bool valid = pi.pt >= 0, is_cut = pi.cutj >= 0;
-        float4* sd4 = reinterpret_cast<float4*>(seeds + 8 * p);
-        if (valid && !is_cut) {
-          float sd[8];
-          const float r2 = uncut_residual_pt<float>(P, net, pi.x, pi.y, pi.z, pi.gx, o, a.scale, sd);
-          loss_acc += r2;
-#pragma unroll
-          for (int i = 0; i < 3; ++i) {
-            sd[1 + i] *= P.inv_h2f;
-            sd[4 + i] *= P.inv_hf;
-          }
-          sd4[0] = make_float4(sd[0], sd[1], sd[2], sd[3]);
-          sd4[1] = make_float4(sd[4], sd[5], sd[6], sd[7]);
-        } else if (valid) {
-          // cut point: the seeds copied at the start of the tile, rescaled
-          float4 lo = sd4[0], hi = sd4[1];
-          lo.y *= P.inv_h2f; lo.z *= P.inv_h2f; lo.w *= P.inv_h2f;
-          hi.x *= P.inv_hf; hi.y *= P.inv_hf; hi.z *= P.inv_hf;
-          sd4[0] = lo;
-          sd4[1] = hi;
-        } else {
-          sd4[0] = make_float4(0.f, 0.f, 0.f, 0.f);
-          sd4[1] = make_float4(0.f, 0.f, 0.f, 0.f);
         }
       }
       named_sync(gbar, 256);

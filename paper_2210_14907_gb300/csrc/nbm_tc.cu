@@ -330,7 +330,7 @@ __global__ void __launch_bounds__(512, 1) k_step_tc(ProbDev P, StepArgs a) {
       if (gtid < 8 * kHP) {
         const PRec& pc = pr[gtid >> 3];
         if (pc.pt >= 0 && pc.cutj >= 0)
-          cp_async4(smem_u32(seeds + gtid),
+          cp_async4(smem_u32(seeds + pair_col(gtid >> 3, gtid & 7)),
                     a.cut_seed + (int64_t)(pc.cutj >> 1) * 16 + net * 8 + (gtid & 7));
       }
 
@@ -342,10 +342,9 @@ __global__ void __launch_bounds__(512, 1) k_step_tc(ProbDev P, StepArgs a) {
 #pragma unroll
         for (int pp = 0; pp < kPPT; pp += 2) {
           const PRec pa = pr[4 * cgl + pp], pb = pr[4 * cgl + pp + 1];
-          float oA[8], oB[8];
-          layer1_pair<FAST>(w1, b1, Td, sd1, pa, pb, oA, oB);
-          store8o<true>(Aimg, poff(pp), oA);
-          store8o<true>(Aimg, poff(pp + 1), oB);
+          F2 o[8];
+          layer1_pair<FAST>(w1, b1, Td, sd1, pa, pb, o);
+          store_pair(Aimg, poff(pp), poff(pp + 1), o);
         }
       }
       fence_proxy_async();
@@ -377,18 +376,13 @@ __global__ void __launch_bounds__(512, 1) k_step_tc(ProbDev P, StepArgs a) {
         tmem_ld32(d_tm + lane_base + col0, acc);
 #pragma unroll
         for (int jp = 0; jp < kPPT; jp += 2) {
-          float oA[8], oB[8];
-          hidden_pair<FAST>(acc + 8 * jp, acc + 8 * jp + 8, bb, pr + 4 * cgl + jp,
-                            pr + 4 * cgl + jp + 1, oA, oB);
+          F2 o[8];
+          hidden_pair<FAST>(acc + 8 * jp, bb, pr + 4 * cgl + jp, pr + 4 * cgl + jp + 1, o);
           if (g < NG) {
-            store8o<true>(Aimg + g * kImgH, poff(jp), oA);
-            store8o<true>(Aimg + g * kImgH, poff(jp + 1), oB);
+            store_pair(Aimg + g * kImgH, poff(jp), poff(jp + 1), o);
           } else {
 #pragma unroll
-            for (int c2 = 0; c2 < 8; ++c2) {
-              last[8 * jp + c2] = oA[c2];
-              last[8 * jp + 8 + c2] = oB[c2];
-            }
+            for (int c2 = 0; c2 < 8; ++c2) f2get(o[c2], last[8 * jp + 2 * c2], last[8 * jp + 2 * c2 + 1]);
           }
         }
         if (!end_phase(ok_w)) {
@@ -416,9 +410,10 @@ __global__ void __launch_bounds__(512, 1) k_step_tc(ProbDev P, StepArgs a) {
       if (gtid < 8 * kHP) {
         const int p = gtid >> 3, c = gtid & 7;
         const unsigned gmask = 0xFFu << (gtid & 24);
-        float oc = red[8 * p + c];
+        const int pc = pair_col(p, c);
+        float oc = red[pc];
 #pragma unroll
-        for (int qq = 1; qq < 4; ++qq) oc += red[64 * qq + 8 * p + c];
+        for (int qq = 1; qq < 4; ++qq) oc += red[64 * qq + pc];
         if (c == 0 || c == 7) oc += bo;
         const float csc = (c >= 1 && c <= 3) ? P.inv_h2f : (c >= 4 && c <= 6) ? P.inv_hf : 1.f;
         oc *= csc;  // the scaled convention of the rows: U, Mt_i = M_i/h^2, Dt_i = D_i/h
@@ -428,7 +423,7 @@ __global__ void __launch_bounds__(512, 1) k_step_tc(ProbDev P, StepArgs a) {
         const float Dtc = __shfl_sync(gmask, oc, 4 + (c >> 1), 8);
         const PRec pi = pr[p];
         const bool valid = pi.pt >= 0, is_cut = pi.cutj >= 0;
-        float* sdp = seeds + 8 * p;
+        float& sdp = seeds[pc];
         if (valid && !is_cut) {
           float sdc, r2;
           bool rows64 = false;
@@ -444,11 +439,11 @@ __global__ void __launch_bounds__(512, 1) k_step_tc(ProbDev P, StepArgs a) {
                                              a.scale, c, gmask, sdc);
             if (c == 0) loss_acc += r2;
           }
-          sdp[c] = sdc * csc;  // seeds in this kernel's column convention
+          sdp = sdc * csc;  // seeds in this kernel's column convention
         } else if (valid) {
-          sdp[c] *= csc;  // cut point: the seeds copied at the start of the tile, rescaled
+          sdp *= csc;  // cut point: the seeds copied at the start of the tile, rescaled
         } else {
-          sdp[c] = 0.f;
+          sdp = 0.f;
         }
       }
       named_sync(gbar, 256);
@@ -457,20 +452,21 @@ __global__ void __launch_bounds__(512, 1) k_step_tc(ProbDev P, StepArgs a) {
         // two points per packed FP32 instruction
 #pragma unroll
         for (int pp = 0; pp < kPPT; pp += 2) {
-          float sA[8], sB[8];
+          F2 sd[8], st[8], gz[8];
           {
             const float4* s4 = reinterpret_cast<const float4*>(seeds + 8 * (4 * cgl + pp));
-            const float4 a0 = s4[0], a1 = s4[1], b0 = s4[2], b1v = s4[3];
-            sA[0] = a0.x; sA[1] = a0.y; sA[2] = a0.z; sA[3] = a0.w;
-            sA[4] = a1.x; sA[5] = a1.y; sA[6] = a1.z; sA[7] = a1.w;
-            sB[0] = b0.x; sB[1] = b0.y; sB[2] = b0.z; sB[3] = b0.w;
-            sB[4] = b1v.x; sB[5] = b1v.y; sB[6] = b1v.z; sB[7] = b1v.w;
-          }
-          const float* stA = last + 8 * pp;
-          const float* stB = stA + 8;
-          F2 sw = mul2(f2(sA[0], sB[0]), f2(stA[0], stB[0]));
 #pragma unroll
-          for (int c = 1; c < 8; ++c) sw = fma2(f2(sA[c], sB[c]), f2(stA[c], stB[c]), sw);
+            for (int c = 0; c < 4; ++c) {
+              const float4 v = s4[c];
+              sd[2 * c] = f2(v.x, v.y);
+              sd[2 * c + 1] = f2(v.z, v.w);
+            }
+          }
+#pragma unroll
+          for (int c = 0; c < 8; ++c) st[c] = f2(last[8 * pp + 2 * c], last[8 * pp + 2 * c + 1]);
+          F2 sw = mul2(sd[0], st[0]);
+#pragma unroll
+          for (int c = 1; c < 8; ++c) sw = fma2(sd[c], st[c], sw);
           {
             float x, y;
             f2get(sw, x, y);
@@ -478,33 +474,27 @@ __global__ void __launch_bounds__(512, 1) k_step_tc(ProbDev P, StepArgs a) {
             gwo += y;
           }
           const F2 WO = f2s(wo);
-          const F2 T = f2(stA[0], stB[0]);
+          const F2 T = st[0];
           const F2 S0 = fma2(mul2(T, f2s(-1.0f)), T, f2s(1.0f));
-          float gA[8], gB[8];
-          F2 gzc = mul2(S0, mul2(WO, f2(sA[0], sB[0])));
+          F2 gzc = mul2(S0, mul2(WO, sd[0]));
 #pragma unroll
-          for (int i = 0; i < 3; ++i) {
-            F2 gm, gd;
-            gzc = add2(gzc, tanh_stencil_bwd_pair(T, S0, f2(stA[1 + i], stB[1 + i]),
-                                                  f2(stA[4 + i], stB[4 + i]),
-                                                  mul2(WO, f2(sA[1 + i], sB[1 + i])),
-                                                  mul2(WO, f2(sA[4 + i], sB[4 + i])), gm, gd));
-            f2get(gm, gA[1 + i], gB[1 + i]);
-            f2get(gd, gA[4 + i], gB[4 + i]);
+          for (int i = 0; i < 3; ++i)
+            gzc = add2(gzc, tanh_stencil_bwd_pair(T, S0, st[1 + i], st[4 + i], mul2(WO, sd[1 + i]),
+                                                  mul2(WO, sd[4 + i]), gz[1 + i], gz[4 + i]));
+          gz[0] = gzc;
+          gz[7] = mul2(fma2(mul2(st[7], f2s(-1.0f)), st[7], f2s(1.0f)), mul2(WO, sd[7]));
+          {
+            float x, y;
+            f2get(add2(gz[0], gz[7]), x, y);
+            gbh[NG - 1] += x;
+            gbh[NG - 1] += y;
           }
-          f2get(gzc, gA[0], gB[0]);
-          const F2 T7 = f2(stA[7], stB[7]);
-          f2get(mul2(fma2(mul2(T7, f2s(-1.0f)), T7, f2s(1.0f)), mul2(WO, f2(sA[7], sB[7]))), gA[7],
-                gB[7]);
-          gbh[NG - 1] += gA[0] + gA[7];
-          gbh[NG - 1] += gB[0] + gB[7];
-          store8o<true>(Aimg + (L - 1) * kImgH, poff(pp), gA);
-          store8o<true>(Aimg + (L - 1) * kImgH, poff(pp + 1), gB);
+          store_pair(Aimg + (L - 1) * kImgH, poff(pp), poff(pp + 1), gz);
         }
       }
       if (gtid == 0) {
         float s = 0.f;
-        for (int p = 0; p < kHP; ++p) s += seeds[8 * p] + seeds[8 * p + 7];
+        for (int p = 0; p < kHP; ++p) s += seeds[pair_col(p, 0)] + seeds[pair_col(p, 7)];
         gbo += s;
       }
       fence_proxy_async();
@@ -536,54 +526,48 @@ __global__ void __launch_bounds__(512, 1) k_step_tc(ProbDev P, StepArgs a) {
         const bool ok_w = wait_mma();
         if (gtid == 0 && ok_w) st_release_s32(done_cnt + grp, nph + 1);
         unsigned char* img = Aimg + (g - 1) * kImgH;  // state of act[g-1]
-        float G[16];  // two points at a time: registers are short here
-        float gzP[8];  // the second point's adjoint of a packed pair
 #pragma unroll
-        for (int j = 0; j < kPPT; ++j) {
-          if ((j & 1) == 0) tmem_ld16(d_tm + lane_base + col0 + 8 * j, G);
-          const int p = 4 * cgl + j;
-          float st[8];
-          load8o<true>(img, poff(j), st);
-          float gz[8];
-          {
-            if ((j & 1) == 0) {
-              // this point and the next one on packed FP32 pairs
-              float sB[8];
-              load8o<true>(img, poff(j + 1), sB);
-              const F2 T = f2(st[0], sB[0]);
-              const F2 S0 = fma2(mul2(T, f2s(-1.0f)), T, f2s(1.0f));
-              F2 gzc = mul2(S0, f2(G[0], G[8]));
+        for (int j = 0; j < kPPT; j += 2) {  // two points at a time: registers are short here
+          float G[16];
+          tmem_ld16(d_tm + lane_base + col0 + 8 * j, G);
+          F2 st[8], gz[8];
+          load_pair(img, poff(j), poff(j + 1), st);
+          const F2 T = st[0];
+          const F2 S0 = fma2(mul2(T, f2s(-1.0f)), T, f2s(1.0f));
+          F2 gzc = mul2(S0, f2(G[0], G[1]));
 #pragma unroll
-              for (int i = 0; i < 3; ++i) {
-                F2 gm, gd;
-                gzc = add2(gzc, tanh_stencil_bwd_pair(T, S0, f2(st[1 + i], sB[1 + i]),
-                                                      f2(st[4 + i], sB[4 + i]),
-                                                      f2(G[1 + i], G[9 + i]),
-                                                      f2(G[4 + i], G[12 + i]), gm, gd));
-                f2get(gm, gz[1 + i], gzP[1 + i]);
-                f2get(gd, gz[4 + i], gzP[4 + i]);
-              }
-              f2get(gzc, gz[0], gzP[0]);
-              const F2 T7 = f2(st[7], sB[7]);
-              f2get(mul2(fma2(mul2(T7, f2s(-1.0f)), T7, f2s(1.0f)), f2(G[7], G[15])), gz[7], gzP[7]);
-            } else {
-#pragma unroll
-              for (int c2 = 0; c2 < 8; ++c2) gz[c2] = gzP[c2];
-            }
-          }
+          for (int i = 0; i < 3; ++i)
+            gzc = add2(gzc, tanh_stencil_bwd_pair(T, S0, st[1 + i], st[4 + i],
+                                                  f2(G[2 + 2 * i], G[3 + 2 * i]),
+                                                  f2(G[8 + 2 * i], G[9 + 2 * i]), gz[1 + i],
+                                                  gz[4 + i]));
+          gz[0] = gzc;
+          gz[7] = mul2(fma2(mul2(st[7], f2s(-1.0f)), st[7], f2s(1.0f)), f2(G[14], G[15]));
+          float gsA, gsB;
+          f2get(add2(gz[0], gz[7]), gsA, gsB);
           if (g > 1) {
-            const float gsum = gz[0] + gz[7];
 #pragma unroll
-            for (int i = 0; i < NG; ++i) gbh[i] += (g - 2 == i) ? gsum : 0.f;
-            store8o<true>(img, poff(j), gz);
+            for (int i = 0; i < NG; ++i) {
+              gbh[i] += (g - 2 == i) ? gsA : 0.f;
+              gbh[i] += (g - 2 == i) ? gsB : 0.f;
+            }
+            store_pair(img, poff(j), poff(j + 1), gz);
           } else {
             // d del_i / d W1[u][i] = h
-            const PRec pi = pr[p];
-            const float dd = P.hf;
-            gW1[0] += fmaf(gz[0], pi.x, fmaf(gz[7], pi.gx, gz[4] * dd));
-            gW1[1] += fmaf(gz[0], pi.y, fmaf(gz[7], pi.gy, gz[5] * dd));
-            gW1[2] += fmaf(gz[0], pi.z, fmaf(gz[7], pi.gz, gz[6] * dd));
-            gb1 += gz[0] + gz[7];
+            const PRec &pa = pr[4 * cgl + j], &pb = pr[4 * cgl + j + 1];
+            const F2 dd = f2s(P.hf);
+            float x, y;
+            f2get(fma2(gz[0], f2(pa.x, pb.x), fma2(gz[7], f2(pa.gx, pb.gx), mul2(gz[4], dd))), x, y);
+            gW1[0] += x;
+            gW1[0] += y;
+            f2get(fma2(gz[0], f2(pa.y, pb.y), fma2(gz[7], f2(pa.gy, pb.gy), mul2(gz[5], dd))), x, y);
+            gW1[1] += x;
+            gW1[1] += y;
+            f2get(fma2(gz[0], f2(pa.z, pb.z), fma2(gz[7], f2(pa.gz, pb.gz), mul2(gz[6], dd))), x, y);
+            gW1[2] += x;
+            gW1[2] += y;
+            gb1 += gsA;
+            gb1 += gsB;
           }
         }
         if (!end_phase(ok_w)) {

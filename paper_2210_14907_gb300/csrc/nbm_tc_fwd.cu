@@ -238,10 +238,9 @@ __global__ void __launch_bounds__(kFwdT, 1) k_fwd_tc(ProbDev P, StepArgs a) {
 #pragma unroll
         for (int pp = 0; pp < kPPT; pp += 2) {
           const PRec& pa = pr[X * kHP + 4 * cgl + pp];
-          float oA[8], oB[8];
-          layer1_pair<FAST>(w1, b1, Td, sd1, pa, (&pa)[1], oA, oB);
-          store8o<true>(Aimg + X * kImgH, poff(pp), oA);
-          store8o<true>(Aimg + X * kImgH, poff(pp + 1), oB);
+          F2 o[8];
+          layer1_pair<FAST>(w1, b1, Td, sd1, pa, (&pa)[1], o);
+          store_pair(Aimg + X * kImgH, poff(pp), poff(pp + 1), o);
         }
         ready(X);
       }
@@ -258,17 +257,13 @@ __global__ void __launch_bounds__(kFwdT, 1) k_fwd_tc(ProbDev P, StepArgs a) {
           tmem_ld32(d_tm + 64 * X + lane_base + col0, acc);
 #pragma unroll
           for (int jp = 0; jp < kPPT; jp += 2) {
-            float oA[8], oB[8];
-            hidden_pair<FAST>(acc + 8 * jp, acc + 8 * jp + 8, bb, px + jp, px + jp + 1, oA, oB);
+            F2 o[8];
+            hidden_pair<FAST>(acc + 8 * jp, bb, px + jp, px + jp + 1, o);
             if (g < NG) {
-              store8o<true>(Aimg + X * kImgH, poff(jp), oA);
-              store8o<true>(Aimg + X * kImgH, poff(jp + 1), oB);
+              store_pair(Aimg + X * kImgH, poff(jp), poff(jp + 1), o);
             } else {
 #pragma unroll
-              for (int c = 0; c < 8; ++c) {
-                acc[8 * jp + c] = oA[c];
-                acc[8 * jp + 8 + c] = oB[c];
-              }
+              for (int c = 0; c < 8; ++c) f2get(o[c], acc[8 * jp + 2 * c], acc[8 * jp + 2 * c + 1]);
             }
           }
           if (g < NG) {
@@ -289,7 +284,7 @@ __global__ void __launch_bounds__(kFwdT, 1) k_fwd_tc(ProbDev P, StepArgs a) {
       if (gtid < 64 * cnt) {
         const int X = gtid >> 6, p = (gtid >> 3) & 7, c = gtid & 7;
         const unsigned gmask = 0xFFu << (gtid & 24);
-        const float* rx = red + X * 256 + 8 * p + c;
+        const float* rx = red + X * 256 + pair_col(p, c);
         float oc = rx[0];
 #pragma unroll
         for (int qq = 1; qq < 4; ++qq) oc += rx[64 * qq];

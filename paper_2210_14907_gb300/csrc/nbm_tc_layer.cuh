@@ -4,7 +4,6 @@
 #pragma once
 
 #include <cuda_bf16.h>
-#include <cuda_fp16.h>
 
 #include "nbm_device.cuh"
 #include "nbm_f32x2.cuh"
@@ -16,64 +15,36 @@ constexpr int kHP = 8;        // points per half-tile (one warp group)
 constexpr int kImg = 32768;   // 128 x 128 16-bit weight image
 constexpr int kImgH = 16384;  // 128 x 64 16-bit operand image of a half-tile
 
-template <bool BF>
-struct F16T;
-template <>
-struct F16T<true> {
-  static __device__ __forceinline__ uint32_t pack(float a, float b) {
-    __nv_bfloat162 v = __floats2bfloat162_rn(a, b);
-    return *reinterpret_cast<uint32_t*>(&v);
-  }
-  static __device__ __forceinline__ float2 unpack(uint32_t u) {
-    __nv_bfloat162 v = *reinterpret_cast<__nv_bfloat162*>(&u);
-    return __bfloat1622float2(v);
-  }
-};
-template <>
-struct F16T<false> {
-  static __device__ __forceinline__ uint32_t pack(float a, float b) {
-    __half2 v = __floats2half2_rn(a, b);
-    return *reinterpret_cast<uint32_t*>(&v);
-  }
-  static __device__ __forceinline__ float2 unpack(uint32_t u) {
-    __half2 v = *reinterpret_cast<__half2*>(&u);
-    return __half22float2(v);
-  }
-};
+// Column order of an operand image.  The 16 columns of two neighbouring points A, B
+// are interleaved: column 16 P + 2 c + s is column c of point 2 P + s.  A thread's
+// accumulator registers 2 c and 2 c + 1 are then the pair (A, B) that the packed FP32
+// instructions take, and a 32-bit word of the image holds the same pair in BF16, so
+// neither needs moves to be put together or taken apart.
+__device__ __forceinline__ int pair_col(int p, int c) { return (p >> 1) * 16 + 2 * c + (p & 1); }
 
-template <bool BF>
-__device__ __forceinline__ void store8o(unsigned char* img, uint32_t off, const float* o) {
-  uint4 pk;
-  pk.x = F16T<BF>::pack(o[0], o[1]);
-  pk.y = F16T<BF>::pack(o[2], o[3]);
-  pk.z = F16T<BF>::pack(o[4], o[5]);
-  pk.w = F16T<BF>::pack(o[6], o[7]);
-  *reinterpret_cast<uint4*>(img + off) = pk;
+__device__ __forceinline__ uint32_t pack_bf2(F2 v) {
+  float a, b;
+  f2get(v, a, b);
+  const __nv_bfloat162 w = __floats2bfloat162_rn(a, b);
+  return *reinterpret_cast<const uint32_t*>(&w);
 }
-template <bool BF>
-__device__ __forceinline__ void load8o(const unsigned char* img, uint32_t off, float* o) {
-  const uint4 pk = *reinterpret_cast<const uint4*>(img + off);
-  float2 a = F16T<BF>::unpack(pk.x), b = F16T<BF>::unpack(pk.y), c = F16T<BF>::unpack(pk.z),
-         d = F16T<BF>::unpack(pk.w);
-  o[0] = a.x; o[1] = a.y; o[2] = b.x; o[3] = b.y;
-  o[4] = c.x; o[5] = c.y; o[6] = d.x; o[7] = d.y;
+__device__ __forceinline__ F2 unpack_bf2(uint32_t u) {
+  return f2(__uint_as_float(u << 16), __uint_as_float(u & 0xffff0000u));
 }
-template <bool BF>
-__device__ __forceinline__ void store8(unsigned char* img, int row, int col0, const float* o) {
-  uint4 pk;
-  pk.x = F16T<BF>::pack(o[0], o[1]);
-  pk.y = F16T<BF>::pack(o[2], o[3]);
-  pk.z = F16T<BF>::pack(o[4], o[5]);
-  pk.w = F16T<BF>::pack(o[6], o[7]);
-  *reinterpret_cast<uint4*>(img + tc::img_off(row, col0)) = pk;
+// the pair's 16 columns: 16-byte chunks at off0 (c = 0..3) and off1 (c = 4..7)
+__device__ __forceinline__ void store_pair(unsigned char* img, uint32_t off0, uint32_t off1,
+                                           const F2 (&o)[8]) {
+  *reinterpret_cast<uint4*>(img + off0) =
+      make_uint4(pack_bf2(o[0]), pack_bf2(o[1]), pack_bf2(o[2]), pack_bf2(o[3]));
+  *reinterpret_cast<uint4*>(img + off1) =
+      make_uint4(pack_bf2(o[4]), pack_bf2(o[5]), pack_bf2(o[6]), pack_bf2(o[7]));
 }
-template <bool BF>
-__device__ __forceinline__ void load8(const unsigned char* img, int row, int col0, float* o) {
-  const uint4 pk = *reinterpret_cast<const uint4*>(img + tc::img_off(row, col0));
-  float2 a = F16T<BF>::unpack(pk.x), b = F16T<BF>::unpack(pk.y), c = F16T<BF>::unpack(pk.z),
-         d = F16T<BF>::unpack(pk.w);
-  o[0] = a.x; o[1] = a.y; o[2] = b.x; o[3] = b.y;
-  o[4] = c.x; o[5] = c.y; o[6] = d.x; o[7] = d.y;
+__device__ __forceinline__ void load_pair(const unsigned char* img, uint32_t off0, uint32_t off1,
+                                          F2 (&o)[8]) {
+  const uint4 a = *reinterpret_cast<const uint4*>(img + off0);
+  const uint4 b = *reinterpret_cast<const uint4*>(img + off1);
+  o[0] = unpack_bf2(a.x); o[1] = unpack_bf2(a.y); o[2] = unpack_bf2(a.z); o[3] = unpack_bf2(a.w);
+  o[4] = unpack_bf2(b.x); o[5] = unpack_bf2(b.y); o[6] = unpack_bf2(b.z); o[7] = unpack_bf2(b.w);
 }
 
 // Sum of wo * x[0..31] over the 32 lanes of the warp: on return lane l holds
@@ -153,8 +124,8 @@ __device__ __forceinline__ void tanh_stencil_fwd_pair(F2 T, F2 NT, F2 S0, F2 MU,
 // W1[u][i]; Td[i] = tanh(del_i), sd1: the series of 1/(1-x) (accurate path).
 template <bool FAST>
 __device__ __forceinline__ void layer1_pair(const float (&w1)[3], float b1, const float (&Td)[3],
-                                            bool sd1, const PRec& pa, const PRec& pb, float (&oA)[8],
-                                            float (&oB)[8]) {
+                                            bool sd1, const PRec& pa, const PRec& pb,
+                                            F2 (&o)[8]) {
   const F2 W0 = f2s(w1[0]), W1 = f2s(w1[1]), W2 = f2s(w1[2]), B1 = f2s(b1);
   float zA, zB;
   f2get(fma2(W0, f2(pa.x, pb.x), fma2(W1, f2(pa.y, pb.y), fma2(W2, f2(pa.z, pb.z), B1))), zA, zB);
@@ -163,7 +134,7 @@ __device__ __forceinline__ void layer1_pair(const float (&w1)[3], float b1, cons
   const F2 SW = fma2(NT, T, f2s(1.0f));
   const F2 NTT = mul2(NT, T);
   const F2 NTS = mul2(NT, SW);
-  f2get(T, oA[0], oB[0]);
+  o[0] = T;
 #pragma unroll
   for (int i = 0; i < 3; ++i) {
     const F2 TD = f2s(Td[i]), TD2 = mul2(TD, TD);
@@ -176,12 +147,12 @@ __device__ __forceinline__ void layer1_pair(const float (&w1)[3], float b1, cons
       f2get(fma2(NTT, TD2, f2s(1.0f)), eA, eB);
       R2 = f2(rcp<FAST>(eA), rcp<FAST>(eB));
     }
-    f2get(mul2(mul2(NTS, TD2), R2), oA[1 + i], oB[1 + i]);
-    f2get(mul2(mul2(SW, TD), R2), oA[4 + i], oB[4 + i]);
+    o[1 + i] = mul2(mul2(NTS, TD2), R2);
+    o[4 + i] = mul2(mul2(SW, TD), R2);
   }
   const bool ja = pa.cutj >= 0 && (pa.cutj & 1), jb = pb.cutj >= 0 && (pb.cutj & 1);
-  oA[7] = ja ? act_tanh<FAST>(fmaf(w1[0], pa.gx, fmaf(w1[1], pa.gy, fmaf(w1[2], pa.gz, b1)))) : 0.f;
-  oB[7] = jb ? act_tanh<FAST>(fmaf(w1[0], pb.gx, fmaf(w1[1], pb.gy, fmaf(w1[2], pb.gz, b1)))) : 0.f;
+  o[7] = f2(ja ? act_tanh<FAST>(fmaf(w1[0], pa.gx, fmaf(w1[1], pa.gy, fmaf(w1[2], pa.gz, b1)))) : 0.f,
+            jb ? act_tanh<FAST>(fmaf(w1[0], pb.gx, fmaf(w1[1], pb.gy, fmaf(w1[2], pb.gz, b1)))) : 0.f);
 }
 
 // tanh(h W1[u][i]) of the first layer (it depends on the unit only); sd1: every
@@ -198,57 +169,57 @@ __device__ __forceinline__ void layer1_increments(const float (&w1)[3], float h,
   for (int i = 0; i < 3; ++i) Td[i] = sd1 ? tanh_small(d[i]) : act_tanh<FAST>(d[i]);
 }
 
-// A hidden layer's outputs of two points in one unit from the GEMM's columns cA, cB
+// A hidden layer's outputs of two points in one unit from the GEMM's 16 columns z
 // and the bias.  Column 7 (the interface point) only matters for cut cells with a
 // jump row; elsewhere its seeds are 0.  The accurate path skips its tanh there (0,
 // as layer 1 leaves it); in the SFU path the test cost more than it saved (C2 6 %
 // slower), so that path keeps computing it.
 template <bool FAST>
-__device__ __forceinline__ void hidden_pair(const float* cA, const float* cB, float bb,
-                                            const PRec* pa, const PRec* pb, float (&oA)[8],
-                                            float (&oB)[8]) {
+__device__ __forceinline__ void hidden_pair(const float* z, float bb, const PRec* pa,
+                                            const PRec* pb, F2 (&o)[8]) {
   constexpr float kSmall = FAST ? kSmallMu : kSmallMuAccurate;
-  const float tA = act_tanh<FAST>(cA[0] + bb), tB = act_tanh<FAST>(cB[0] + bb);
-  oA[0] = tA;
-  oB[0] = tB;
+  const F2 BB = f2s(bb);
+  float zA, zB;
+  f2get(add2(f2(z[0], z[1]), BB), zA, zB);
+  const float tA = act_tanh<FAST>(zA), tB = act_tanh<FAST>(zB);
+  const F2 T = f2(tA, tB);
+  o[0] = T;
   const bool smA = __all_sync(0xffffffffu,
-                              fmaxf(fabsf(cA[1]), fmaxf(fabsf(cA[2]), fabsf(cA[3]))) <= kSmall);
+                              fmaxf(fabsf(z[2]), fmaxf(fabsf(z[4]), fabsf(z[6]))) <= kSmall);
   const bool smB = __all_sync(0xffffffffu,
-                              fmaxf(fabsf(cB[1]), fmaxf(fabsf(cB[2]), fabsf(cB[3]))) <= kSmall);
+                              fmaxf(fabsf(z[3]), fmaxf(fabsf(z[5]), fabsf(z[7]))) <= kSmall);
   // accurate path: antisymmetric increments small in every lane (their series)
   bool sdA = false, sdB = false;
   if constexpr (!FAST) {
-    sdA = __all_sync(0xffffffffu, fmaxf(fabsf(cA[4]), fmaxf(fabsf(cA[5]), fabsf(cA[6]))) <=
+    sdA = __all_sync(0xffffffffu, fmaxf(fabsf(z[8]), fmaxf(fabsf(z[10]), fabsf(z[12]))) <=
                                       kSmallDelAccurate);
-    sdB = __all_sync(0xffffffffu, fmaxf(fabsf(cB[4]), fmaxf(fabsf(cB[5]), fabsf(cB[6]))) <=
+    sdB = __all_sync(0xffffffffu, fmaxf(fabsf(z[9]), fmaxf(fabsf(z[11]), fabsf(z[13]))) <=
                                       kSmallDelAccurate);
   }
   if (smA && smB) {
-    const F2 T = f2(tA, tB), NT = mul2(T, f2s(-1.0f));
+    const F2 NT = mul2(T, f2s(-1.0f));
     const F2 S0 = fma2(NT, T, f2s(1.0f));
 #pragma unroll
-    for (int i = 0; i < 3; ++i) {
-      F2 M, D;
-      tanh_stencil_fwd_pair<FAST>(T, NT, S0, f2(cA[1 + i], cB[1 + i]), f2(cA[4 + i], cB[4 + i]), M,
-                                  D, sdA && sdB);
-      f2get(M, oA[1 + i], oB[1 + i]);
-      f2get(D, oA[4 + i], oB[4 + i]);
-    }
+    for (int i = 0; i < 3; ++i)
+      tanh_stencil_fwd_pair<FAST>(T, NT, S0, f2(z[2 + 2 * i], z[3 + 2 * i]),
+                                  f2(z[8 + 2 * i], z[9 + 2 * i]), o[1 + i], o[4 + i], sdA && sdB);
   } else {
 #pragma unroll
     for (int i = 0; i < 3; ++i) {
-      tanh_stencil_fwd<FAST>(tA, cA[1 + i], cA[4 + i], 1.f, 1.f, 1.f, 1.f, oA[1 + i], oA[4 + i],
-                             smA, sdA);
-      tanh_stencil_fwd<FAST>(tB, cB[1 + i], cB[4 + i], 1.f, 1.f, 1.f, 1.f, oB[1 + i], oB[4 + i],
-                             smB, sdB);
+      float mA, dA, mB, dB;
+      tanh_stencil_fwd<FAST>(tA, z[2 + 2 * i], z[8 + 2 * i], 1.f, 1.f, 1.f, 1.f, mA, dA, smA, sdA);
+      tanh_stencil_fwd<FAST>(tB, z[3 + 2 * i], z[9 + 2 * i], 1.f, 1.f, 1.f, 1.f, mB, dB, smB, sdB);
+      o[1 + i] = f2(mA, mB);
+      o[4 + i] = f2(dA, dB);
     }
   }
+  float gA, gB;
+  f2get(add2(f2(z[14], z[15]), BB), gA, gB);
   if constexpr (FAST) {
-    oA[7] = act_tanh<FAST>(cA[7] + bb);
-    oB[7] = act_tanh<FAST>(cB[7] + bb);
+    o[7] = f2(act_tanh<FAST>(gA), act_tanh<FAST>(gB));
   } else {
-    oA[7] = (pa->cutj >= 0 && (pa->cutj & 1)) ? act_tanh<FAST>(cA[7] + bb) : 0.f;
-    oB[7] = (pb->cutj >= 0 && (pb->cutj & 1)) ? act_tanh<FAST>(cB[7] + bb) : 0.f;
+    o[7] = f2((pa->cutj >= 0 && (pa->cutj & 1)) ? act_tanh<FAST>(gA) : 0.f,
+              (pb->cutj >= 0 && (pb->cutj & 1)) ? act_tanh<FAST>(gB) : 0.f);
   }
 }
 

@@ -115,7 +115,7 @@ __global__ void __launch_bounds__(kEvalThreads, 1) k_eval_tc(ProbDev P, const fl
                                                     int* status) {
   constexpr int H = 128, NG = L - 1, kTP = 64, kImgG = 16384, kX = kEvalTiles;
   extern __shared__ unsigned char smem_raw[];
-  unsigned char* sm = (unsigned char*)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
+  unsigned char* sm = align1024(smem_raw);
   const int tid = threadIdx.x, w = tid >> 5, lane = tid & 31;
   const bool issuer = w >= 16;
   const int grp = issuer ? w - 16 : tid >> 8, gtid = tid & 255, gw = gtid >> 5;
@@ -136,6 +136,8 @@ __global__ void __launch_bounds__(kEvalThreads, 1) k_eval_tc(ProbDev P, const fl
   int* flag = (int*)(misc + kFlag) + grp * kX * kTP;           // [kX][64]
 
   const uint32_t idf = idesc_f16_n(BF, false, true, kTP);
+  // the 16-byte chunk c8 of this thread's row and columns: off0 ^ 16 c8
+  const uint32_t off0 = img_off(u, col0);
   if (tid == 0) {
     mbar_init(smem_u32(bar_w), 1);
     for (int b = 0; b < 2 * kX; ++b) {
@@ -346,7 +348,7 @@ __global__ void __launch_bounds__(kEvalThreads, 1) k_eval_tc(ProbDev P, const fl
             z[4 * h4 + 2] = fmaf(w10, px.z, fmaf(w11, py.z, fmaf(w12, pz.z, b1)));
             z[4 * h4 + 3] = fmaf(w10, px.w, fmaf(w11, py.w, fmaf(w12, pz.w, b1)));
           }
-          *reinterpret_cast<uint4*>(dst + img_off(u, col0 + 8 * c8)) =
+          *reinterpret_cast<uint4*>(dst + (off0 ^ (uint32_t)(c8 << 4))) =
               make_uint4(tanh_pack2<BF>(z[0], z[1]), tanh_pack2<BF>(z[2], z[3]),
                          tanh_pack2<BF>(z[4], z[5]), tanh_pack2<BF>(z[6], z[7]));
         }
@@ -375,7 +377,7 @@ __global__ void __launch_bounds__(kEvalThreads, 1) k_eval_tc(ProbDev P, const fl
 #pragma unroll
               for (int i = 0; i < 8; i += 2)
                 f2get(add2(f2(acc[8 * c8 + i], acc[8 * c8 + i + 1]), BB), z[i], z[i + 1]);
-              *reinterpret_cast<uint4*>(dst + img_off(u, col0 + 8 * c8)) =
+              *reinterpret_cast<uint4*>(dst + (off0 ^ (uint32_t)(c8 << 4))) =
                   make_uint4(tanh_pack2<BF>(z[0], z[1]), tanh_pack2<BF>(z[2], z[3]),
                              tanh_pack2<BF>(z[4], z[5]), tanh_pack2<BF>(z[6], z[7]));
             }

@@ -75,7 +75,7 @@ __global__ void __launch_bounds__(512, 1) k_step_tc(ProbDev P, StepArgs a) {
   // the 32 KB weight read from shared memory.
   constexpr bool kWTmem = NG == 2;
   extern __shared__ unsigned char smem_raw[];
-  unsigned char* sm = (unsigned char*)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
+  unsigned char* sm = align1024(smem_raw);
   const int tid = threadIdx.x, w = tid >> 5, lane = tid & 31;
   const int grp = tid >> 8, gtid = tid & 255;  // warp group and rank in it
   const int q = w & 3, cgl = (w >> 2) & 1;     // TMEM lane quadrant, column group
@@ -98,10 +98,10 @@ __global__ void __launch_bounds__(512, 1) k_step_tc(ProbDev P, StepArgs a) {
   float* red = (float*)(Aimg + (L - 1) * kImgH);     // [4][64] scratch (forward end only)
 
   // image byte offset of (unit u, point 4cgl + j): the row part is fixed per
-  // thread, the 16-byte chunk is ((4cgl + j) mod 8) xor (u mod 8)
-  const uint32_t row_off = (uint32_t)((u >> 3) * 1024 + (u & 7) * 128);
-  const uint32_t pbase = (uint32_t)(cgl << 2), uxor = (uint32_t)(u & 7);
-  auto poff = [&](int j) -> uint32_t { return row_off + ((((pbase + j) ^ uxor) & 7u) << 4); };
+  // thread, the 16-byte chunk is (4cgl + j) xor u, mod 8 (the
+  // chunks of j = 0 .. 3 differ by an xor)
+  const uint32_t off0 = (uint32_t)((u >> 3) * 1024 + (u & 7) * 128 + ((((cgl << 2) ^ u) & 7) << 4));
+  auto poff = [&](int j) -> uint32_t { return off0 ^ (uint32_t)(j << 4); };
   const uint32_t id_fwd = idesc_f16_n(true, false, true, kHP * 8);
   const uint32_t id_dgr = idesc_f16_n(true, true, true, kHP * 8);
   const uint32_t id_wgr = idesc_f16_n(true, false, false, 128);

@@ -45,7 +45,7 @@ __global__ void __launch_bounds__(kFwdT, 1) k_fwd_tc(ProbDev P, StepArgs a) {
   constexpr uint32_t NCOLS = 512, kWCol = 2 * kX * 64;  // TMEM columns; the first past the D's
   constexpr int kWT = NG < 2 ? NG : 2;                  // layers with their weights in TMEM
   extern __shared__ unsigned char smem_raw[];
-  unsigned char* sm = (unsigned char*)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
+  unsigned char* sm = align1024(smem_raw);
   const int tid = threadIdx.x, w = tid >> 5, lane = tid & 31;
   const bool issuer = w >= 16;
   const int grp = issuer ? w - 16 : tid >> 8, gtid = tid & 255;
@@ -63,9 +63,9 @@ __global__ void __launch_bounds__(kFwdT, 1) k_fwd_tc(ProbDev P, StepArgs a) {
   double* loss_red = (double*)(misc + kLossRed);                 // [16]
   float* red = (float*)(misc + kRed) + grp * kX * 4 * 64;        // [kX][4][64]
   PRec* pbuf = (PRec*)(misc + kPbuf) + grp * 2 * kX * kHP;       // [2][kX][8]
-  const uint32_t row_off = (uint32_t)((u >> 3) * 1024 + (u & 7) * 128);
-  const uint32_t pbase = (uint32_t)(cgl << 2), uxor = (uint32_t)(u & 7);
-  auto poff = [&](int j) -> uint32_t { return row_off + ((((pbase + j) ^ uxor) & 7u) << 4); };
+  // (point chunk j of this thread's row: the swizzled 16-byte chunks differ by an xor)
+  const uint32_t off0 = (uint32_t)((u >> 3) * 1024 + (u & 7) * 128 + ((((cgl << 2) ^ u) & 7) << 4));
+  auto poff = [&](int j) -> uint32_t { return off0 ^ (uint32_t)(j << 4); };
   const uint32_t idf = idesc_f16_n(true, false, true, kHP * 8);
 
   if (tid == 0) {

@@ -21,6 +21,14 @@ __device__ __forceinline__ uint32_t smem_u32(const void* p) {
   return (uint32_t)__cvta_generic_to_shared(p);
 }
 
+// First 1024-byte boundary of a dynamic shared array.  By pointer arithmetic: through
+// an integer and back the compiler loses the shared address space, and every access
+// becomes a generic one with 64-bit addresses (training step C2 2007 -> 1905 us per two
+// steps, four layers 6.48 -> 6.10 ms, 513^3 evaluation 29.9 -> 28.3 ms without that).
+__device__ __forceinline__ unsigned char* align1024(unsigned char* p) {
+  return p + ((0u - smem_u32(p)) & 1023u);
+}
+
 // byte offset of element (row, col) in the swizzled 128x128 image
 __host__ __device__ __forceinline__ uint32_t img_off(int row, int col) {
   const int cb = col >> 6, cc = col & 63;

@@ -86,7 +86,7 @@ __device__ __forceinline__ void warp_transpose_reduce32(const float (&x)[32], fl
 
 // Two points' tanh stencil layer on packed FP32 pairs (unscaled columns, every
 // lane's symmetric increments small): the arithmetic of tanh_stencil_fwd's
-// series path, operation for operation.
+// series path.
 template <bool FAST>
 __device__ __forceinline__ void tanh_stencil_fwd_pair(F2 T, F2 NT, F2 S0, F2 MU, F2 DE, F2& M,
                                                       F2& D, bool small_de = false) {
@@ -106,17 +106,18 @@ __device__ __forceinline__ void tanh_stencil_fwd_pair(F2 T, F2 NT, F2 S0, F2 MU,
   const F2 ntw = mul2(tw, f2s(-1.0f));
   const F2 sw = fma2(ntw, tw, f2s(1.0f));
   const F2 td2 = mul2(TD, TD);
+  const F2 ntd = mul2(ntw, td2);
   F2 r2;
   if (sde) {
     const F2 x = mul2(mul2(tw, tw), td2);  // 1/(1-x) = 1 + x (1 + x (1 + x))
     r2 = fma2(x, fma2(x, add2(x, f2s(1.0f)), f2s(1.0f)), f2s(1.0f));
   } else {
     float eA, eB;
-    f2get(fma2(add2(sw, f2s(-1.0f)), td2, f2s(1.0f)), eA, eB);
+    f2get(fma2(ntd, tw, f2s(1.0f)), eA, eB);  // 1 - tw^2 Td^2
     r2 = f2(rcp<FAST>(eA), rcp<FAST>(eB));
   }
   const F2 k = mul2(sw, r2);
-  M = fma2(mul2(ntw, td2), k, dm);
+  M = fma2(ntd, k, dm);
   D = mul2(k, TD);
 }
 
@@ -184,33 +185,37 @@ __device__ __forceinline__ void hidden_pair(const float* z, float bb, const PRec
   const float tA = act_tanh<FAST>(zA), tB = act_tanh<FAST>(zB);
   const F2 T = f2(tA, tB);
   o[0] = T;
-  const bool smA = __all_sync(0xffffffffu,
-                              fmaxf(fabsf(z[2]), fmaxf(fabsf(z[4]), fabsf(z[6]))) <= kSmall);
-  const bool smB = __all_sync(0xffffffffu,
-                              fmaxf(fabsf(z[3]), fmaxf(fabsf(z[5]), fabsf(z[7]))) <= kSmall);
-  // accurate path: antisymmetric increments small in every lane (their series)
-  bool sdA = false, sdB = false;
+  // small increments of both points in every lane: the series (symmetric; accurate
+  // path: antisymmetric too)
+  const float mA = fmaxf(fabsf(z[2]), fmaxf(fabsf(z[4]), fabsf(z[6])));
+  const float mB = fmaxf(fabsf(z[3]), fmaxf(fabsf(z[5]), fabsf(z[7])));
+  const bool sm = __all_sync(0xffffffffu, fmaxf(mA, mB) <= kSmall);
+  float dA = 0.f, dB = 0.f;
+  bool sd = false;
   if constexpr (!FAST) {
-    sdA = __all_sync(0xffffffffu, fmaxf(fabsf(z[8]), fmaxf(fabsf(z[10]), fabsf(z[12]))) <=
-                                      kSmallDelAccurate);
-    sdB = __all_sync(0xffffffffu, fmaxf(fabsf(z[9]), fmaxf(fabsf(z[11]), fabsf(z[13]))) <=
-                                      kSmallDelAccurate);
+    dA = fmaxf(fabsf(z[8]), fmaxf(fabsf(z[10]), fabsf(z[12])));
+    dB = fmaxf(fabsf(z[9]), fmaxf(fabsf(z[11]), fabsf(z[13])));
+    sd = __all_sync(0xffffffffu, fmaxf(dA, dB) <= kSmallDelAccurate);
   }
-  if (smA && smB) {
+  if (sm) {
     const F2 NT = mul2(T, f2s(-1.0f));
     const F2 S0 = fma2(NT, T, f2s(1.0f));
 #pragma unroll
     for (int i = 0; i < 3; ++i)
       tanh_stencil_fwd_pair<FAST>(T, NT, S0, f2(z[2 + 2 * i], z[3 + 2 * i]),
-                                  f2(z[8 + 2 * i], z[9 + 2 * i]), o[1 + i], o[4 + i], sdA && sdB);
+                                  f2(z[8 + 2 * i], z[9 + 2 * i]), o[1 + i], o[4 + i], sd);
   } else {
+    const bool smA = __all_sync(0xffffffffu, mA <= kSmall);
+    const bool smB = __all_sync(0xffffffffu, mB <= kSmall);
+    const bool sdA = !FAST && __all_sync(0xffffffffu, dA <= kSmallDelAccurate);
+    const bool sdB = !FAST && __all_sync(0xffffffffu, dB <= kSmallDelAccurate);
 #pragma unroll
     for (int i = 0; i < 3; ++i) {
-      float mA, dA, mB, dB;
-      tanh_stencil_fwd<FAST>(tA, z[2 + 2 * i], z[8 + 2 * i], 1.f, 1.f, 1.f, 1.f, mA, dA, smA, sdA);
-      tanh_stencil_fwd<FAST>(tB, z[3 + 2 * i], z[9 + 2 * i], 1.f, 1.f, 1.f, 1.f, mB, dB, smB, sdB);
-      o[1 + i] = f2(mA, mB);
-      o[4 + i] = f2(dA, dB);
+      float m0, d0, m1, d1;
+      tanh_stencil_fwd<FAST>(tA, z[2 + 2 * i], z[8 + 2 * i], 1.f, 1.f, 1.f, 1.f, m0, d0, smA, sdA);
+      tanh_stencil_fwd<FAST>(tB, z[3 + 2 * i], z[9 + 2 * i], 1.f, 1.f, 1.f, 1.f, m1, d1, smB, sdB);
+      o[1 + i] = f2(m0, m1);
+      o[4 + i] = f2(d0, d1);
     }
   }
   float gA, gB;

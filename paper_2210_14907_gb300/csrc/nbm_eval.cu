@@ -187,12 +187,14 @@ __global__ void __launch_bounds__(kEvalThreads, 1) k_eval_tc(ProbDev P, const fl
           const uint32_t wt = tmem + kWCol + 64u * (uint32_t)g;
 #pragma unroll
           for (int k = 0; k < 8; ++k)
-            mma_f16_ta(d_tm + kTP * X, wt + 8u * (uint32_t)k, desc_mnmajor(ab, k), idf, k > 0);
+            mma_f16_ta(d_tm + kTP * X, wt + 8u * (uint32_t)k, desc_mnmajor(ab) + kstep_mnmajor(k),
+                       idf, k > 0);
         } else {
           const uint32_t wa = smem_u32(Wimg + g * kImgE);
 #pragma unroll
           for (int k = 0; k < 8; ++k)
-            mma_f16(d_tm + kTP * X, desc_kmajor(wa, k), desc_mnmajor(ab, k), idf, k > 0);
+            mma_f16(d_tm + kTP * X, desc_kmajor(wa) + kstep_kmajor(k),
+                    desc_mnmajor(ab) + kstep_mnmajor(k), idf, k > 0);
         }
         mma_commit(smem_u32(bar_mma + X));
       }

@@ -362,12 +362,14 @@ __global__ void __launch_bounds__(512, 1) k_step_tc(ProbDev P, StepArgs a) {
             const uint32_t wt = tmem + 384u + 64u * (uint32_t)(g - 1);
 #pragma unroll
             for (int k = 0; k < 8; ++k)
-              mma_f16_ta(d_tm, wt + 8u * (uint32_t)k, desc_mnmajor(ab, k), id_fwd, k > 0);
+              mma_f16_ta(d_tm, wt + 8u * (uint32_t)k, desc_mnmajor(ab) + kstep_mnmajor(k), id_fwd,
+                         k > 0);
           } else {
             const uint32_t wa = smem_u32(Wimg + (g - 1) * kImg);
 #pragma unroll
             for (int k = 0; k < 8; ++k)
-              mma_f16(d_tm, desc_kmajor(wa, k), desc_mnmajor(ab, k), id_fwd, k > 0);
+              mma_f16(d_tm, desc_kmajor(wa) + kstep_kmajor(k), desc_mnmajor(ab) + kstep_mnmajor(k),
+                      id_fwd, k > 0);
           }
           mma_commit(smem_u32(bar_mma));
         }
@@ -516,10 +518,12 @@ __global__ void __launch_bounds__(512, 1) k_step_tc(ProbDev P, StepArgs a) {
           const uint32_t ain = smem_u32(Aimg + (g - 1) * kImgH);  // act[g-1]
 #pragma unroll
           for (int k = 0; k < 8; ++k)  // input gradient: D = W^T gz
-            mma_f16(d_tm, desc_mnmajor(wa, k), desc_mnmajor(gzb, k), id_dgr, k > 0);
+            mma_f16(d_tm, desc_mnmajor(wa) + kstep_mnmajor(k), desc_mnmajor(gzb) + kstep_mnmajor(k),
+                    id_dgr, k > 0);
 #pragma unroll
           for (int k = 0; k < kHP / 2; ++k)  // weight gradient: Wacc += gz act^T (K = 8 kHP)
-            mma_f16(tmem + 128u * g, desc_kmajor(gzb, k), desc_kmajor(ain, k), id_wgr,
+            mma_f16(tmem + 128u * g, desc_kmajor(gzb) + kstep_kmajor(k),
+                    desc_kmajor(ain) + kstep_kmajor(k), id_wgr,
                     (k > 0 || acc_w) ? 1u : 0u);
           mma_commit(smem_u32(bar_mma));
         }

@@ -131,12 +131,14 @@ __global__ void __launch_bounds__(kFwdT, 1) k_fwd_tc(ProbDev P, StepArgs a) {
           const uint32_t wt = tmem + kWCol + 64u * (uint32_t)g;
 #pragma unroll
           for (int k = 0; k < 8; ++k)
-            mma_f16_ta(d_tm + 64 * X, wt + 8u * (uint32_t)k, desc_mnmajor(ab, k), idf, k > 0);
+            mma_f16_ta(d_tm + 64 * X, wt + 8u * (uint32_t)k, desc_mnmajor(ab) + kstep_mnmajor(k), idf,
+                       k > 0);
         } else {
           const uint32_t wa = smem_u32(Wimg + g * kImg);
 #pragma unroll
           for (int k = 0; k < 8; ++k)
-            mma_f16(d_tm + 64 * X, desc_kmajor(wa, k), desc_mnmajor(ab, k), idf, k > 0);
+            mma_f16(d_tm + 64 * X, desc_kmajor(wa) + kstep_kmajor(k),
+                    desc_mnmajor(ab) + kstep_mnmajor(k), idf, k > 0);
         }
         mma_commit(smem_u32(bar_mma + X));
       }

@@ -100,7 +100,10 @@ __device__ __forceinline__ uint32_t tanh_pack2(float a, float b) {
 // written its part of a tile's image arrives on the tile's `ready` barrier and goes
 // on to the next tile, whose accumulators it waits for by itself; the issuing
 // warp waits for all 8 arrivals.  So the warps of a group meet only at the ends of
-// a set, not after every tile and layer, and run up to a tile apart.
+// a set, not after every tile and layer, and run up to a tile apart.  513^3 nodes,
+// 3 -> 128 x 4 -> 1, FP16: 37.0 ms with a group barrier per tile and layer, 29.9 with
+// the issuing warps, 27.6 with shared-space addresses and descriptors by addition
+// (480 TFLOP/s; the 69 G tanh, two to an instruction, are 7 ms of the SFUs).
 //
 // Pass 0 (the minus network) decides every point's side and keeps it in
 // `side` (per 128 points, bit c: point c is in Omega-; each 64-point tile owns

@@ -1,5 +1,6 @@
-// nbm_tc.cu -- the mixed-precision fused NBM step on the 5th-generation tensor
-// cores (tcgen05, TMEM accumulators), arXiv 2210.14907 Sec. 3 / Fig. 2.
+// nbm_tc.cu -- the mixed-precision fused NBM training step on the 5th-generation
+// tensor cores (tcgen05, TMEM accumulators), arXiv 2210.14907 Sec. 3 / Fig. 2.
+// (The forward-only passes are nbm_tc_fwd.cu's.)
 //
 // One persistent CTA per SM, 16 warps in two groups of 8.  Each group owns a
 // half-tile: 8 collocation points x 8 columns (centre value, symmetric and
@@ -8,20 +9,28 @@
 // operand images and its own 64 TMEM accumulator columns.  The groups run
 // independently, so that one group's epilogue (CUDA cores) overlaps the other
 // group's GEMMs (tensor pipe).  Every hidden layer is one 128 x 64 x 128
-// product D[unit][col] = W[unit][k] A[k][col] with 16-bit operands and FP32
+// product D[unit][col] = W[unit][k] A[k][col] with BF16 operands and FP32
 // accumulation in TMEM; warp w reads TMEM lanes 32(w%4).. (one unit per
 // thread) for 32 columns (4 points).  The epilogue applies the tanh stencil
-// layer in FP32 and writes the next 16-bit operand image to shared memory.
+// layer in FP32 and writes the next BF16 operand image to shared memory.
 // The first layer (K = 3), the output layer (H -> 1, a warp
 // transpose-reduction), the residual rows and the seeds stay FP32 (FP64 rows
-// on request).  In the BF16 training path the epilogues' FP32 arithmetic runs
-// on packed pairs (add/mul/fma .f32x2: two points per instruction, each
-// rounded as its scalar form).  The backward reuses the stored images: per hidden layer one
+// on request).  The epilogues' FP32 arithmetic runs on packed pairs
+// (add/mul/fma .f32x2: two points per instruction, each rounded as its scalar
+// form).  The backward reuses the stored images: per hidden layer one
 // input-gradient MMA (W^T gz, into the group's D columns) and one
 // weight-gradient MMA (gz A^T, K = 64) accumulated across all half-tiles of
 // the CTA in shared TMEM columns, in a fixed order of the half-tiles, so the
 // weight gradient never leaves the SM until the CTA's partial is written once
 // per network and is bitwise reproducible.
+//
+// Bound: instruction issue in the epilogues and the GEMM latency of a group's
+// phases that the other group does not fill.  262,144 points, 3 -> 128 x 3 -> 1: a step
+// took 1.080 ms with 601 M warp instructions and takes 0.932 with 467 M (issue slots
+// busy 45 %, tensor pipe 19 %); what was taken out were the moves that put points'
+// columns together into pairs (they are interleaved in the images now), generic
+// addresses, votes per point and the descriptors' arithmetic.  Two groups of 8 warps
+// are what 120 registers a thread leave room for.
 //
 // Shared memory: (L-1) weight images of 32 KB + 2 x L operand images of 16 KB.
 // TMEM: 2 x 64 columns for D + 128 per hidden layer for the weight gradient.

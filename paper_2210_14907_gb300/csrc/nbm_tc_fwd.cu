@@ -15,7 +15,7 @@
 // three half-tiles, before the rows.
 // The training kernel ran these passes with one half-tile per group in flight and
 // every GEMM exposed to its group: a residual call of 50,001 points, 3 -> 128 x 3 -> 1,
-// over four spacings took 874 us and takes 694 with this kernel.
+// over four spacings took 874 us and takes 636 with this kernel.
 #include "nbm_device.cuh"
 #include "nbm_tc_layer.cuh"
 #include "nbm_tc_ptx.cuh"

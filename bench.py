@@ -45,14 +45,14 @@ BATCH = 262_144
 # of that kernel on this workload, with the SHA-256 (first 16 hex digits) of
 # the kernel's sources at the time of the capture.  The bench line reports the
 # figure only while the sources still hash to that value (else null).
-FUSED_TRAFFIC = {"bytes": 8_957_952, "sources_sha16": "b819b011302ab88b"}
-FUSED_SOURCES = ("paper_2210_14907_gb300/csrc/nbm_tc.cu", "paper_2210_14907_gb300/csrc/nbm_tc_ptx.cuh",
-                 "paper_2210_14907_gb300/csrc/nbm_device.cuh")
+FUSED_TRAFFIC = {"bytes": 9_036_800, "sources_sha16": "48a8b9e994804bc6"}
+FUSED_SOURCES = ("paper_2210_14907_gb300/csrc/nbm_tc.cu", "paper_2210_14907_gb300/csrc/nbm_tc_layer.cuh",
+                 "paper_2210_14907_gb300/csrc/nbm_tc_ptx.cuh", "paper_2210_14907_gb300/csrc/nbm_device.cuh")
 # libnbm kernel launches per timed step.  One nbm_train_steps call of one C2
 # step: k_sample_classify (its extra blocks restage the weights), k_scatter
 # (up to 2048 blocks of points it also does the block-count scan, so no
 # k_scan_counts; it writes the uncut points' tile records); k_cut_geometry
-# (the cut cells' records); k_step_tc (cut-cell forward), k_cut_residual;
+# (the cut cells' records); k_fwd_tc (cut-cell forward), k_cut_residual;
 # k_step_tc (fused train step); k_reduce_adam (loss, gradient, update).  The
 # data-parallel step (N > 1) runs the same chain through nbm_loss_grad_shard
 # (k_reduce_adam writes the loss and gradient only) and then k_adam: one more.

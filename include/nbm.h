@@ -259,8 +259,8 @@ int nbm_train_steps(nbm_problem* p, float* params, float* adam_m, float* adam_v,
  * `precision` selects the hidden-GEMM type (nbm_precision): NBM_PREC_FP32
  * (CUDA cores; asynchronous), or NBM_PREC_BF16 / NBM_PREC_FP16 (tensor cores;
  * width 128 and 2..4 hidden layers only; these keep their scratch with the
- * problem -- the sides of more than 2^29 points or so are allocated for the
- * call -- and synchronize the stream).
+ * problem -- a call of more than 2^29 points or so allocates its own, and so
+ * does one beside another thread's -- and synchronize the stream).
  * Returns NBM_ERR_INVALID_ARG for a NULL or misaligned argument, n outside
  * 1..4096 or an unsupported precision, NBM_ERR_OOM if the scratch cannot be
  * allocated, NBM_ERR_DEVICE_TIMEOUT if a bounded device wait gave up. */

@@ -839,28 +839,31 @@ static int eval_common(nbm_problem* p, const float* params, int n, const float* 
     else e = cudaErrorInvalidValue;
   } else {
     // The scratch stays with the problem: three allocations and frees per call cost
-    // 160 us of the 220 that a call with a few points took.  The sides of very many
-    // points (over kKeepSideBytes, 537 M points) are allocated for the call.
+    // 160 us of the 220 that a call with a few points took.  A call has its own when
+    // another thread's evaluation uses the kept one, on another device, and for the
+    // sides of very many points (over kKeepSideBytes, 537 M points).
     const size_t bytes = (size_t)2 * (d.n_hidden - 1) * kImgE;
     const int64_t total = pts ? npts : (int64_t)(n + 1) * (n + 1) * (n + 1);
     const int64_t side_n = (total + 127) / 128;
-    EvalScratch& ev = problem_eval_scratch(p);
-    if (!ev.wimg) e = cudaMalloc((void**)&ev.wimg, bytes);
+    EvalScratch& held = problem_eval_scratch(p);
+    std::unique_lock<std::mutex> lock(held.mu, std::try_to_lock);
+    int dev = 0;
+    e = cudaGetDevice(&dev);
+    const bool kept = lock.owns_lock() && (held.device < 0 || held.device == dev) &&
+                      sizeof(uint4) * (size_t)side_n <= kKeepSideBytes;
+    EvalScratch own;
+    EvalScratch& ev = kept ? held : own;
+    ev.device = dev;
+    if (e == cudaSuccess && !ev.wimg) e = cudaMalloc((void**)&ev.wimg, bytes);
     if (e == cudaSuccess && !ev.status) e = cudaMalloc((void**)&ev.status, sizeof(int));
-    uint4* side = nullptr;  // per 128-point tile: bit c set if point c is in Omega-
-    const bool own_side = sizeof(uint4) * (size_t)side_n > kKeepSideBytes;
-    if (e == cudaSuccess && own_side) {
-      e = cudaMalloc((void**)&side, sizeof(uint4) * (size_t)side_n);
-    } else if (e == cudaSuccess) {
-      if (ev.side_cap < side_n) {
-        if (ev.side) cudaFree(ev.side);
-        ev.side = nullptr;
-        ev.side_cap = 0;
-        e = cudaMalloc((void**)&ev.side, sizeof(uint4) * (size_t)side_n);
-        if (e == cudaSuccess) ev.side_cap = side_n;
-      }
-      side = ev.side;
+    if (e == cudaSuccess && ev.side_cap < side_n) {  // bit c of a 128-point tile: c is in Omega-
+      if (ev.side) cudaFree(ev.side);
+      ev.side = nullptr;
+      ev.side_cap = 0;
+      e = cudaMalloc((void**)&ev.side, sizeof(uint4) * (size_t)side_n);
+      if (e == cudaSuccess) ev.side_cap = side_n;
     }
+    uint4* side = ev.side;
     unsigned char* wimg = ev.wimg;
     int* status = ev.status;
     if (e == cudaSuccess) e = cudaMemsetAsync(status, 0, sizeof(int), st);
@@ -882,7 +885,8 @@ static int eval_common(nbm_problem* p, const float* params, int n, const float* 
     if (e == cudaSuccess) e = cudaMemcpyAsync(&hs, status, sizeof(int), cudaMemcpyDeviceToHost, st);
     if (e == cudaSuccess) e = cudaStreamSynchronize(st);
     else cudaStreamSynchronize(st);  // nothing of a failed call still uses the scratch
-    if (own_side && side) cudaFree(side);
+    for (void* q : {(void*)own.wimg, (void*)own.status, (void*)own.side})
+      if (q) cudaFree(q);
     if (e == cudaSuccess && (hs & 2)) {
       set_error_message("grid evaluation: a bounded device wait gave up");
       return NBM_ERR_DEVICE_TIMEOUT;

@@ -4,6 +4,7 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include <mutex>
 #include <vector>
 
 #include "nbm.h"
@@ -132,6 +133,8 @@ struct EvalScratch {
   int* status = nullptr;
   uint4* side = nullptr;          // sides of side_cap 128-point tiles
   int64_t side_cap = 0;
+  int device = -1;                // where the buffers are
+  std::mutex mu;                  // held by the call that uses them
 };
 
 struct Problem {

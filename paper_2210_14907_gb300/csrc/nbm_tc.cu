@@ -26,8 +26,8 @@
 //
 // Bound: instruction issue in the epilogues and the GEMM latency of a group's
 // phases that the other group does not fill.  262,144 points, 3 -> 128 x 3 -> 1: a step
-// took 1.080 ms with 601 M warp instructions and takes 0.932 with 467 M (issue slots
-// busy 45 %, tensor pipe 19 %); what was taken out were the moves that put points'
+// took 1.080 ms with 601 M warp instructions and takes 0.932 with 462 M (issue slots
+// busy 46 %, tensor pipe 20 %); what was taken out were the moves that put points'
 // columns together into pairs (they are interleaved in the images now), generic
 // addresses, votes per point and the descriptors' arithmetic.  Two groups of 8 warps
 // are what 120 registers a thread leave room for.

@@ -1,9 +1,10 @@
 """The tensor-core forward and evaluation kernels at the edges of their tiles: 8 points
 to a forward tile (its work items and 48-row groups, with all kinds of points mixed),
 64 and 128 points to an evaluation tile, and evaluation batches that grow, shrink and
-grow again.  Tolerances: the per-point bound of the mixed path (tests/parity.py) and its
-2e-3 norm-wise from 1000 points on; evaluation against FP32 evaluation, 2e-3 (FP16) and
-1e-2 (BF16) of the root mean square norm-wise, five times that at each point."""
+grow again, from one thread or two.  Tolerances: the per-point bound of the mixed path
+(tests/parity.py) and its 2e-3 norm-wise from 1000 points on; evaluation against FP32
+evaluation, 2e-3 (FP16) and 1e-2 (BF16) of the root mean square norm-wise, five times
+that at each point."""
 import numpy as np
 import pytest
 import torch
@@ -54,3 +55,25 @@ def test_eval_tiles_and_batches_that_grow_and_shrink(L, prec, tol, geometry):
         assert got.shape[0] == n and float(d.max()) <= 5 * tol * rms, n
         if n >= 1000:
             assert float(d.pow(2).mean().sqrt()) <= tol * rms, n
+
+
+def test_eval_from_two_threads_on_one_problem():
+    import threading
+    import paper_2210_14907_gb300 as nbm
+    prob = nbm.Problem(nbm.ProblemDesc(geometry=nbm.GEOM_SPHERE, n_hidden=3, width=128))
+    xs = [torch.from_numpy(inputs.uniform_points(n, n).astype(np.float32)).cuda() for n in (3001, 70000)]
+    ths = [torch.from_numpy(inputs.glorot_params(128, 3, seed=s, bias_scale=0.2)).cuda() for s in (1, 2)]
+    want = [prob.eval_points(t, x, precision=nbm.PREC_FP16).clone() for t, x in zip(ths, xs)]
+    bad = []
+
+    def run(t, x, w):
+        with torch.cuda.stream(torch.cuda.Stream()):
+            for _ in range(40):
+                if not torch.equal(prob.eval_points(t, x, precision=nbm.PREC_FP16), w):
+                    bad.append(1)
+
+    torch.cuda.synchronize()
+    threads = [threading.Thread(target=run, args=a) for a in zip(ths, xs, want)]
+    [t.start() for t in threads]
+    [t.join() for t in threads]
+    assert not bad

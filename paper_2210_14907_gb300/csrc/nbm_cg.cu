@@ -1086,7 +1086,8 @@ struct CgSetup {
 // SMs; a CTA's range of r and p with its neighbour rows must fit the shared memory)
 // or the device cannot hold one CTA per SM.  Where it fits it is the faster path (whole
 // solves, FP64 / refined, against three launches per iteration): 24^3 2.2 / 2.4 against
-// 2.5 / 3.2 ms, 64^3 7.2 / 7.6 against 9.2 / 9.5, 128^3 34.3 / 28.2 against 46.8 / 29.3.
+// 2.5 / 3.2 ms, 64^3 7.2 / 7.6 against 9.2 / 9.5, 128^3 34.3 / 28.2 against 46.8 / 29.3
+// (with every row assembled in full; listed rows take 2.4 ms off either side at 128^3).
 // In FP32 twice the unknowns would fit, but there the coded rows of three launches
 // win: 150^3 refined 50.8 against 43.0 ms.
 struct PersistLaunch {

@@ -14,7 +14,7 @@
 // each other's latencies.  With one point per warp (10 of 32 lanes busy),
 // block barriers in every layer and the weight gradient summed in global
 // memory tile by tile, a step of 16,384 points through 5 x 10 sine networks took
-// 229 us in this kernel, and takes 132 now (of 148 for the step, which took 270); the
+// 229 us in this kernel (the step 270; 132 now); the
 // bound now is the warps' dependency chains.
 // At the end of a network the lanes' sums are added over the warps in a fixed
 // order (deterministic).
@@ -182,53 +182,61 @@ __global__ void __launch_bounds__(small_threads(HM), 1) k_step_small(ProbDev P, 
   int wrote0 = 0, wrote1 = 0;
 
   // this CTA's partial of net `net`: the lanes' sums staged in each warp's column
-  // memory, added over warps and point slots in a fixed order
-  auto flush = [&](int net) {
+  // memory, added over the `used` warps that had tiles and their point slots in a
+  // fixed order.  At H <= 16 the sums of all layers fit at once (32 (H + 1) (L - 1) +
+  // 160 floats of 512 L + 96), else layer by layer.  Layer by layer and over all 16
+  // warps, a step of 2,293 points took 116 us (89 now), of 16,384 145 (132 now).
+  auto flush = [&](int net, int used) {
     float* gp = a.gpart + ((int64_t)blockIdx.x * 2 + net) * P.gstride;
     const int wf = small_warp_floats(L), hh = H * H;
     const int64_t oo = 4 * H + (int64_t)(L - 1) * (hh + H);
+    constexpr bool kAll = HM <= 16;
+    const int hid = kAll ? (L - 1) * (hh + H) : 0, per = hid + 5 * H;  // last staging, per point slot
+    float go = gbo;
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) go += __shfl_xor_sync(0xffffffffu, go, o);
+    if (lane == 0) gbo_red[w] = go;
 #pragma unroll
     for (int g = 0; g < kLM - 1; ++g) {
       if (g >= L - 1) break;
-      __syncthreads();
+      if (!kAll || g == 0) __syncthreads();
       if (own) {
-        float* st = wsm + pq * (hh + H);
+        float* st = kAll ? wsm + pq * per + g * (hh + H) : wsm + pq * (hh + H);
 #pragma unroll
         for (int k = 0; k < HM; ++k)
           if (k < H) st[u * H + k] = gW[g][k];
         st[hh + u] = gbh[g];
       }
-      __syncthreads();
-      for (int i = tid; i < hh + H; i += NT) {
-        float s = 0.f;
-        for (int ww = 0; ww < NW; ++ww)
-          for (int q = 0; q < ppw; ++q) s += sbuf[ww * wf + q * (hh + H) + i];
-        gp[4 * H + (int64_t)g * (hh + H) + i] = s;  // weights, then biases
+      if constexpr (!kAll) {
+        __syncthreads();
+        for (int i = tid; i < hh + H; i += NT) {
+          float s = 0.f;
+          for (int ww = 0; ww < used; ++ww)
+            for (int q = 0; q < ppw; ++q) s += sbuf[ww * wf + q * (hh + H) + i];
+          gp[4 * H + (int64_t)g * (hh + H) + i] = s;  // weights, then biases
+        }
       }
     }
-    __syncthreads();
+    if constexpr (!kAll) __syncthreads();
     if (own) {
-      float* st = wsm + pq * 5 * H;
+      float* st = wsm + pq * per + hid;
       st[3 * u] = gW1[0];
       st[3 * u + 1] = gW1[1];
       st[3 * u + 2] = gW1[2];
       st[3 * H + u] = gb1;
       st[4 * H + u] = gwo;
     }
-    float go = gbo;
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) go += __shfl_xor_sync(0xffffffffu, go, o);
-    if (lane == 0) gbo_red[w] = go;
     __syncthreads();
-    for (int i = tid; i < 5 * H; i += NT) {
+    for (int i = tid; i < per; i += NT) {
       float s = 0.f;
-      for (int ww = 0; ww < NW; ++ww)
-        for (int q = 0; q < ppw; ++q) s += sbuf[ww * wf + q * 5 * H + i];
-      gp[i < 4 * H ? i : oo + i - 4 * H] = s;
+      for (int ww = 0; ww < used; ++ww)
+        for (int q = 0; q < ppw; ++q) s += sbuf[ww * wf + q * per + i];
+      const int r = i - hid;  // hidden layers' weights and biases, then layer 1 and the output
+      gp[r < 0 ? 4 * H + i : r < 4 * H ? r : oo + r - 4 * H] = s;
     }
-    if (tid == 0) {
+    if (tid == NT - 1) {
       float s = 0.f;
-      for (int ww = 0; ww < NW; ++ww) s += gbo_red[ww];
+      for (int ww = 0; ww < used; ++ww) s += gbo_red[ww];
       gp[oo + H] = s;
     }
     gW1[0] = gW1[1] = gW1[2] = gb1 = gwo = gbo = 0.f;
@@ -460,7 +468,7 @@ __global__ void __launch_bounds__(small_threads(HM), 1) k_step_small(ProbDev P, 
         gb1 += gzv[0] + gzv[7];
       }
     }
-    if (train) flush(net);
+    if (train) flush(net, (int)(s1 - s0 < NW ? s1 - s0 : NW));
     else __syncthreads();  // before the next network's weights
   }
   // loss partial of this CTA (fixed order)

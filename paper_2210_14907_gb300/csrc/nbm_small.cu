@@ -14,7 +14,7 @@
 // each other's latencies.  With one point per warp (10 of 32 lanes busy),
 // block barriers in every layer and the weight gradient summed in global
 // memory tile by tile, a step of 16,384 points through 5 x 10 sine networks took
-// 229 us in this kernel (the step 270; 132 now); the
+// 229 us in this kernel (the step 270; 123 now); the
 // bound now is the warps' dependency chains.
 // At the end of a network the lanes' sums are added over the warps in a fixed
 // order (deterministic).
@@ -165,8 +165,16 @@ __global__ void __launch_bounds__(small_threads(HM), 1) k_step_small(ProbDev P, 
   const bool cutfwd = a.mode == MODE_CUT_FWD, train = a.mode == MODE_TRAIN;
   const int64_t T0 = ((cutfwd ? nc : nm) + ppw - 1) / ppw;
   const int64_t T = cutfwd ? 2 * T0 : T0 + (np + ppw - 1) / ppw;
-  const int64_t tb = (int64_t)blockIdx.x * T / gridDim.x;
-  const int64_t te = (int64_t)(blockIdx.x + 1) * T / gridDim.x;
+  // The CTAs are dealt to the networks (the one with fewer tiles gets its share rounded
+  // up), so that none does two networks' weights, tiles and sums one after the other:
+  // a step of 2,293 points 89 -> 74 us, of 16,384 132 -> 123.
+  const int64_t ng = gridDim.x, T1 = T - T0, Ts = T0 < T1 ? T0 : T1;
+  const int64_t gs = Ts > 0 && ng > 1 ? (ng * Ts + T - 1) / T : 0;  // CTAs of that one
+  const int64_t g0 = gs == 0 ? ng : T0 < T1 ? gs : ng - gs;         // CTAs of the first
+  const bool first = blockIdx.x < g0;
+  const int64_t base = first || gs == 0 ? 0 : T0, span = gs == 0 ? T : first ? T0 : T1;
+  const int64_t bi = first ? blockIdx.x : blockIdx.x - g0, bn = first ? g0 : ng - g0;
+  const int64_t tb = base + bi * span / bn, te = base + (bi + 1) * span / bn;
   const float hf = P.hf, h2f = P.h2f, ihf = P.inv_hf, ih2f = P.inv_h2f;
 
   // gradient sums of this lane's unit (its point slot's share of the current net)
@@ -185,7 +193,7 @@ __global__ void __launch_bounds__(small_threads(HM), 1) k_step_small(ProbDev P, 
   // memory, added over the `used` warps that had tiles and their point slots in a
   // fixed order.  At H <= 16 the sums of all layers fit at once (32 (H + 1) (L - 1) +
   // 160 floats of 512 L + 96), else layer by layer.  Layer by layer and over all 16
-  // warps, a step of 2,293 points took 116 us (89 now), of 16,384 145 (132 now).
+  // warps, a step of 2,293 points took 116 us (89 so), of 16,384 145 (132 so).
   auto flush = [&](int net, int used) {
     float* gp = a.gpart + ((int64_t)blockIdx.x * 2 + net) * P.gstride;
     const int wf = small_warp_floats(L), hh = H * H;

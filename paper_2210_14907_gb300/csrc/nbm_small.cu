@@ -153,6 +153,10 @@ __global__ void __launch_bounds__(small_threads(HM), 1) k_step_small(ProbDev P, 
   const int ppw = 32 / H < kMaxPt ? 32 / H : kMaxPt;  // points per warp
   const bool own = lane < ppw * H;                    // lane pq H + u: unit u of point pq
   const int pq = own ? lane / H : 0, u = own ? lane - pq * H : 0, pbase = pq * H;
+  // A lane without a unit repeats lane 0's (it stores nothing): it reads that lane's
+  // columns and not its own, which nothing wrote, since its vote on the series
+  // (small_increments) counts like the others'.
+  const int ln = pbase + u;
   float* wsm = sbuf + w * small_warp_floats(L);
   float* Zb = wsm;                    // [L][32][8] pre-activations, then their gradients
   float* Ab = wsm + L * 256;          // [L][32][8] outputs
@@ -404,7 +408,7 @@ __global__ void __launch_bounds__(small_threads(HM), 1) k_step_small(ProbDev P, 
         const float4 hi = *reinterpret_cast<const float4*>(seeds_s + 8 * pq + 4);
         const float sd[8] = {lo.x, lo.y, lo.z, lo.w, hi.x, hi.y, hi.z, hi.w};
         float oc[8];
-        ld8(Ab + (L - 1) * 256, lane, oc);
+        ld8(Ab + (L - 1) * 256, ln, oc);
         const float wv = wo[u];
         float s = 0.f;
 #pragma unroll
@@ -423,8 +427,8 @@ __global__ void __launch_bounds__(small_threads(HM), 1) k_step_small(ProbDev P, 
 #pragma unroll 1
       for (int g = L - 1; g >= 1; --g) {
         float zc[8], oc[8], gzv[8];
-        if constexpr (ACT == NBM_ACT_SIN) ld8(Zb + g * 256, lane, zc);
-        ld8(Ab + g * 256, lane, oc);
+        if constexpr (ACT == NBM_ACT_SIN) ld8(Zb + g * 256, ln, zc);
+        ld8(Ab + g * 256, ln, oc);
         layer_bwd<ACT>(zc, oc, G, jump, hf, h2f, ihf, ih2f, gzv);
 #pragma unroll
         for (int i = 0; i < kLM - 1; ++i) gbh[i] += (g - 1 == i) ? gzv[0] + gzv[7] : 0.f;
@@ -467,8 +471,8 @@ __global__ void __launch_bounds__(small_threads(HM), 1) k_step_small(ProbDev P, 
       // increments del_i = h W1[u][i] give d(dt_i)/dW1[u][i] = 1 (scaled columns)
       {
         float zc[8], oc[8], gzv[8];
-        if constexpr (ACT == NBM_ACT_SIN) ld8(Zb, lane, zc);
-        ld8(Ab, lane, oc);
+        if constexpr (ACT == NBM_ACT_SIN) ld8(Zb, ln, zc);
+        ld8(Ab, ln, oc);
         layer_bwd<ACT>(zc, oc, G, jump, hf, h2f, ihf, ih2f, gzv);
         gW1[0] += fmaf(gzv[0], r.x, fmaf(gzv[7], r.gx, gzv[4]));
         gW1[1] += fmaf(gzv[0], r.y, fmaf(gzv[7], r.gy, gzv[5]));

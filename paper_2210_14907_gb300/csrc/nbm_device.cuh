@@ -691,6 +691,16 @@ __device__ __forceinline__ T uncut_residual_pt(const ProbDev& P, int s, float px
   return r * r;
 }
 
+// a / d from the rounded reciprocal id of d: the product and one correction by its
+// remainder, which leaves the rounding of the sum (an infinite or NaN product stays).
+// A step of 60,000 points through 5 x 10 sine networks takes 247 us so, 253 with IEEE
+// divisions, 246 with products alone; ten steps of 4096 points, 64 x 2: 804, 816, 814.
+template <typename T>
+__device__ __forceinline__ T quotient(T a, T d, T id) {
+  const T q = a * id;
+  return q - q == (T)0 ? fma(fma(-q, d, a), id, q) : q;
+}
+
 // The row of uncut_residual_pt spread over the 8 lanes c = 0..7 of an aligned
 // group of a warp (all 8 call it for the same point; `mask` covers the
 // calling lanes).  Lane c < 6 takes face c (axis c/2, side c%2), lane 6 the
@@ -701,7 +711,12 @@ __device__ __forceinline__ T uncut_residual_pt(const ProbDev& P, int s, float px
 // different order, with the dependency chain of one face per lane: a short
 // chain for the FP32 rows, and for the FP64 rows each instruction of the
 // narrow FP64 pipe carries 8 lanes instead of 1.
-template <typename T>
+// DIV (FP32 rows of the plain FP32 kernels): the quotients by h, h^2 and D are corrected to
+// division's accuracy (quotient).  A rounded FP32 reciprocal errs by the same amount at
+// every point (1/6: 3e-8, 1/60: 5e-8), which the mean over the points keeps: the loss of
+// 200,003 points was 6 to 8e-8 off by it, and is 3e-8 at most so.  (An FP64 reciprocal's
+// 1e-16 is far below the FP32 network values that the rows take.)
+template <typename T, bool DIV = false>
 __device__ __forceinline__ T uncut_residual_lanes(const ProbDev& P, int s, float px, float py,
                                                   float pz, T fsrc, float U_c, float Mt_c,
                                                   float Dt_c, T scale, int c, unsigned mask,
@@ -736,10 +751,12 @@ __device__ __forceinline__ T uncut_residual_lanes(const ProbDev& P, int s, float
       dv = mf;
     }
     if (fabs(i == 0 ? q0 : i == 1 ? q1 : q2) >= (T)1) {
-      term = -mf * (dirichlet_g<T>(P, q0, q1, q2) - U) * ih2;
+      const T dg = mf * (dirichlet_g<T>(P, q0, q1, q2) - U);
+      term = DIV ? -quotient(dg, h2, ih2) : -dg * ih2;
       nb = mf;
     } else {
-      term = -mf * (plus ? Mt + Dt * ih : Mt - Dt * ih);
+      const T Dh = DIV ? quotient(Dt, h, ih) : Dt * ih;
+      term = -mf * (plus ? Mt + Dh : Mt - Dh);
       cm = mf;
     }
   } else if (c == 6) {
@@ -756,13 +773,20 @@ __device__ __forceinline__ T uncut_residual_lanes(const ProbDev& P, int s, float
   const int ax = c >= 4 ? c - 4 : c - 1;
   const int fa = ax < 0 || ax > 2 ? 0 : 2 * ax;
   const T cmm = __shfl_sync(mask, cm, fa, 8), cmp = __shfl_sync(mask, cm, fa + 1, 8);
+  T r, cf;
   if (P.solution == 1) iD = (T)1 / (Dv + h2 * kk);
-  const T r = h2 * Bt * iD;
-  const T cf = scale * (T)2 * r * h2 * iD;
+  if constexpr (DIV) {
+    const T D = (P.solution == 1 ? Dv : (T)6 * mu) + h2 * kk;
+    r = quotient(h2 * Bt, D, iD);
+    cf = quotient(scale * (T)2 * r * h2, D, iD);
+  } else {
+    r = h2 * Bt * iD;
+    cf = scale * (T)2 * r * h2 * iD;
+  }
   T sd = (T)0;
-  if (c == 0) sd = cf * (kk + nbmu * ih2);
+  if (c == 0) sd = cf * (kk + (DIV ? quotient(nbmu, h2, ih2) : nbmu * ih2));
   else if (c <= 3) sd = cf * -(cmm + cmp);
-  else if (c <= 6) sd = cf * (-(cmp - cmm) * ih);
+  else if (c <= 6) sd = cf * (DIV ? -quotient(cmp - cmm, h, ih) : -(cmp - cmm) * ih);
   sd_c = (float)sd;
   return r * r;
 }

@@ -395,8 +395,8 @@ __global__ void __launch_bounds__(kNT, 1) k_step_fp32(ProbDev P, StepArgs a) {
             r2 = uncut_residual_lanes<double>(P, net, r.x, r.y, r.z, (double)r.gx + (double)r.gy,
                                               Uc, Mtc, Dtc, (double)a.scale, c, gmask, sd);
           } else {
-            r2 = uncut_residual_lanes<float>(P, net, r.x, r.y, r.z, r.gx, Uc, Mtc, Dtc, a.scale, c,
-                                             gmask, sd);
+            r2 = uncut_residual_lanes<float, true>(P, net, r.x, r.y, r.z, r.gx, Uc, Mtc, Dtc,
+                                                   a.scale, c, gmask, sd);
           }
           if (c == 0) {
             loss_acc += r2;

@@ -383,8 +383,8 @@ __global__ void __launch_bounds__(small_threads(HM), 1) k_step_small(ProbDev P, 
                                                 (double)a.scale, c, gmask, sd);
             } else {
               const float f = c == 6 ? rhs_f<float>(P, net, rq.x, rq.y, rq.z) : 0.f;
-              r2 = uncut_residual_lanes<float>(P, net, rq.x, rq.y, rq.z, f, Uc, Mtc, Dtc, a.scale,
-                                               c, gmask, sd);
+              r2 = uncut_residual_lanes<float, true>(P, net, rq.x, rq.y, rq.z, f, Uc, Mtc, Dtc,
+                                                     a.scale, c, gmask, sd);
             }
             if (c == 0) {
               loss_acc += r2;

@@ -204,6 +204,22 @@ __global__ void __launch_bounds__(small_threads(HM), 1) k_step_small(ProbDev P, 
     const int64_t oo = 4 * H + (int64_t)(L - 1) * (hh + H);
     constexpr bool kAll = HM <= 16;
     const int hid = kAll ? (L - 1) * (hh + H) : 0, per = hid + 5 * H;  // last staging, per point slot
+    // sum over the warps and their point slots (stride `st` floats) of staged element i:
+    // a warp's slots first, then the warps in four chains.  (One chain over all 48 at H = 10
+    // rounds more: the gradient of 16,384 points 7.3e-8 off against 5.3e-8, and 0.7 us longer.)
+    auto warps = [&](int i, int st) {
+      float t[4] = {0.f, 0.f, 0.f, 0.f};
+      for (int ww = 0; ww < used; ww += 4)
+#pragma unroll
+        for (int k = 0; k < 4; ++k)
+          if (ww + k < used) {
+            const float* e = sbuf + (ww + k) * wf + i;
+            float s = e[0];
+            for (int q = 1; q < ppw; ++q) s += e[q * st];
+            t[k] += s;
+          }
+      return (t[0] + t[1]) + (t[2] + t[3]);
+    };
     float go = gbo;
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) go += __shfl_xor_sync(0xffffffffu, go, o);
@@ -222,10 +238,7 @@ __global__ void __launch_bounds__(small_threads(HM), 1) k_step_small(ProbDev P, 
       if constexpr (!kAll) {
         __syncthreads();
         for (int i = tid; i < hh + H; i += NT) {
-          float s = 0.f;
-          for (int ww = 0; ww < used; ++ww)
-            for (int q = 0; q < ppw; ++q) s += sbuf[ww * wf + q * (hh + H) + i];
-          gp[4 * H + (int64_t)g * (hh + H) + i] = s;  // weights, then biases
+          gp[4 * H + (int64_t)g * (hh + H) + i] = warps(i, hh + H);  // weights, then biases
         }
       }
     }
@@ -240,9 +253,7 @@ __global__ void __launch_bounds__(small_threads(HM), 1) k_step_small(ProbDev P, 
     }
     __syncthreads();
     for (int i = tid; i < per; i += NT) {
-      float s = 0.f;
-      for (int ww = 0; ww < used; ++ww)
-        for (int q = 0; q < ppw; ++q) s += sbuf[ww * wf + q * per + i];
+      const float s = warps(i, per);
       const int r = i - hid;  // hidden layers' weights and biases, then layer 1 and the output
       gp[r < 0 ? 4 * H + i : r < 4 * H ? r : oo + r - 4 * H] = s;
     }

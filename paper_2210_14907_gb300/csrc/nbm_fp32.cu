@@ -22,7 +22,8 @@
 // tile, added to this CTA's slice of the partial-gradient buffer by
 // fire-and-forget reductions: each element belongs to one thread, so they
 // apply in tile order (no atomics across threads: the final reduction over
-// CTAs runs in a fixed order).
+// CTAs runs in a fixed order).  (A load, a sum and a store in their place read the slice
+// through L2: 200,003 points at 128 x 3 7.93 ms against 7.27.)
 //
 // Bound: the FFMA pipe (42 H^2 FMA per point and hidden layer).  200,003
 // points, 3 -> 128 x 3 -> 1: 17.4 -> 7.2 ms per launch (48 % of the 80.5 TFLOP/s
@@ -73,7 +74,10 @@ __device__ __forceinline__ void cp_async_wait() {
   asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory");
 }
 // reduction without a return value: the calling thread's additions to one
-// address apply in program order
+// address apply in program order.  It takes subnormal operands and results as 0, so
+// only values of at least kRedMin go through it: there a subnormal in memory is below
+// half a unit of the sum's last place, and a sum of opposite signs is 0 or normal.
+constexpr float kRedMin = 0x1p-101f;
 __device__ __forceinline__ void red_add(float* p, float v) {
   asm volatile("red.relaxed.gpu.global.add.f32 [%0], %1;" ::"l"(p), "f"(v) : "memory");
 }
@@ -505,16 +509,31 @@ __global__ void __launch_bounds__(kNT, 1) k_step_fp32(ProbDev P, StepArgs a) {
           gq += q & 1 ? PS - gx : gx;
           aq += q & 1 ? PS - ax : ax;
         }
+        bool tiny = false;
 #pragma unroll
         for (int i = 0; i < NU; ++i)
 #pragma unroll
           for (int j = 0; j < NK; ++j) {
             float ev, od;
             f2get(c[i][j], ev, od);
+            const float v = ev + od;
             float* dst = gp + 16 * i * H + 32 * j;
-            if (first_tile) *dst = ev + od;
-            else red_add(dst, ev + od);
+            if (first_tile) *dst = v;
+            else if (fabsf(v) >= kRedMin) red_add(dst, v);
+            else tiny |= v != 0.f;  // (NaN included)
           }
+        if (tiny) {
+#pragma unroll
+          for (int i = 0; i < NU; ++i)
+#pragma unroll
+            for (int j = 0; j < NK; ++j) {
+              float ev, od;
+              f2get(c[i][j], ev, od);
+              const float v = ev + od;
+              float* dst = gp + 16 * i * H + 32 * j;
+              if (!(fabsf(v) >= kRedMin) && v != 0.f) __stcg(dst, __ldcg(dst) + v);
+            }
+        }
       }
       // input gradient: G[k][c] = sum_u W_g[u][k] gz[u][c]
 #pragma unroll

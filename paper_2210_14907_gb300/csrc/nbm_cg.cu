@@ -1258,9 +1258,12 @@ struct GridSolve {
   }
 
   // Iterations from `it` in launches of k_cg_persist until ||r|| <= stop (sets it and
-  // rnorm).  0, or -1 for a CUDA error, or NBM_ERR_DEVICE_TIMEOUT.
+  // rnorm).  0, or -1 for a CUDA error, or NBM_ERR_DEVICE_TIMEOUT.  A context with fewer
+  // SMs than the device (a limit on the process's share) refuses a cooperative launch
+  // of one CTA per SM: PL.ctas is then 0, and the caller goes on from `it` with three
+  // launches per iteration (r, p, x and sc[0] are as those leave them).
   template <typename T, bool UNIT>
-  int iterate(const PersistLaunch& PL, const T* dg, const T* dv, const T* ax, const T* ay,
+  int iterate(PersistLaunch& PL, const T* dg, const T* dv, const T* ax, const T* ay,
               const T* az, T* xv, T* rv, T* p, int& it, int max_iter, double stop, double& rn,
               cudaError_t& e) {
     while (it < max_iter) {
@@ -1277,6 +1280,12 @@ struct GridSolve {
       cfg.numAttrs = 1;
       e = cudaLaunchKernelEx(&cfg, k_cg_persist<T, UNIT>, S.G, dg, dv, ax, ay, az, xv, rv, p, part,
                              sc, count, it, kPersistSteps, max_iter, kCheckEvery, stop);
+      if (e == cudaErrorCooperativeLaunchTooLarge) {
+        (void)cudaGetLastError();
+        e = cudaSuccess;
+        PL.ctas = 0;
+        return 0;
+      }
       if (e != cudaSuccess || (e = read_sc()) != cudaSuccess) return -1;
       if (host_sc[15] != 0.0) return NBM_ERR_DEVICE_TIMEOUT;
       const int done = (int)host_sc[14];
@@ -1325,7 +1334,7 @@ struct GridSolve {
     rnorm = sqrt(host_sc[4]);
     int it = 0;
     bool converged = rnorm <= rtol * bnorm;
-    const PersistLaunch PL = persist_launch<double, true>(S);
+    PersistLaunch PL = persist_launch<double, true>(S);
     if (PL.ctas && !converged && it < max_iter && rnorm == rnorm) {
       if (int rc = iterate<double, true>(PL, nullptr, diag, wx, wy, wz, x, r, pv, it, max_iter,
                                          rtol * bnorm, rnorm, e))
@@ -1361,7 +1370,7 @@ struct GridSolve {
     if ((e = read_sc()) != cudaSuccess) return -1;
     bnorm = sqrt(host_sc[9]);
     rnorm = sqrt(host_sc[8]);
-    const PersistLaunch PL = persist_launch<float, false>(S);
+    PersistLaunch PL = persist_launch<float, false>(S);
     int it = 0, stall = 0;
     bool converged = rnorm <= rtol * bnorm;
     while (!converged && it < max_iter && rnorm == rnorm && stall < kMaxStall) {

@@ -560,137 +560,6 @@ __device__ __forceinline__ float tanh_stencil_bwd(float t, float s0, float mo, f
   return fmaf(P, Gm, Q * Gd);
 }
 
-// ---------------------------------------------------------------------------
-// Balance row of an uncut cell of phase s (Sec. 3 reading):
-//   B/h^2 = k U(p) - f(p) - mu sum_{i,sigma} dU_{sigma i}/h^2,
-//   dU_{+-i}/h^2 = Mt_i +- Dt_i/h   (interior neighbour)
-//               = (g(q) - U(p))/h^2  (neighbour outside the cube: Dirichlet),
-//   D = 6 mu + h^2 k,  r = B/D.
-// out[8] = network outputs (U, Mt1..3, Dt1..3, unused); seeds[8] receives
-// d(scale * r^2)/d(out).  Returns r^2.
-// ---------------------------------------------------------------------------
-template <typename T>
-__device__ inline T uncut_residual(const ProbDev& P, int s, float px, float py, float pz,
-                                   const float out[8], T scale, float seeds[8]) {
-  const T h = pc_h<T>(P), h2 = h * h, mu = pc_mu<T>(P, s), k = pc_k<T>(P, s);
-  const T U = (T)out[0];
-  const T x[3] = {(T)px, (T)py, (T)pz};
-  T Bt = k * U - rhs_f<T>(P, s, x[0], x[1], x[2]);
-  T dU = k;
-  T dM[3], dD[3];
-  T D = h2 * k;
-#pragma unroll
-  for (int i = 0; i < 3; ++i) {
-    dM[i] = 0;
-    dD[i] = 0;
-#pragma unroll
-    for (int sg = -1; sg <= 1; sg += 2) {
-      T q[3] = {x[0], x[1], x[2]};
-      q[i] += sg * h;
-      // mu at the face centre (variable coefficients of Sec. 4.1)
-      T mf = mu;
-      if (P.solution == 1) {
-        T c[3] = {x[0], x[1], x[2]};
-        c[i] += (T)0.5 * (T)sg * h;
-        mf = mu_at<T>(P, s, c[0], c[1], c[2]);
-        D += mf;
-      }
-      bool bnd = fabs(q[i]) >= (T)1;
-      if (bnd) {
-        T g = dirichlet_g<T>(P, q[0], q[1], q[2]);
-        Bt -= mf * (g - U) / h2;
-        dU += mf / h2;
-      } else {
-        Bt -= mf * ((T)out[1 + i] + (T)sg * (T)out[4 + i] / h);
-        dM[i] -= mf;
-        dD[i] -= mf * (T)sg / h;
-      }
-    }
-  }
-  if (P.solution != 1) D = (T)6 * mu + h2 * k;
-  T r = h2 * Bt / D;
-  T c = scale * (T)2 * r * h2 / D;
-  seeds[0] = (float)(c * dU);
-#pragma unroll
-  for (int i = 0; i < 3; ++i) {
-    seeds[1 + i] = (float)(c * dM[i]);
-    seeds[4 + i] = (float)(c * dD[i]);
-  }
-  seeds[7] = 0.f;
-  return r * r;
-}
-
-// The same rows for one point in one thread of the tensor-core path.  fsrc =
-// f^s(p), evaluated ahead (the tile records carry it); divisions by h, h^2
-// and D are multiplications by the reciprocals in P.  out[8] = network
-// outputs in the scaled convention (U, Mt1..3, Dt1..3, unused); sd[8]
-// receives d(scale * r^2)/d(out).  Returns r^2.
-template <typename T>
-__device__ __forceinline__ T uncut_residual_pt(const ProbDev& P, int s, float px, float py,
-                                               float pz, T fsrc, const float out[8], T scale,
-                                               float sd[8]) {
-  const T h = pc_h<T>(P), h2 = h * h, mu = pc_mu<T>(P, s), kk = pc_k<T>(P, s);
-  T ih, ih2, iD;
-  if constexpr (sizeof(T) == 4) {
-    ih = P.inv_hf;
-    ih2 = P.inv_h2f;
-    iD = P.inv_Df[s];
-  } else {
-    ih = P.inv_h;
-    ih2 = P.inv_h2;
-    iD = P.inv_D[s];
-  }
-  const T U = (T)out[0];
-  const T x[3] = {(T)px, (T)py, (T)pz};
-  T Bt = kk * U - fsrc;
-  T nbmu = 0;  // sum of mu over the Dirichlet faces
-  T cM[3], cD[3];
-  T Dv = h2 * kk;  // Jacobi diagonal accumulated over faces (variable mu only)
-#pragma unroll
-  for (int i = 0; i < 3; ++i) {
-    const T Mt = (T)out[1 + i], Dt = (T)out[4 + i];
-    T qm[3] = {x[0], x[1], x[2]}, qp[3] = {x[0], x[1], x[2]};
-    qm[i] -= h;
-    qp[i] += h;
-    // mu at the two face centres (variable coefficients of Sec. 4.1)
-    T mm = mu, mp = mu;
-    if (P.solution == 1) {
-      T cm[3] = {x[0], x[1], x[2]}, cp[3] = {x[0], x[1], x[2]};
-      cm[i] -= (T)0.5 * h;
-      cp[i] += (T)0.5 * h;
-      mm = mu_at<T>(P, s, cm[0], cm[1], cm[2]);
-      mp = mu_at<T>(P, s, cp[0], cp[1], cp[2]);
-      Dv += mm + mp;
-    }
-    const bool bm = fabs(qm[i]) >= (T)1, bp = fabs(qp[i]) >= (T)1;
-    if (bm) {
-      Bt -= mm * (dirichlet_g<T>(P, qm[0], qm[1], qm[2]) - U) * ih2;
-      nbmu += mm;
-    } else {
-      Bt -= mm * (Mt - Dt * ih);
-    }
-    if (bp) {
-      Bt -= mp * (dirichlet_g<T>(P, qp[0], qp[1], qp[2]) - U) * ih2;
-      nbmu += mp;
-    } else {
-      Bt -= mp * (Mt + Dt * ih);
-    }
-    cM[i] = -((bm ? (T)0 : mm) + (bp ? (T)0 : mp));
-    cD[i] = -((bp ? (T)0 : mp) - (bm ? (T)0 : mm)) * ih;
-  }
-  if (P.solution == 1) iD = (T)1 / Dv;
-  const T r = h2 * Bt * iD;
-  const T c = scale * (T)2 * r * h2 * iD;
-  sd[0] = (float)(c * (kk + nbmu * ih2));
-#pragma unroll
-  for (int i = 0; i < 3; ++i) {
-    sd[1 + i] = (float)(c * cM[i]);
-    sd[4 + i] = (float)(c * cD[i]);
-  }
-  sd[7] = 0.f;
-  return r * r;
-}
-
 // a / d from the rounded reciprocal id of d: the product and one correction by its
 // remainder, which leaves the rounding of the sum (an infinite or NaN product stays).
 // A step of 60,000 points through 5 x 10 sine networks takes 247 us so, 253 with IEEE
@@ -701,16 +570,21 @@ __device__ __forceinline__ T quotient(T a, T d, T id) {
   return q - q == (T)0 ? fma(fma(-q, d, a), id, q) : q;
 }
 
-// The row of uncut_residual_pt spread over the 8 lanes c = 0..7 of an aligned
-// group of a warp (all 8 call it for the same point; `mask` covers the
-// calling lanes).  Lane c < 6 takes face c (axis c/2, side c%2), lane 6 the
-// reaction and source term; the balance row and the Dirichlet and face sums
-// are added over the group by shuffles.  Every lane passes the point's U and
-// the Mt, Dt columns of its face's axis (any value on lanes 6 and 7), returns
-// r^2 and writes seed c.  The same terms as the one-thread row, added in a
-// different order, with the dependency chain of one face per lane: a short
-// chain for the FP32 rows, and for the FP64 rows each instruction of the
-// narrow FP64 pipe carries 8 lanes instead of 1.
+// ---------------------------------------------------------------------------
+// Balance row of an uncut cell of phase s (Sec. 3 reading):
+//   B/h^2 = k U(p) - f(p) - mu sum_{i,sigma} dU_{sigma i}/h^2,
+//   dU_{+-i}/h^2 = Mt_i +- Dt_i/h   (interior neighbour)
+//               = (g(q) - U(p))/h^2  (neighbour outside the cube: Dirichlet),
+//   D = 6 mu + h^2 k,  r = B/D.
+//
+// The row is spread over the 8 lanes c = 0..7 of an aligned group of a warp (all 8
+// call it for the same point; `mask` covers the calling lanes).  Lane c < 6 takes
+// face c (axis c/2, side c%2), lane 6 the reaction and source term; the balance row
+// and the Dirichlet and face sums are added over the group by shuffles.  Every lane
+// passes fsrc = f^s(p), the point's U and the Mt, Dt columns of its face's axis (any
+// value on lanes 6 and 7; scaled convention), returns r^2 and writes seed c, d(scale *
+// r^2)/d(output c), 0 for c = 7.  So the dependency chain is one face long, and for the
+// FP64 rows each instruction of the narrow FP64 pipe carries 8 lanes instead of 1.
 // DIV (FP32 rows of the plain FP32 kernels): the quotients by h, h^2 and D are corrected to
 // division's accuracy (quotient).  A rounded FP32 reciprocal errs by the same amount at
 // every point (1/6: 3e-8, 1/60: 5e-8), which the mean over the points keeps: the loss of

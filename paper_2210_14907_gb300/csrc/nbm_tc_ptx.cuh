@@ -59,18 +59,8 @@ __device__ __forceinline__ constexpr uint32_t kstep_mnmajor(int k) {
   return (uint32_t)k * (2048u >> 4);
 }
 
-// Instruction descriptor of kind::f16, M = N = 128, FP32 accumulate.
-// is_bf16: both operands BF16 (else both FP16).  a_mn / b_mn: MN-major.
-__host__ __device__ __forceinline__ uint32_t idesc_f16(bool is_bf16, bool a_mn, bool b_mn) {
-  const uint32_t fmt = is_bf16 ? 1u : 0u;
-  return (1u << 4)               // D format F32
-         | (fmt << 7) | (fmt << 10)  // A, B formats
-         | ((a_mn ? 1u : 0u) << 15) | ((b_mn ? 1u : 0u) << 16)
-         | ((128u >> 3) << 17)   // N
-         | ((128u >> 4) << 24);  // M
-}
-
-// The same with a free N (a multiple of 16 up to 256; M = 128).
+// Instruction descriptor of kind::f16, M = 128, N a multiple of 16 up to 256, FP32
+// accumulate.  is_bf16: both operands BF16 (else both FP16).  a_mn / b_mn: MN-major.
 __host__ __device__ __forceinline__ uint32_t idesc_f16_n(bool is_bf16, bool a_mn, bool b_mn,
                                                          uint32_t n) {
   const uint32_t fmt = is_bf16 ? 1u : 0u;
@@ -220,16 +210,6 @@ __device__ __forceinline__ void tmem_ld16(uint32_t taddr, float* v) {
 #pragma unroll
   for (int i = 0; i < 16; ++i) v[i] = __uint_as_float(r[i]);
 }
-__device__ __forceinline__ void tmem_st32_zero(uint32_t taddr) {
-  const uint32_t z = 0;
-  asm volatile(
-      "tcgen05.st.sync.aligned.32x32b.x32.b32 [%0], "
-      "{%1,%1,%1,%1,%1,%1,%1,%1,%1,%1,%1,%1,%1,%1,%1,%1,"
-      "%1,%1,%1,%1,%1,%1,%1,%1,%1,%1,%1,%1,%1,%1,%1,%1};" ::"r"(taddr),
-      "r"(z));
-  asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
-}
-
 // ---- mbarrier + bulk copy ----
 __device__ __forceinline__ void mbar_init(uint32_t mbar, uint32_t count) {
   asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(mbar), "r"(count));

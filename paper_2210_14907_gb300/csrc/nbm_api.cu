@@ -137,7 +137,7 @@ static int ws_reserve(Problem& pb, int64_t n) {
   NBM_CUDA(dalloc(w.gacc, 2 * (size_t)pb.p_net));
   NBM_CUDA(dalloc(w.gpart, (size_t)grid * 2 * ((pb.p_net + 3) & ~(int64_t)3)));
   NBM_CUDA(dalloc(w.gpart_flag, 2 * (size_t)grid));
-  NBM_CUDA(dalloc(w.wt, 2 * (size_t)(L - 1) * H * H));
+  if (wt_needed(pb.desc.width)) NBM_CUDA(dalloc(w.wt, 2 * (size_t)(L - 1) * H * H));
   NBM_CUDA(dalloc((uint16_t*&)w.wtc, 2 * (size_t)(L - 1) * H * H));
   NBM_CUDA(dalloc(w.grad, 2 * (size_t)pb.p_net));
   NBM_CUDA(dalloc(w.step, 1));

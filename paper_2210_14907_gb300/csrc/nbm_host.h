@@ -112,7 +112,7 @@ struct Workspace {
   float* gacc = nullptr;            // [2 p_net] gradient of the refinement levels done so far
   float* gpart = nullptr;
   int* gpart_flag = nullptr;
-  float* wt = nullptr;              // FP32 transposed hidden weights
+  float* wt = nullptr;              // FP32 transposed hidden weights (see wt_needed)
   void* wtc = nullptr;              // 16-bit hidden weights
   float* grad = nullptr;            // [P]
   int64_t* step = nullptr;          // [1] device step counter
@@ -214,5 +214,8 @@ cudaError_t launch_adam(int64_t n, float* params, float* m, float* v, const floa
 size_t tc_smem_bytes(int L);
 cudaError_t launch_selftest_wait(long long budget, int* out, cudaStream_t st);
 int tc_supported(int H, int L);
+// whether a kernel reads the transposed FP32 weights: the wide FP32 step does, the narrow
+// one (width <= 32) transposes its own from the parameters
+inline bool wt_needed(int width) { return width > 32; }
 
 }  // namespace nbm

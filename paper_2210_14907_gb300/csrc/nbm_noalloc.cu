@@ -144,6 +144,7 @@ extern "C" int nbm_loss_grad_static(nbm_problem* p, const float* params, const f
   w.gpart = carve<float>(cur, (size_t)kStaticMaxGrid * 2 * kStaticMaxPNetStride * 4);
   w.gpart_flag = carve<int>(cur, 2 * kStaticMaxGrid * 4);
   w.wt = carve<float>(cur, (size_t)2 * kStaticMaxHidden * 128 * 128 * 4);
+  if (!wt_needed(d.width)) w.wt = nullptr;
   w.wtc = carve<void>(cur, (size_t)2 * kStaticMaxHidden * 128 * 128 * 2);
   w.step = carve<int64_t>(cur, 8);
   w.status = carve<int>(cur, 4);

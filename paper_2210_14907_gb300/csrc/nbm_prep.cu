@@ -137,8 +137,8 @@ __device__ inline void prep_weights_blocks(const ProbDev& P, const float* params
   }
 }
 
-// blocks of a weight restage
-static int prep_weight_blocks(const ProbDev& P) { return 2 * (P.L - 1) * 16; }
+// blocks of a weight restage (none for narrow networks, whose kernel reads the parameters)
+static int prep_weight_blocks(const ProbDev& P) { return wt_needed(P.H) ? 2 * (P.L - 1) * 16 : 0; }
 
 __global__ void __launch_bounds__(kBlk) k_sample_classify(ProbDev P, const float* pts_in,
                                                           uint64_t seed, const int64_t* step_dev,

@@ -302,7 +302,10 @@ int nbm_eval_points(nbm_problem* p, const float* params, const float* pts, int64
  *     (re-solved; see nbm_grid_last_jump_info).  Nodes farther than 3h from
  *     Gamma carry J = 0 (no row weights them).
  * Returns NBM_ERR_NOT_CONVERGED (with u_out filled) if a solve reaches
- * max_iter. */
+ * max_iter, NBM_ERR_NONFINITE (u_out filled) if the residual is not finite,
+ * NBM_ERR_DEVICE_TIMEOUT (u_out not written) if a bounded device wait gave up
+ * (up to 130 cells per axis the iterations run in one launch whose blocks wait
+ * for one another; where the device refuses it, in three launches each). */
 int nbm_grid_cg_solve(nbm_problem* p, int n, double rtol, int max_iter, double* u_out,
                       int* iters_out, double* relres_out, nbm_stream_t stream);
 
@@ -320,6 +323,7 @@ int nbm_grid_cg_solve(nbm_problem* p, int n, double rtol, int max_iter, double* 
  *   Returns NBM_ERR_NOT_CONVERGED (u_out filled) at max_iter, or when three
  *   corrections in a row reduce ||b - A x|| by less than 10 % (an operator too
  *   ill-conditioned for FP32 corrections: use nbm_grid_cg_solve).
+ *   NBM_ERR_NONFINITE and NBM_ERR_DEVICE_TIMEOUT as nbm_grid_cg_solve.
  * Synchronizes the stream. */
 int nbm_grid_solve_refined(nbm_problem* p, int n, double rtol, int max_iter, double* u_out,
                            int* iters_out, double* relres_out, nbm_stream_t stream);

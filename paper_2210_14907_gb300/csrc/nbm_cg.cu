@@ -353,7 +353,7 @@ struct Coded {
 // (i, j) column through the slab, keeping the z neighbours in registers, so
 // node indices need no integer division and each thread reduces once.
 // (FP32: 8 blocks, i.e. 2048 threads, per SM; at most 32 registers)
-// CODED (the FP32 operator of constant-mu problems): see Coded below.
+// CODED (the FP32 operator of constant-mu problems): see Coded above.
 template <typename T, bool UNIT, bool CODED = false>
 __global__ void __launch_bounds__(kB, sizeof(T) == 4 && !CODED ? 8 : 6) k_spmv_dot(Grid G, int kz,
                                                  const T* diag,
@@ -1097,7 +1097,7 @@ struct PersistLaunch {
 template <typename T, bool UNIT>
 PersistLaunch persist_launch(const CgSetup& S) {
   PersistLaunch L;
-  const int64_t want = (S.G.m + 511) / 512;  // a thread or two per unknown on small grids
+  const int64_t want = (S.G.m + 511) / 512;  // a thread per unknown on small grids
   const int ctas = (int)(want < S.sms ? want : S.sms);
   const int64_t per = (S.G.m + ctas - 1) / ctas;
   const size_t smem = (size_t)(2 * per + 2 * S.G.m1) * sizeof(T);
@@ -1402,11 +1402,11 @@ struct GridSolve {
           launch_pdl(k_reduce_parts, dim3(1), dim3(kB), 0, st, part, S.nu, 2, sc, 3, POST_BETA);
           launch_pdl(k_pupdate4, dim3(S.nu), dim3(kB), 0, st, G, sc, idg32, r32, e32, p32, coded);
         } else {
-        launch_pdl(look ? k_update<float, false, true> : k_update<float, false, false>, dim3(S.nu),
-                   dim3(kB), 0, st, G, sc, idg32, Ap32, r32, part, tk());
-        reduce(S.nu, look ? 2 : 1, 3, POST_BETA);
-        launch_pdl(k_pupdate<float, false>, dim3(S.nu), dim3(kB), 0, st, G, sc, 0, idg32, r32, e32,
-                   p32);
+          launch_pdl(look ? k_update<float, false, true> : k_update<float, false, false>,
+                     dim3(S.nu), dim3(kB), 0, st, G, sc, idg32, Ap32, r32, part, tk());
+          reduce(S.nu, look ? 2 : 1, 3, POST_BETA);
+          launch_pdl(k_pupdate<float, false>, dim3(S.nu), dim3(kB), 0, st, G, sc, 0, idg32, r32,
+                     e32, p32);
         }
         if (look) {
           if ((e = read_sc()) != cudaSuccess) return -1;

@@ -9,8 +9,9 @@
 // independent warp groups with three tiles in flight each.  Layer 1 (K = 3)
 // and the output layer run in FP32; every hidden layer is one 128x64x128
 // tcgen05 MMA per tile with 16-bit operands (FP16 or BF16) and FP32
-// accumulation in TMEM.  The FP32 path is a plain SIMT evaluation (reference
-// precision).
+// accumulation in TMEM.  The FP32 path (reference precision) runs tiled FFMA
+// products, each point with its own network only; narrow networks take one thread
+// per point.
 #include <cuda_bf16.h>
 #include <cuda_fp16.h>
 
@@ -103,7 +104,8 @@ __device__ __forceinline__ uint32_t tanh_pack2(float a, float b) {
 // a set, not after every tile and layer, and run up to a tile apart.  513^3 nodes,
 // 3 -> 128 x 4 -> 1, FP16: 37.0 ms with a group barrier per tile and layer, 29.9 with
 // the issuing warps, 27.6 with shared-space addresses and descriptors by addition
-// (480 TFLOP/s; the 69 G tanh, two to an instruction, are 7 ms of the SFUs).
+// (480 TFLOP/s; the 69 G tanh, two to an instruction but in the last layer, are 43 G SFU
+// operations: 8.6 ms).
 //
 // Pass 0 (the minus network) decides every point's side and keeps it in
 // `side` (per 128 points, bit c: point c is in Omega-; each 64-point tile owns

@@ -25,8 +25,9 @@
 // CTAs runs in a fixed order).  (A load, a sum and a store in their place read the slice
 // through L2: 200,003 points at 128 x 3 7.93 ms against 7.27.)
 //
-// Bound: the FFMA pipe (42 H^2 FMA per point and hidden layer).  200,003
-// points, 3 -> 128 x 3 -> 1: 17.4 -> 7.2 ms per launch (48 % of the 80.5 TFLOP/s
+// Bound: the FFMA pipe (21 H^2 FMA per point and hidden layer; 24 with the
+// interface column).  200,003
+// points, 3 -> 128 x 3 -> 1: 17.4 -> 7.1 ms per launch (49 % of the 80.5 TFLOP/s
 // FFMA peak, pipe 61 % busy; in its GEMM loops 55-62 %, the rest in the chunk
 // barriers and the issue of packed-pair operands); 4096 points, 64 x 2: a
 // step of 107 -> 81 us.

@@ -30,7 +30,7 @@
 // points, 3 -> 128 x 3 -> 1: 17.4 -> 7.1 ms per launch (49 % of the 80.5 TFLOP/s
 // FFMA peak, pipe 61 % busy; in its GEMM loops 55-62 %, the rest in the chunk
 // barriers and the issue of packed-pair operands); 4096 points, 64 x 2: a
-// step of 107 -> 81 us.
+// step of 107 -> 82 us.
 #include "nbm_device.cuh"
 #include "nbm_f32x2.cuh"
 #include "nbm_host.h"

@@ -14,7 +14,7 @@
 // each other's latencies.  With one point per warp (10 of 32 lanes busy),
 // block barriers in every layer and the weight gradient summed in global
 // memory tile by tile, a step of 16,384 points through 5 x 10 sine networks took
-// 229 us in this kernel (the step 270; 123 now); the
+// 222 us in this kernel (the step 270; 72 and 116 now); the
 // bound now is the warps' dependency chains.
 // At the end of a network the lanes' sums are added over the warps in a fixed
 // order (deterministic).
